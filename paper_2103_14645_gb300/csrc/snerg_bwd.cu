@@ -77,9 +77,9 @@ __device__ __forceinline__ void scatter_recorded(const DevScene& s, const Ray& r
             }
             // a block without samples is never recorded by a march
             if (cur.slot >= 0) {
-                float f[3], g[3], fl[3];
+                float f[3], g[3];
                 int fi[3];
-                stencil_weights(cur.u, f, g, fl, fi);
+                stencil_weights(cur.u, f, g, fi);
                 scatter_sample(s, cur.slot, fi, cur.o3, f, g, cur.w, gfeat, grad_atlas);
             }
             cur = nxt;

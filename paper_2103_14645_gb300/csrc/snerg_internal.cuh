@@ -180,7 +180,8 @@ __device__ __forceinline__ float float_small(int v) { return __fsub_rn(__int_as_
 
 // a lattice coordinate lies within the grid up to rounding (|u| <= N + 1 <= 16385)
 __device__ __forceinline__ int nearest_voxel(float u, int N) {
-    return min(max(floor_int_small(u), 0), N - 1);
+    // max(min(floor(u), N - 1), 0) with the offset of the exact add, one instruction
+    return __viaddmin_s32_relu(__float_as_int(__fadd_rd(u, kMagic)), -kMagicBits, N - 1);
 }
 
 // A box of blocks lo..hi (inclusive, per axis) as bounds on the sample position: the
@@ -248,22 +249,9 @@ __device__ __forceinline__ float exit_margin(const Ray& r, float fN) {
 // arithmetic would (see exit_margin). Then every sample before ceil(K) is inside on every
 // face still ahead (their crossings are no earlier than K's) and the sample at ceil(K)
 // is outside. A margin of 1 or more disables this.
-__device__ __forceinline__ float box_exit(const Ray& r, const float inv_d[3], float kmax, float k, const Box& bx,
-                                          float margin) {
-    float te = r.t1;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        if (r.d[i] > 0.0f) te = fminf(te, (bx.hi[i] - r.o[i]) * inv_d[i]);
-        else if (r.d[i] < 0.0f) te = fminf(te, (bx.lo[i] - r.o[i]) * inv_d[i]);
-    }
-    const float K = te - r.t0 - 0.5f;
-    const float n = ceil_small(K);        // |K| <= t1 - t0 + 1 (or NaN, kept)
-    // fr in [0, 1). n - K is exact for K >= 1/2 (Sterbenz) and for K <= 0; for K in
-    // (0, 1/2), n = 1 and 1 - K rounds by at most 2^-25, far inside the margin (at least
-    // 4 * 2^-20, four times the bound on the estimate's own error), so the test below
-    // decides the same way.
-    const float fr = n - K;
-    if (n >= k + 1.0f && n < kmax && fr >= margin && fr < 1.0f - margin) return n;
+//
+// box_search: the exact search from an estimate n.
+__device__ __forceinline__ float box_search(const Ray& r, float kmax, float k, float n, const Box& bx) {
     // estimate clamped to [k + 1, kmax] (fminf/fmaxf also map a NaN estimate into range)
     const float ke = fmaxf(fminf(n, kmax), k + 1.0f);
     float lo_k = k, hi_k;
@@ -287,6 +275,60 @@ __device__ __forceinline__ float box_exit(const Ray& r, const float inv_d[3], fl
         if (in_box(r, mid, bx)) lo_k = mid; else hi_k = mid;
     }
     return hi_k;
+}
+
+__device__ __forceinline__ float box_exit(const Ray& r, const float inv_d[3], float kmax, float k, const Box& bx,
+                                          float margin) {
+    float te = r.t1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        if (r.d[i] > 0.0f) te = fminf(te, (bx.hi[i] - r.o[i]) * inv_d[i]);
+        else if (r.d[i] < 0.0f) te = fminf(te, (bx.lo[i] - r.o[i]) * inv_d[i]);
+    }
+    const float K = te - r.t0 - 0.5f;
+    const float n = ceil_small(K);        // |K| <= t1 - t0 + 1 (or NaN, kept)
+    // fr in [0, 1). n - K is exact for K >= 1/2 (Sterbenz) and for K <= 0; for K in
+    // (0, 1/2), n = 1 and 1 - K rounds by at most 2^-25, far inside the margin (at least
+    // 4 * 2^-20, four times the bound on the estimate's own error), so the test below
+    // decides the same way.
+    const float fr = n - K;
+    if (n >= k + 1.0f && n < kmax && fr >= margin && fr < 1.0f - margin) return n;
+    return box_search(r, kmax, k, n, bx);
+}
+
+// box_exit for the march's own boxes, from sample kh (= k + 1/2) of the voxel j: the blocks
+// within D - 1 (D >= 1) of j's block towards the ray's octant, so that on every axis only
+// the face ahead can be crossed. The estimate is box_exit's with two differences. A face on
+// or beyond the grid's border is not clipped to infinity: its crossing is at or behind t1 up
+// to the rounding that the margin covers, and t1 is in the minimum. And the margin test is
+// taken as |fr - 1/2| < half = 1/2 - margin. Lanes that stand in an empty box and in an
+// occupied block (D = 1) share this code. Returns k' + 1/2.
+//
+// A block entry was about 100 instructions, issued once for a warp's empty lanes and again
+// for its occupied ones (the march is bound by issue in full launches, by the chain of
+// dependent steps in small ones); one shared copy with a face instead of a box per axis:
+// 64 mixed views of a 1024^3 grid 6.01 -> 5.64 ms, one 800^2 view 190 -> 183 us, 262,147
+// scattered rays 283 -> 255 us.
+__device__ __forceinline__ float march_exit(const DevScene& s, const Ray& r, const float inv_d[3], float kh,
+                                            const int j[3], int D, float half) {
+    const int DB = D << s.lgB, BD = s.B - DB;
+    float te = r.t1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float face = float_small((j[i] & -s.B) + (r.d[i] < 0.0f ? BD : DB));
+        te = fminf(te, (face - r.o[i]) * inv_d[i]);          // d_i = 0: +inf or NaN, no bound
+    }
+    const float K = te - r.t0 - 0.5f;
+    const float n = ceil_small(K);
+    if (n > kh && n < (float)s.kmax && fabsf((n - K) - 0.5f) < half) return n + 0.5f;
+    int lo[3], hi[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int b = j[i] >> s.lgB;
+        lo[i] = r.d[i] < 0.0f ? b - D + 1 : b;
+        hi[i] = r.d[i] < 0.0f ? b : b + D - 1;
+    }
+    return box_search(r, (float)s.kmax, kh - 0.5f, n, make_box(s, lo, hi)) + 0.5f;
 }
 
 // Byte `byte` of w as a float, exactly: the byte is placed in the low mantissa bits of
@@ -332,29 +374,46 @@ __device__ __forceinline__ void accumulate_colour(MarchState& st, const uint2 cv
     st.acc[6] = a6;
 }
 
-// The trilinear stencil of a sample at u in block-padded coordinates (block origin minus
-// one at o, integer voxel coordinates): the fractional weights f, g = 1 - f, the lower
-// corner (as the float fl and the integer fi, both from one add), and the 8 corners'
-// codes (index z*4 + y*2 + x). The lower corner is in [0, B] for a sample of this block
-// (the apron holds the neighbours and the clamped border); the index clamp only guards
-// the address.
-__device__ __forceinline__ void stencil_weights(const float u[3], float f[3], float g[3], float fl[3], int fi[3]) {
+// floor(x) with the exact add's offset still in it: floor(x) + kMagicBits. Voxel
+// coordinates go into the padded index in this form; its base takes the offsets out
+// (integer arithmetic modulo 2^32).
+__device__ __forceinline__ uint32_t floor_raw(float x) { return (uint32_t)__float_as_int(__fadd_rd(x, kMagic)); }
+
+// For the block of voxel j: padded index = (v2 P + v1) P + v0 - base, v raw coordinates
+// (floor_raw) and (j & -B) - 1 the origin of the block's padded copy.
+__device__ __forceinline__ uint32_t padded_base(const DevScene& s, const int j[3]) {
+    const uint32_t P = (uint32_t)s.P, B = (uint32_t)-s.B, c = (uint32_t)kMagicBits - 1u;
+    return (((uint32_t)j[2] & B) * P + ((uint32_t)j[1] & B)) * P + ((uint32_t)j[0] & B) + c * (P * P + P + 1u);
+}
+
+// clamped to [0, top]
+__device__ __forceinline__ int padded_index(uint32_t v0, uint32_t v1, uint32_t v2, int P, uint32_t base, int top) {
+    return __viaddmin_s32_relu((int)((v2 * (uint32_t)P + v1) * (uint32_t)P + v0), (int)(0u - base), top);
+}
+
+// The trilinear stencil of a sample at u in its block's padded copy (base: padded_base):
+// the fractional weights f, g = 1 - f, the lower corner's voxel coordinates fi, and the 8
+// corners' codes (index z*4 + y*2 + x). The lower corner is in [0, B] for a sample of this
+// block (the apron holds the neighbours and the clamped border); the index clamp only
+// guards the address.
+__device__ __forceinline__ void stencil_weights(const float u[3], float f[3], float g[3], int fi[3]) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const float x = __fsub_rn(u[i], 0.5f);
         const float m = __fadd_rd(x, kMagic);            // floor_small / floor_int_small of x
-        fl[i] = __fsub_rn(m, kMagic);
         fi[i] = __float_as_int(m) - kMagicBits;
-        f[i] = __fsub_rn(x, fl[i]);
+        f[i] = __fsub_rn(x, __fsub_rn(m, kMagic));
         g[i] = __fsub_rn(1.0f, f[i]);
     }
 }
 
-__device__ __forceinline__ void load_stencil(const float u[3], const int o[3], int P, int P3, const uint2* pa,
-                                             float f[3], float g[3], float fl[3], int fi[3], uint2 cv[8]) {
-    stencil_weights(u, f, g, fl, fi);
+__device__ __forceinline__ void load_stencil(const float u[3], uint32_t base, int P, int P3, const uint2* pa,
+                                             float f[3], float g[3], int fi[3], uint2 cv[8]) {
+    stencil_weights(u, f, g, fi);
     const int PP = P * P;
-    const int i0 = min(max(((fi[2] - o[2]) * P + (fi[1] - o[1])) * P + (fi[0] - o[0]), 0), P3 - 1 - (PP + P + 1));
+    const uint32_t c = (uint32_t)kMagicBits;
+    const int i0 = padded_index((uint32_t)fi[0] + c, (uint32_t)fi[1] + c, (uint32_t)fi[2] + c, P, base,
+                                P3 - 1 - (PP + P + 1));
     const uint2* p0 = pa + i0;
     cv[0] = __ldg(p0);
     cv[1] = __ldg(p0 + 1);
@@ -480,10 +539,10 @@ __device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchStat
     st.blocks = 0;
     st.limit = false;
     if (!r.hit) return;
-    const int N = s.N, B = s.B, P = s.P;
+    const int N = s.N, P = s.P;
     float inv_d[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) inv_d[i] = __fdividef(1.0f, r.d[i]);
+    for (int i = 0; i < 3; ++i) inv_d[i] = __fdividef(1.0f, r.d[i] == 0.0f ? 0.0f : r.d[i]);   // +inf for -0 too
     // Voxel-skip rate: between samples k and k+s every coordinate moves by at most
     // s*m + eps voxels, m = max_i |d_i| and eps bounding the rounding of the binary32
     // lattice arithmetic (a few ulps of the largest t or u the ray meets; max(t1, N) *
@@ -493,67 +552,58 @@ __device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchStat
     const float m_max = fmaxf(fmaxf(fabsf(r.d[0]), fabsf(r.d[1])), fabsf(r.d[2]));
     const float skip_inv_m = (1.0f - 1.0f / 1048576.0f) / m_max;   // biased down: never overshoots
     const float skip_eps = fmaxf(r.t1, s.fN) * (1.0f / 524288.0f);
-    const float exit_m = exit_margin(r, s.fN);
+    const float exit_half = 0.5f - exit_margin(r, s.fN);
     const int oct = (r.d[0] < 0.0f ? 1 : 0) | (r.d[1] < 0.0f ? 2 : 0) | (r.d[2] < 0.0f ? 4 : 0);
     const int32_t* ind = s.ind + oct * s.ind_oct;
     const uint8_t* vskip = s.vskip + oct * s.vskip_oct;
-    const float kmax = (float)s.kmax;
-    float k = (float)k_begin;
+    // the loop's lattice positions are k + 1/2, exact, so that t takes one addition
+    float kh = (float)k_begin + 0.5f;
     float k_spec = -1.0f;   // the sample after the last composited one
     float steps = 0.0f;
     bool done = false;
     if (k_first) *k_first = s.kmax;
     for (;;) {
-        if (k >= kmax) { st.limit = true; break; }
-        const float t = lattice_t(r, k);
+        if (kh >= (float)s.kmax) { st.limit = true; break; }
+        const float t = __fadd_rn(r.t0, kh);
         if (!(t < r.t1)) break;
         int b[3];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) b[i] = nearest_voxel(lattice_u(r, t, i), N) >> s.lgB;
-        const int bi = (b[2] * s.G + b[1]) * s.G + b[0];
-        const int slot = __ldg(ind + bi);
+        for (int i = 0; i < 3; ++i) b[i] = nearest_voxel(lattice_u(r, t, i), N);
+        const int slot = __ldg(ind + ((b[2] >> s.lgB) * s.G + (b[1] >> s.lgB)) * s.G + (b[0] >> s.lgB));
         st.blocks++;
+        // an empty block (slot = -D): every block of the ray's cone within Chebyshev distance
+        // D - 1 is empty, leave that one-sided box; a stored one: its samples up to kx
+        const float kx = march_exit(s, r, inv_d, kh, b, max(-slot, 1), exit_half);
         if (slot < 0) {
-            // every block of the ray's cone within Chebyshev distance D-1 of b is empty:
-            // leave that one-sided box
-            const int D1 = -slot - 1;
-            int lo[3], hi[3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                lo[i] = ((oct >> i) & 1) ? b[i] - D1 : b[i];
-                hi[i] = ((oct >> i) & 1) ? b[i] : b[i] + D1;
-            }
-            k = box_exit(r, inv_d, kmax, k, make_box(s, lo, hi), exit_m);
+            kh = kx;
             continue;
         }
-        const float kx = box_exit(r, inv_d, kmax, k, make_box(s, b, b), exit_m);
         const uint8_t* vs = vskip + (size_t)slot * s.P3;
         const uint2* pa = s.patlas + (size_t)slot * s.P3;
-        // block origin minus one, so that the padded local coordinate is floor(u) - o
-        const int o3[3] = {(b[0] << s.lgB) - 1, (b[1] << s.lgB) - 1, (b[2] << s.lgB) - 1};
-        float kk = k;
+        // the padded index of the block's voxel with local coordinates l (1 .. B inside) is
+        // (l2 P + l1) P + l0 = (v2 P + v1) P + v0 - base for the grid's voxel v
+        const uint32_t base = padded_base(s, b);
+        float kk = kh;
         while (kk < kx) {
-            const float tk = lattice_t(r, kk);
+            const float tk = __fadd_rn(r.t0, kk);
             float u[3];
 #pragma unroll
             for (int i = 0; i < 3; ++i) u[i] = lattice_u(r, tk, i);
-            // nearest voxel in padded block coordinates, floor(u) - origin + 1: in [1, B] for
-            // a sample of this block, or 0 / B+1 where rounding puts u a hair outside the
-            // grid -- apron cells that hold the clamped edge voxel's value (the grid clamp
-            // is built into the plane). The index clamp only guards the address.
-            const int lx = floor_int_small(u[0]) - o3[0], ly = floor_int_small(u[1]) - o3[1],
-                      lz = floor_int_small(u[2]) - o3[2];
-            const int pidx = min(max((lz * P + ly) * P + lx, 0), s.P3 - 1);
+            // nearest voxel in padded block coordinates: in [1, B] for a sample of this
+            // block, or 0 / B+1 where rounding puts u a hair outside the grid -- apron cells
+            // that hold the clamped edge voxel's value (the grid clamp is built into the
+            // plane). The index clamp only guards the address.
+            const int pidx = padded_index(floor_raw(u[0]), floor_raw(u[1]), floor_raw(u[2]), P, base, s.P3 - 1);
             // SPEC: the sample's stencil is loaded before the probe's answer when the
             // previous sample was composited (inside a surface the next one usually is
             // too, and one memory latency then serves both), after it otherwise. It pays
             // in latency-bound launches (ray lists, the adjoint); where the launch is
             // issue-bound, lanes that disagree on the guess run the stencil code twice.
-            float f[3], g[3], fl[3];
+            float f[3], g[3];
             int fi[3];
             uint2 cv[8];
             const bool spec = SPEC && (kk == k_spec);
-            if (spec) load_stencil(u, o3, P, s.P3, pa, f, g, fl, fi, cv);
+            if (spec) load_stencil(u, base, P, s.P3, pa, f, g, fi, cv);
             const int vd = __ldg(vs + pidx);
             if (vd != 0) {
                 // no voxel of this block in the ray's cone within Chebyshev distance vd-1
@@ -566,14 +616,14 @@ __device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchStat
             if (TRACE && st.active < trace_cap)
                 trace[st.active] = ((uint64_t)nearest_voxel(u[2], N) * N + (uint64_t)nearest_voxel(u[1], N)) * N +
                                    (uint64_t)nearest_voxel(u[0], N);
-            if (k_first && st.active == 0) *k_first = (int)kk;
+            if (k_first && st.active == 0) *k_first = (int)kk;      // kk = k + 1/2
             st.active++;
             // trilinear stencil on the virtual grid, cell-centred
-            if (!spec) load_stencil(u, o3, P, s.P3, pa, f, g, fl, fi, cv);
+            if (!spec) load_stencil(u, base, P, s.P3, pa, f, g, fi, cv);
             bool saturated;
             const float wk = composite(s, cv, f, g, st.T, st.tau, saturated);
             if (REC && st.active <= kRecCap) {
-                rec[st.active - 1] = make_float2(kk, wk);
+                rec[st.active - 1] = make_float2(kk - 0.5f, wk);
                 if (st.active == kRecCap) rec[kRecCap] = make_float2(st.T, st.tau);
             }
             accumulate_colour(st, cv, wk, f, g);
@@ -599,9 +649,12 @@ __device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchStat
 #pragma unroll
                 for (int c = 0; c < 3; ++c) st.rgb_ps[c] = fmaf(wk, cdk[c] + res[c], st.rgb_ps[c]);
             }
-            if (GRAD) scatter_sample(s, slot, fi, o3, f, g, wk, gfeat, grad_atlas);
+            if (GRAD) {
+                const int o3[3] = {(b[0] & -s.B) - 1, (b[1] & -s.B) - 1, (b[2] & -s.B) - 1};
+                scatter_sample(s, slot, fi, o3, f, g, wk, gfeat, grad_atlas);
+            }
             if (saturated) {
-                steps += kk - k + 1.0f;
+                steps += kk - kh + 1.0f;
                 done = true;
                 break;
             }
@@ -609,8 +662,8 @@ __device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchStat
             if (SPEC) k_spec = kk;
         }
         if (done) break;
-        steps += kx - k;
-        k = kx;
+        steps += kx - kh;
+        kh = kx;
     }
     st.steps = (int)steps;
 }
