@@ -168,28 +168,24 @@ extern "C" snerg_status snerg_create(const snerg_scene_desc* desc, const int32_t
     int32_t* blk = (int32_t*)(h->ws + L.blk);
     uint8_t* vskip = h->ws + L.vskip;
     uint2* patlas = (uint2*)(h->ws + L.patlas);
-    // the voxel distance transform runs before the padded atlas exists and borrows its
-    // region (8 (B+2)^3 >= 7 B^3 bytes per block) as scratch
-    uint8_t* vscratch = (uint8_t*)patlas;
-
+    // everything is queued before the one wait: an invalid indirection grid (reported from
+    // *err) stops the block kernel before it uses an entry as an index
+    int32_t* d_err = h->hdr + kHdrCreateErr;
     cudaError_t e = cudaMemsetAsync(h->hdr, 0, kAlign, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ws_ind, d_indirection, (size_t)G3 * 4, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess && num_blocks > 0) e = cudaMemsetAsync(blk, 0xff, (size_t)num_blocks * 4, st);
-    if (e == cudaSuccess) e = launch_validate(ws_ind, G3, num_blocks, blk, h->hdr + kHdrCreateErr, st);
+    if (e == cudaSuccess) e = launch_validate(d_indirection, G3, num_blocks, blk, d_err, st);
+    h->launches = 1;
+    if (e == cudaSuccess)
+        e = launch_block_distance_octants(d_indirection, G, kBlockDistCap, btmp, btmp + G3, bdist, ws_ind, &h->launches,
+                                          st);
+    if (e == cudaSuccess)
+        e = launch_prep_blocks(d_indirection, blk, d_err, d_atlas, num_blocks, G, ilog2_exact(B), patlas, vskip, st);
+    if (num_blocks > 0) h->launches++;
     int32_t err = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, h->hdr + kHdrCreateErr, 4, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, d_err, 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { delete h; return SNERG_E_CUDA; }
     if (err != 0) { delete h; return SNERG_E_INVAL; }
-    // the padded atlas reads occupancy from ws_ind, whose sign every octant copy keeps
-    e = launch_block_distance_octants(ws_ind, G, kBlockDistCap, btmp, btmp + G3, bdist, ws_ind, st);
-    if (e == cudaSuccess) e = launch_voxel_distance_octants(d_atlas, num_blocks, B, vscratch, vskip, st);
-    if (e == cudaSuccess)
-        e = launch_build_padded(ws_ind, blk, d_atlas, num_blocks, N, B, ilog2_exact(B), patlas, st);
-    if (e == cudaSuccess) e = launch_fill_vskip_border(vskip, blk, num_blocks, N, B, ilog2_exact(B), 8, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) { delete h; return SNERG_E_CUDA; }
-    h->launches = 2 + 8 * 5 + (num_blocks > 0 ? 15 + 1 + 1 : 0);
 
     DevScene& s = h->ds;
     s.ind = ws_ind;

@@ -976,19 +976,16 @@ cudaError_t launch_backward_rays(const DevScene& s, const CamTable& cams, int32_
                                  const int32_t* fwd_counts, float* grad_atlas, float* grad_mlp, cudaStream_t st);
 cudaError_t launch_validate(const int32_t* ind, int64_t n_ind, int64_t nb, int32_t* blk_of_slot, int32_t* err,
                             cudaStream_t st);
-cudaError_t launch_build_padded(const int32_t* ind, const int32_t* blk_of_slot, const uint8_t* atlas, int64_t nb,
-                                int N, int B, int lgB, uint2* patlas, cudaStream_t st);
-// Chebyshev distance maps (three separable passes, distances capped at `cap`):
-// block level over the G^3 indirection grid, voxel level inside each stored block.
-// The render maps are per octant of the ray direction (distances inside its cone).
+// the padded atlas and the 8 octants' voxel-distance planes of every stored block; a launch
+// that finds *err set does nothing
+cudaError_t launch_prep_blocks(const int32_t* ind, const int32_t* blk_of_slot, const int32_t* err, const uint8_t* atlas,
+                               int64_t nb, int G, int lgB, uint2* patlas, uint8_t* vskip, cudaStream_t st);
+// Chebyshev distance maps over the G^3 indirection grid, distances capped at `cap`: the
+// two-sided one, and the render's (per octant of the ray direction, inside its cone).
 cudaError_t launch_block_distance(const int32_t* ind, int G, int cap, uint8_t* tmp0, uint8_t* tmp1,
                                   uint8_t* bdist, cudaStream_t st);
 cudaError_t launch_block_distance_octants(const int32_t* ind, int G, int cap, uint8_t* tmp0, uint8_t* tmp1,
-                                          uint8_t* bdist, int32_t* ind_oct, cudaStream_t st);
-cudaError_t launch_voxel_distance_octants(const uint8_t* atlas, int64_t nb, int B, uint8_t* scratch, uint8_t* vskip,
-                                          cudaStream_t st);
-cudaError_t launch_fill_vskip_border(uint8_t* vskip, const int32_t* blk_of_slot, int64_t nb, int N, int B, int lgB,
-                                     int n_planes, cudaStream_t st);
+                                          uint8_t* bdist, int32_t* ind_oct, int64_t* launches, cudaStream_t st);
 
 struct PersistentParams {
     snerg_camera cams[kMaxCams];

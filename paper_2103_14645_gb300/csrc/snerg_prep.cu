@@ -1,6 +1,6 @@
 // snerg_prep.cu -- scene set-up kernels: validate the indirection grid (Sec. 5.1),
 // build the device layout of the atlas (apron-padded blocks) and the two Chebyshev
-// distance maps the march uses to skip empty space.
+// distance maps the march uses to skip empty space; requantise fine-tuned values.
 //
 // The paper's viewer keeps density in its own 8-bit texture so that empty space inside
 // occupied blocks costs one byte per sample (App. A); the voxel distance plane here
@@ -22,35 +22,6 @@ __global__ void validate_kernel(const int32_t* __restrict__ ind, int64_t n_ind, 
         } else if (v >= 0) {
             if (atomicCAS(blk_of_slot + v, -1, (int32_t)i) != -1) atomicOr(err, 2);
         }
-    }
-}
-
-// One thread per padded voxel. Padded coordinate p in [0, B+2) maps to the global voxel
-// block_origin + p - 1, clamped to the grid (clamp-to-edge at the border); its owner
-// block supplies the value, or 0 if that block is empty.
-__global__ void build_padded_kernel(const int32_t* __restrict__ ind, const int32_t* __restrict__ blk_of_slot,
-                                    const uint2* __restrict__ atlas, int64_t nb, int N, int B, int lgB,
-                                    uint2* __restrict__ patlas) {
-    const int P = B + 2, P3 = P * P * P, G = N >> lgB;
-    const int64_t total = nb * (int64_t)P3;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t slot = t / P3;
-        const int r = (int)(t - slot * P3);
-        const int px = r % P, py = (r / P) % P, pz = r / (P * P);
-        const int blk = blk_of_slot[slot];
-        uint2 v = make_uint2(0u, 0u);
-        if (blk >= 0) {
-            const int bx = blk % G, by = (blk / G) % G, bz = blk / (G * G);
-            const int gx = min(max(bx * B + px - 1, 0), N - 1);
-            const int gy = min(max(by * B + py - 1, 0), N - 1);
-            const int gz = min(max(bz * B + pz - 1, 0), N - 1);
-            const int owner = ind[((gz >> lgB) * G + (gy >> lgB)) * G + (gx >> lgB)];
-            if (owner >= 0) {
-                const int loc = ((gz & (B - 1)) * B + (gy & (B - 1))) * B + (gx & (B - 1));
-                v = atlas[(int64_t)owner * B * B * B + loc];
-            }
-        }
-        patlas[t] = v;
     }
 }
 
@@ -146,34 +117,9 @@ __global__ void block_seed_kernel(const int32_t* __restrict__ ind, int64_t n, in
         out[t] = ind[t] >= 0 ? 0 : (uint8_t)cap;
 }
 
-// 0 where the voxel's density code is non-zero, cap elsewhere (unpadded [nb][B^3])
-__global__ void voxel_seed_kernel(const uint8_t* __restrict__ atlas, int64_t n, int cap, uint8_t* __restrict__ out) {
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-        out[t] = atlas[t * 8] != 0 ? 0 : (uint8_t)cap;
-}
-
-// z pass of the voxel transform, written into the padded plane (apron cells = 255)
-__global__ void dt_pass_z_padded_kernel(const uint8_t* __restrict__ in, uint8_t* __restrict__ vskip, int B,
-                                        int64_t nb, int cap, int side) {
-    const int P = B + 2, P3 = P * P * P;
-    const int64_t B3 = (int64_t)B * B * B;
-    const int64_t total = nb * P3;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t slot = t / P3;
-        const int r = (int)(t - slot * P3);
-        const int px = r % P - 1, py = (r / P) % P - 1, pz = r / (P * P) - 1;
-        uint8_t v = 255;
-        if (px >= 0 && py >= 0 && pz >= 0 && px < B && py < B && pz < B) {
-            const int64_t base = slot * B3 + (int64_t)py * B + px;
-            v = (uint8_t)dt_line(in, base, (int64_t)B * B, pz, B, cap, side);
-        }
-        vskip[t] = v;
-    }
-}
-
 // dst[i] = src[i] for an occupied block, -bdist[i] (>= 1) for an empty one: the march
-// reads one word per block. src and dst may be the same array.
-__global__ void encode_distance_kernel(const int32_t* src, const uint8_t* __restrict__ bdist, int32_t* dst,
+// reads one word per block.
+__global__ void encode_distance_kernel(const int32_t* __restrict__ src, const uint8_t* __restrict__ bdist, int32_t* __restrict__ dst,
                                        int64_t n) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         const int32_t v = src[t];
@@ -181,33 +127,328 @@ __global__ void encode_distance_kernel(const int32_t* src, const uint8_t* __rest
     }
 }
 
-// Apron cells of the voxel-distance plane that lie outside the grid get the value of the
-// voxel they clamp to (clamp-to-edge, as in the padded atlas). A sample that rounding puts
-// a hair outside the grid then finds its clamped nearest voxel's value without a clamp.
-// (n_planes planes of [nb][P^3] one after the other; each is filled from itself)
-__global__ void fill_vskip_border_kernel(uint8_t* __restrict__ vskip, const int32_t* __restrict__ blk_of_slot,
-                                         int64_t nb, int N, int B, int lgB, int n_planes) {
-    const int P = B + 2, P3 = P * P * P, G = N >> lgB;
-    const int64_t total = n_planes * nb * (int64_t)P3;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t ps = t / P3;                       // plane * nb + slot
-        const int64_t slot = ps % nb;
-        const int r = (int)(t - ps * P3);
-        const int p[3] = {r % P, (r / P) % P, r / (P * P)};
-        if (p[0] >= 1 && p[0] <= B && p[1] >= 1 && p[1] <= B && p[2] >= 1 && p[2] <= B) continue;   // interior
-        const int blk = blk_of_slot[slot];
-        if (blk < 0) continue;
-        const int b[3] = {blk % G, (blk / G) % G, blk / (G * G)};
-        int q[3];
-        bool ok = true;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int g = b[i] * B + p[i] - 1;
-            if (p[i] >= 1 && p[i] <= B) { q[i] = p[i]; continue; }
-            if (g >= 0 && g < N) { ok = false; break; }      // faces an interior neighbour: never probed
-            q[i] = min(max(g, 0), N - 1) - b[i] * B + 1;     // the clamped voxel, inside this block
+// ---------------------------------------------------------------------------------
+// The device layout of the stored blocks, one CTA of 8 warps for one block (B >= 32) or
+// for 32 / B blocks side by side in a warp's lanes:
+//   1. the block's voxels are read once, row by row, copied into the padded atlas, and each
+//      row's non-zero density codes kept as a bit mask in shared memory;
+//   2. the apron: padded coordinate p in [0, B+2) is the global voxel block_origin + p - 1,
+//      clamped to the grid (clamp-to-edge); its owner block supplies the value, 0 if empty;
+//   3. warp o computes octant o's voxel distances from the masks, with no pass over memory
+//      but the store of the result. The distance to the nearest set voxel in the cone obeys
+//          D(p) = 0 if p is set, else 1 + min over the 7 neighbours p + {0, 1}^3 \ 0
+//      (steps in the cone's directions). Along x, D(x) <= 1 + D(x + 1) in the rows already
+//      done, so all of a row's candidates but two reduce to the distance to the row's own next
+//      set bit: D = min(bits, 1 + m(x), 1 + m(x + 1)), m the minimum over the three rows behind
+//      at y + 1 and z + 1. Lanes hold x in the order that puts the cone's next voxel into the
+//      lane before, the z + 1 slice stays in registers, and a row costs about 14 instructions
+//      without any barrier.
+// Apron cells of the distance planes hold 255, or, outside the grid, the value of the voxel
+// that they clamp to, so that a sample which rounding puts a hair outside the grid finds its
+// clamped nearest voxel's value without a clamp.
+// Bound by issue and by the latency of the first two parts: 0.77 ms for 2,144 blocks of 32^3,
+// whose 1.8 GB read and written would take 0.27 ms at the copy rate. Separate seed, x, y, z,
+// apron and border passes with a scan per voxel took 25.4 ms.
+// ---------------------------------------------------------------------------------
+constexpr int kPrepThreads = 256;
+
+template <int LGB>
+struct PrepShape {
+    static constexpr int B = 1 << LGB, P = B + 2, P2 = P * P, P3 = P2 * P, B2 = B * B, B3 = B2 * B;
+    static constexpr int LX = B < 32 ? B : 32;      // lanes along x
+    static constexpr int NB = 32 / LX;              // blocks per CTA
+    static constexpr int VPL = B / LX;              // voxels per lane along x (2 for B = 64)
+    static constexpr int kApron = P3 - B3;
+    static constexpr int kMinCtas = VPL == 2 ? 2 : 4;
+    static constexpr int kSmem = 2 * VPL * B2 * 4 + kPrepThreads / 32 * NB * P2;    // row masks, slices
+};
+
+// the cone distance of one row: prev / pprev the z + 1 slice's rows y and y + 1, cur the row
+// y + 1 (16-bit pairs for two voxels per lane); wa, wb the row's masks in lane order
+template <int VPL>
+__device__ __forceinline__ uint32_t prep_row(uint32_t cur, uint32_t prev, uint32_t pprev, uint32_t wa, uint32_t wb,
+                                             int lane, uint32_t le, uint32_t lt, int lx) {
+    if (VPL == 1) {
+        const int m = (int)min(min(cur, prev), pprev);
+        const int mx = __shfl_up_sync(0xffffffffu, m, 1, lx);     // the first lane of a block gets its own m back
+        int D = __viaddmin_s32(min(m, mx), 1, 255);
+        if (wa) {                                                 // the same for all lanes
+            const uint32_t t = wa & le;
+            if (t) D = min(D, lane - (31 - __clz(t)));
         }
-        if (ok) vskip[t] = vskip[ps * P3 + (q[2] * P + q[1]) * P + q[0]];
+        return (uint32_t)D;
+    }
+    const uint32_t m = __vminu2(__vminu2(cur, prev), pprev);
+    uint32_t up = __shfl_up_sync(0xffffffffu, m, 1);
+    if (lane == 0) up = 0x00ff00ffu;
+    const uint32_t mx = __byte_perm(m, up, 0x1076);               // (low: the lane before's high; high: own low)
+    uint32_t D = __vminu2(__vadd2(__vminu2(m, mx), 0x00010001u), 0x00ff00ffu);
+    if (wa | wb) {
+        const uint32_t ta = wa & le, tb = wb & le, ua = wb & lt;
+        const int la = 31 - __clz(ta), lb = 31 - __clz(tb), lu = 31 - __clz(ua);
+        const int da = min(ta ? 2 * (lane - la) : 255, ua ? 2 * (lane - lu) - 1 : 255);
+        const int db = min(tb ? 2 * (lane - lb) : 255, ta ? 2 * (lane - la) + 1 : 255);
+        D = __vminu2(D, (uint32_t)da | ((uint32_t)db << 16));
+    }
+    return D;
+}
+
+// one slice (z) of one octant's plane into shared memory; SY: the cone's side along y
+template <int LGB, bool SY>
+__device__ __forceinline__ void prep_slice(uint32_t (&prev)[1 << LGB], const uint32_t* ma, const uint32_t* mb,
+                                           uint8_t* out_a, uint8_t* out_b, int lane, uint32_t le, uint32_t lt) {
+    using S = PrepShape<LGB>;
+    uint32_t cur = S::VPL == 1 ? 255u : 0x00ff00ffu, pprev = cur;
+#pragma unroll
+    for (int yi = 0; yi < S::B; ++yi) {
+        const int y = SY ? yi : S::B - 1 - yi;
+        cur = prep_row<S::VPL>(cur, prev[yi], pprev, ma[y], S::VPL == 2 ? mb[y] : 0u, lane, le, lt, S::LX);
+        pprev = prev[yi];
+        prev[yi] = cur;
+        out_a[(y + 1) * S::P] = (uint8_t)cur;
+        if (S::VPL == 2) out_b[(y + 1) * S::P] = (uint8_t)(cur >> 16);
+    }
+}
+
+template <int LGB>
+__global__ void __launch_bounds__(kPrepThreads, PrepShape<LGB>::kMinCtas) prep_blocks_kernel(
+    const int32_t* __restrict__ ind, const int32_t* __restrict__ blk_of_slot, const int32_t* __restrict__ err,
+    const uint2* __restrict__ atlas, int64_t nb, int G, uint2* __restrict__ patlas, uint8_t* __restrict__ vskip) {
+    using S = PrepShape<LGB>;
+    constexpr int B = S::B, P = S::P, LX = S::LX;
+    extern __shared__ __align__(16) uint32_t s_mem[];
+    // a row's mask: bit g * LX + x (VPL 2: one word for even, one for odd x), and bit-reversed
+    uint32_t(*s_mask)[S::VPL][S::B2] = reinterpret_cast<uint32_t(*)[S::VPL][S::B2]>(s_mem);
+    // a warp's slice of its plane
+    uint8_t(*s_slice)[S::NB][S::P2] = reinterpret_cast<uint8_t(*)[S::NB][S::P2]>(s_mem + 2 * S::VPL * S::B2);
+    __shared__ int s_own[S::NB][27];             // slots of the 3^3 blocks around, -1 empty
+    __shared__ int s_edge[S::NB];                // bit 2 a (+ 1): first (last) block along axis a
+    if (*err) return;                            // an invalid indirection grid: the host reports it
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t slot0 = (int64_t)blockIdx.x * S::NB;
+    for (int i = tid; i < S::NB * 27; i += kPrepThreads) {
+        const int g = i / 27, k = i % 27;
+        const int blk = slot0 + g < nb ? blk_of_slot[slot0 + g] : -1;
+        int own = -1;
+        if (blk >= 0) {
+            const int bx = blk % G, by = (blk / G) % G, bz = blk / (G * G);
+            const int x = min(max(bx + k % 3 - 1, 0), G - 1), y = min(max(by + (k / 3) % 3 - 1, 0), G - 1),
+                      z = min(max(bz + k / 9 - 1, 0), G - 1);
+            own = ind[((int64_t)z * G + y) * G + x];
+            if (k == 0)
+                s_edge[g] = (bx == 0 ? 1 : 0) | (bx == G - 1 ? 2 : 0) | (by == 0 ? 4 : 0) | (by == G - 1 ? 8 : 0) |
+                            (bz == 0 ? 16 : 0) | (bz == G - 1 ? 32 : 0);
+        } else if (k == 0) {
+            s_edge[g] = 0;
+        }
+        s_own[g][k] = own;
+    }
+    __syncthreads();
+
+    // 1. the blocks' own voxels (an unreferenced slot is stored as zeros)
+    {
+        const int g = lane / LX, x = lane % LX;
+        const int64_t slot = slot0 + g;
+        const bool in = slot < nb, used = in && s_own[g][13] >= 0;
+        const uint2* src = atlas + slot * S::B3;
+        uint2* dst = patlas + slot * S::P3 + S::P2 + P + 1;
+        // kRows rows' loads in flight (the votes keep them from being moved up)
+        constexpr int kRows = 8, kWarps = kPrepThreads / 32;
+        for (int r0 = warp; r0 < S::B2; r0 += kRows * kWarps) {
+            uint2 v[kRows][S::VPL];
+#pragma unroll
+            for (int u = 0; u < kRows; ++u)
+#pragma unroll
+                for (int q = 0; q < S::VPL; ++q) {
+                    const int row = r0 + u * kWarps;
+                    const bool on = used && (S::B2 % (kRows * kWarps) == 0 || row < S::B2);
+                    // 8-byte loads: the atlas need not be aligned to more
+                    v[u][q] = on ? __ldg(src + row * B + S::VPL * x + q) : make_uint2(0u, 0u);
+                }
+#pragma unroll
+            for (int u = 0; u < kRows; ++u) {
+                const int row = r0 + u * kWarps;
+                if (S::B2 % (kRows * kWarps) != 0 && row >= S::B2) break;
+                uint2* d = dst + ((row >> LGB) * P + (row & (B - 1))) * P + S::VPL * x;
+#pragma unroll
+                for (int q = 0; q < S::VPL; ++q) {
+                    if (in) d[q] = v[u][q];
+                    const uint32_t m = __ballot_sync(0xffffffffu, (v[u][q].x & 0xffu) != 0u);
+                    if (lane == 0) {
+                        s_mask[0][S::VPL - 1 - q][row] = __brev(m);
+                        s_mask[1][q][row] = m;
+                    }
+                }
+            }
+        }
+    }
+    // 2. the apron: two z faces of P x P, two y faces of P x B, two x faces of B x B
+    constexpr int kCells = 4;       // loads in flight per thread
+    for (int i0 = tid; i0 < S::NB * S::kApron; i0 += kCells * kPrepThreads) {
+        uint2 v[kCells];
+        int64_t at[kCells];
+#pragma unroll
+        for (int u = 0; u < kCells; ++u) {
+            const int i = i0 + u * kPrepThreads, g = i / S::kApron;
+            int a = i % S::kApron, px, py, pz;
+            at[u] = -1;
+            if (i >= S::NB * S::kApron || slot0 + g >= nb) continue;
+            if (a < 2 * S::P2) {
+                pz = a < S::P2 ? 0 : P - 1;
+                a %= S::P2;
+                py = a / P;
+                px = a % P;
+            } else if (a < 2 * S::P2 + 2 * P * B) {
+                a -= 2 * S::P2;
+                py = a < P * B ? 0 : P - 1;
+                a %= P * B;
+                pz = 1 + a / P;
+                px = a % P;
+            } else {
+                a -= 2 * S::P2 + 2 * P * B;
+                px = a < S::B2 ? 0 : P - 1;
+                a %= S::B2;
+                pz = 1 + a / B;
+                py = 1 + a % B;
+            }
+            const int p[3] = {px, py, pz};
+            int l[3], k = 0;
+            const int edge = s_edge[g];
+#pragma unroll
+            for (int c = 2; c >= 0; --c) {
+                const int n = p[c] == 0 ? 0 : (p[c] == P - 1 ? 2 : 1);
+                k = k * 3 + n;
+                // the neighbour's facing voxel, or the clamped one of this block's
+                l[c] = n == 1 ? p[c] - 1 : (n == 0 ? ((edge >> (2 * c)) & 1 ? 0 : B - 1) : ((edge >> (2 * c + 1)) & 1 ? B - 1 : 0));
+            }
+            const int own = s_own[g][k];
+            at[u] = (slot0 + g) * S::P3 + (pz * P + py) * P + px;
+            v[u] = own >= 0 ? __ldg(atlas + (int64_t)own * S::B3 + (l[2] * B + l[1]) * B + l[0]) : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < kCells; ++u)
+            if (at[u] >= 0) patlas[at[u]] = v[u];
+    }
+    __syncthreads();
+
+    // 3. warp o: octant o's distance plane
+    const int o = warp;
+    const bool sx = o & 1, sy = o & 2, sz = o & 4;        // set: the cone runs towards lower coordinates
+    const int bit = sx ? lane : 31 - lane;                // this lane's bit in a row's mask
+    const int g = S::VPL == 1 ? bit / LX : 0;
+    const uint32_t le = (2u << lane) - 1u, lt = le >> 1;
+    const uint32_t own_le = S::VPL == 1 ? le & ~((1u << (lane / LX * LX)) - 1u) : le;
+    // this lane's voxel(s) along x: xa (whose cone neighbour is in the lane before) and xb
+    const int xa = S::VPL == 1 ? bit % LX : 2 * bit + (sx ? 0 : 1);
+    const int xb = S::VPL == 1 ? xa : xa ^ 1;
+    uint32_t prev[B];
+#pragma unroll
+    for (int y = 0; y < B; ++y) prev[y] = S::VPL == 1 ? 255u : 0x00ff00ffu;
+    const uint32_t* mask_a = s_mask[sx][0];
+    const uint32_t* mask_b = s_mask[sx][S::VPL - 1];
+    uint8_t* out_a = s_slice[warp][g] + 1 + xa;
+    uint8_t* out_b = s_slice[warp][g] + 1 + xb;
+#pragma unroll 1
+    for (int zi = 0; zi < B; ++zi) {
+        const int z = sz ? zi : B - 1 - zi;
+        if (sy) prep_slice<LGB, true>(prev, mask_a + z * B, mask_b + z * B, out_a, out_b, lane, own_le, lt);
+        else prep_slice<LGB, false>(prev, mask_a + z * B, mask_b + z * B, out_a, out_b, lane, own_le, lt);
+        __syncwarp();
+        // the x and then the y apron: 255, or outside the grid the voxel that they clamp to
+        for (int i = lane; i < S::NB * 2 * B; i += 32) {
+            const int gi = i / (2 * B), hi = i & 1, py = 1 + ((i % (2 * B)) >> 1);
+            uint8_t* sl = s_slice[warp][gi] + py * P;
+            sl[hi ? P - 1 : 0] = (s_edge[gi] >> hi) & 1 ? sl[hi ? B : 1] : (uint8_t)255;
+        }
+        __syncwarp();
+        for (int i = lane; i < S::NB * 2 * P; i += 32) {
+            const int gi = i / (2 * P), q = i % (2 * P), hi = q >= P, px = hi ? q - P : q;
+            uint8_t* sl = s_slice[warp][gi];
+            sl[(hi ? P - 1 : 0) * P + px] = (s_edge[gi] >> (2 + hi)) & 1 ? sl[(hi ? B : 1) * P + px] : (uint8_t)255;
+        }
+        __syncwarp();
+        // the slice goes out in words (P^2 and P^3 are multiples of 4), and once more where it
+        // is beside the z apron: there as 255, or outside the grid as it is
+        for (int i = lane; i < S::NB * (S::P2 / 4); i += 32) {
+            const int gi = i / (S::P2 / 4), q = i % (S::P2 / 4);
+            if (slot0 + gi >= nb) break;
+            const uint32_t w = reinterpret_cast<const uint32_t*>(s_slice[warp][gi])[q];
+            uint32_t* d = reinterpret_cast<uint32_t*>(vskip + ((int64_t)o * nb + slot0 + gi) * S::P3 + (z + 1) * S::P2) + q;
+            *d = w;
+            if (z == 0) d[-(S::P2 / 4)] = (s_edge[gi] & 16) ? w : 0xffffffffu;
+            if (z == B - 1) d[S::P2 / 4] = (s_edge[gi] & 32) ? w : 0xffffffffu;
+        }
+        __syncwarp();
+    }
+}
+
+// ---------------------------------------------------------------------------------
+// The block-level maps of grids of up to 64 blocks a side, one CTA per octant o:
+// ind_oct[o] = the indirection grid with every empty entry replaced by -D, D >= 1 the
+// Chebyshev distance (capped) to the nearest occupied block of o's cone, by the same
+// recurrence as the voxel maps. Rows on one anti-diagonal y + z = s depend only on the two
+// diagonals before and go to the CTA's warps side by side. A grid of 32^3 blocks takes 33 us;
+// separate seed, x, y, z and encode passes were 40 launches and 240 us.
+// ---------------------------------------------------------------------------------
+constexpr int kMapThreads = 1024, kMapMaxG = 64;
+
+// W: 32-block words per row
+template <int W>
+__global__ void __launch_bounds__(kMapThreads) block_maps_kernel(const int32_t* __restrict__ ind, int G, int cap,
+                                                                 int32_t* __restrict__ ind_oct) {
+    constexpr int M = 32 * W;
+    __shared__ uint32_t s_bits[M * M][W];              // occupied blocks of a row in the cone's order along x
+    // distances of the last three diagonals by row y + 1; rows that a diagonal does not have
+    // (y = -1, z = -1) keep the cap
+    __shared__ uint8_t s_diag[3][M + 1][M];
+    const int o = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool sx = o & 1, sy = o & 2, sz = o & 4;
+    int32_t* out = ind_oct + (int64_t)o * G * G * G;
+    for (int i = threadIdx.x; i < 3 * (M + 1) * M; i += kMapThreads) (&s_diag[0][0][0])[i] = (uint8_t)cap;
+    // occupied blocks keep their slot; the diagonals below write the empty ones
+#pragma unroll 4
+    for (int row = warp; row < G * G; row += kMapThreads / 32) {
+#pragma unroll
+        for (int h = 0; h < W; ++h) {
+            const int c = 32 * h + lane, i = row * G + (sx ? c : G - 1 - c);
+            const int32_t v = c < G ? __ldg(ind + i) : -1;
+            if (v >= 0) out[i] = v;
+            const uint32_t m = __ballot_sync(0xffffffffu, v >= 0);
+            if (lane == 0) s_bits[row][h] = m;
+        }
+    }
+    __syncthreads();
+    const uint32_t le = (2u << lane) - 1u;
+    int b0 = 0, b1 = 2, b2 = 1;                        // this diagonal's buffer and the two before
+    for (int s = 0; s <= 2 * (G - 1); ++s) {
+        for (int yi = max(0, s - G + 1) + warp; yi <= min(s, G - 1); yi += kMapThreads / 32) {
+            const int zi = s - yi;
+            const int row = (sz ? zi : G - 1 - zi) * G + (sy ? yi : G - 1 - yi);
+            int carry_m = cap, carry_d = cap;          // of the voxel before the word
+#pragma unroll
+            for (int h = 0; h < W; ++h) {
+                const int c = 32 * h + lane;
+                const int m = min(min((int)s_diag[b1][yi][c], (int)s_diag[b1][yi + 1][c]), (int)s_diag[b2][yi][c]);
+                int mx = __shfl_up_sync(0xffffffffu, m, 1);
+                if (h > 0 && lane == 0) mx = carry_m;
+                const uint32_t t = s_bits[row][h] & le;
+                const int dist = t ? lane - (31 - __clz(t)) : min(cap, carry_d + 1 + lane);
+                const int D = min(min(min(m, mx) + 1, dist), cap);
+                if (h + 1 < W) {
+                    carry_m = __shfl_sync(0xffffffffu, m, 31);
+                    carry_d = __shfl_sync(0xffffffffu, dist, 31);
+                }
+                if (c < G) {
+                    s_diag[b0][yi + 1][c] = (uint8_t)D;
+                    if (D > 0) out[row * G + (sx ? c : G - 1 - c)] = -D;
+                }
+            }
+        }
+        __syncthreads();
+        const int t = b2;
+        b2 = b1;
+        b1 = b0;
+        b0 = t;
     }
 }
 
@@ -232,42 +473,25 @@ cudaError_t launch_block_distance(const int32_t* ind, int G, int cap, uint8_t* t
     return cudaGetLastError();
 }
 
-// For each octant o, ind_oct[o] = the indirection grid with every empty entry replaced by
+// For each octant o, ind_oct[o] = the indirection grid `ind` with every empty entry replaced by
 // -D_o, D_o >= 1 the Chebyshev distance (in blocks, capped) to the nearest occupied block
-// in o's cone. `ind` may be ind_oct[0].
+// in o's cone. Grids beyond block_maps_kernel's shared memory run one pass per axis and
+// octant over tmp0, tmp1 and bdist (G^3 bytes each). Adds the launches to *launches.
 cudaError_t launch_block_distance_octants(const int32_t* ind, int G, int cap, uint8_t* tmp0, uint8_t* tmp1,
-                                          uint8_t* bdist, int32_t* ind_oct, cudaStream_t st) {
+                                          uint8_t* bdist, int32_t* ind_oct, int64_t* launches, cudaStream_t st) {
     const int64_t n = (int64_t)G * G * G;
-    for (int o = 7; o >= 0; --o) {          // octant 0 last: ind may alias its copy
+    if (G <= kMapMaxG) {
+        if (G <= 32) block_maps_kernel<1><<<8, kMapThreads, 0, st>>>(ind, G, cap, ind_oct);
+        else block_maps_kernel<2><<<8, kMapThreads, 0, st>>>(ind, G, cap, ind_oct);
+        *launches += 1;
+        return cudaGetLastError();
+    }
+    for (int o = 0; o < 8; ++o) {
         const int side[3] = {octant_side(o, 0), octant_side(o, 1), octant_side(o, 2)};
         block_distance(ind, G, cap, tmp0, tmp1, bdist, side, st);
         encode_distance_kernel<<<grid_for(n), 256, 0, st>>>(ind, bdist, ind_oct + (size_t)o * n, n);
     }
-    return cudaGetLastError();
-}
-
-// For each octant o, plane o of vskip ([8][nb][P^3]) holds per interior voxel the
-// Chebyshev distance to the nearest voxel of the same block with a non-zero density code
-// in o's cone (apron cells 255; the grid-border apron is filled afterwards). The x pass
-// depends only on o's x side, the y pass on its x and y sides, so the eight transforms
-// share them: 2 x passes, 4 y passes, 8 z passes. `scratch` holds 7 nb B^3 bytes.
-cudaError_t launch_voxel_distance_octants(const uint8_t* atlas, int64_t nb, int B, uint8_t* scratch, uint8_t* vskip,
-                                          cudaStream_t st) {
-    if (nb <= 0) return cudaSuccess;
-    const int64_t n = nb * (int64_t)B * B * B;
-    const int64_t plane = nb * (int64_t)(B + 2) * (B + 2) * (B + 2);
-    const int cap = 255;
-    uint8_t* seed = scratch;
-    uint8_t* xs = scratch + n;          // [2][n]: x side (bit 0 of o)
-    uint8_t* ys = scratch + 3 * n;      // [4][n]: x and y sides (bits 0, 1 of o)
-    voxel_seed_kernel<<<grid_for(n), 256, 0, st>>>(atlas, n, cap, seed);
-    for (int a = 0; a < 2; ++a)
-        dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(seed, xs + a * n, B, nb, 0, cap, octant_side(a, 0));
-    for (int a = 0; a < 4; ++a)
-        dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(xs + (a & 1) * n, ys + a * n, B, nb, 1, cap, octant_side(a, 1));
-    for (int o = 0; o < 8; ++o)
-        dt_pass_z_padded_kernel<<<grid_for(plane), 256, 0, st>>>(ys + (o & 3) * n, vskip + (size_t)o * plane, B, nb,
-                                                                 cap, octant_side(o, 2));
+    *launches += 8 * 5;
     return cudaGetLastError();
 }
 
@@ -279,13 +503,32 @@ cudaError_t launch_validate(const int32_t* ind, int64_t n_ind, int64_t nb, int32
     return cudaGetLastError();
 }
 
-cudaError_t launch_build_padded(const int32_t* ind, const int32_t* blk_of_slot, const uint8_t* atlas, int64_t nb,
-                                int N, int B, int lgB, uint2* patlas, cudaStream_t st) {
-    if (nb <= 0) return cudaSuccess;
-    const int64_t total = nb * (int64_t)(B + 2) * (B + 2) * (B + 2);
-    build_padded_kernel<<<grid_for(total), 256, 0, st>>>(ind, blk_of_slot, reinterpret_cast<const uint2*>(atlas), nb,
-                                                          N, B, lgB, patlas);
+template <int LGB>
+static cudaError_t prep_blocks(const int32_t* ind, const int32_t* blk_of_slot, const int32_t* err,
+                               const uint8_t* atlas, int64_t nb, int G, uint2* patlas, uint8_t* vskip, cudaStream_t st) {
+    constexpr int n = PrepShape<LGB>::NB, smem = PrepShape<LGB>::kSmem;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(prep_blocks_kernel<LGB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   smem);
+        if (e != cudaSuccess) return e;
+    }
+    prep_blocks_kernel<LGB><<<(unsigned)((nb + n - 1) / n), kPrepThreads, smem, st>>>(
+        ind, blk_of_slot, err, reinterpret_cast<const uint2*>(atlas), nb, G, patlas, vskip);
     return cudaGetLastError();
+}
+
+cudaError_t launch_prep_blocks(const int32_t* ind, const int32_t* blk_of_slot, const int32_t* err, const uint8_t* atlas,
+                               int64_t nb, int G, int lgB, uint2* patlas, uint8_t* vskip, cudaStream_t st) {
+    if (nb <= 0) return cudaSuccess;
+    switch (lgB) {
+        case 1: return prep_blocks<1>(ind, blk_of_slot, err, atlas, nb, G, patlas, vskip, st);
+        case 2: return prep_blocks<2>(ind, blk_of_slot, err, atlas, nb, G, patlas, vskip, st);
+        case 3: return prep_blocks<3>(ind, blk_of_slot, err, atlas, nb, G, patlas, vskip, st);
+        case 4: return prep_blocks<4>(ind, blk_of_slot, err, atlas, nb, G, patlas, vskip, st);
+        case 5: return prep_blocks<5>(ind, blk_of_slot, err, atlas, nb, G, patlas, vskip, st);
+        case 6: return prep_blocks<6>(ind, blk_of_slot, err, atlas, nb, G, patlas, vskip, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_requantize_padded(const int32_t* ind, const int32_t* blk_of_slot, const float* values, int64_t nb,
@@ -295,14 +538,6 @@ cudaError_t launch_requantize_padded(const int32_t* ind, const int32_t* blk_of_s
     requantize_padded_kernel<<<grid_for(total), 256, 0, st>>>(ind, blk_of_slot, reinterpret_cast<const float4*>(values),
                                                                nb, N, B, lgB, patlas,
                                                                reinterpret_cast<uint2*>(atlas_out));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fill_vskip_border(uint8_t* vskip, const int32_t* blk_of_slot, int64_t nb, int N, int B, int lgB,
-                                     int n_planes, cudaStream_t st) {
-    if (nb <= 0) return cudaSuccess;
-    fill_vskip_border_kernel<<<grid_for(n_planes * nb * (int64_t)(B + 2) * (B + 2) * (B + 2)), 256, 0, st>>>(
-        vskip, blk_of_slot, nb, N, B, lgB, n_planes);
     return cudaGetLastError();
 }
 }  // namespace snerg
