@@ -278,6 +278,14 @@ snerg_status snerg_grad_blocks_scatter(const float* d_packed, const int32_t* d_l
  * render the new codes. */
 snerg_status snerg_requantize_atlas(snerg_handle h, const float* d_values, uint8_t* d_atlas_out, void* stream);
 
+/* snerg_adam_step on d_values (n = all their floats, channel 0 included) followed by
+ * snerg_requantize_atlas, in one pass over the values: the end of a fine-tuning step that
+ * also tunes the baked colours and features. Arguments as for the two calls, except that
+ * d_values, d_m, d_v and d_grad must be 16-byte aligned. */
+snerg_status snerg_adam_requantize_atlas(snerg_handle h, float* d_values, float* d_m, float* d_v,
+                                         const float* d_grad, float lr, float beta1, float beta2, float eps,
+                                         int32_t step, uint8_t* d_atlas_out, void* stream);
+
 /* One fine-tuning step's render, loss and adjoint for a ray list in a single launch (Sec.
  * 5.5, Eq. 3): each ray is marched and shaded as by snerg_render_rays, its L2 loss
  * |C - C*|^2 is ADDED to *d_loss (caller zeroes; nullable), dL/dC = 2 (C - C*) is taken in

@@ -987,6 +987,38 @@ cudaError_t launch_block_distance(const int32_t* ind, int G, int cap, uint8_t* t
 cudaError_t launch_block_distance_octants(const int32_t* ind, int G, int cap, uint8_t* tmp0, uint8_t* tmp1,
                                           uint8_t* bdist, int32_t* ind_oct, int64_t* launches, cudaStream_t st);
 
+// Adam's constants for one step (Sec. 5.5): c1, c2 the bias corrections 1 - b^step
+struct AdamArgs {
+    float lr, b1, b2, eps, c1, c2;
+};
+
+// One Adam step on four parameters: m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
+// p -= lr (m / c1) / (sqrt(v / c2) + eps). Where gradient and moments are all zero nothing
+// changes (finite lr), and false is returned: most voxels of a fine-tuned grid are never
+// touched, and three exact divisions and a root per parameter are what such a pass would be
+// bound by.
+__device__ __forceinline__ bool adam_quad(const AdamArgs& a, const float4& g, float4& m, float4& v, float4& p) {
+    const float ga[4] = {g.x, g.y, g.z, g.w};
+    float ma[4] = {m.x, m.y, m.z, m.w}, va[4] = {v.x, v.y, v.z, v.w}, pa[4] = {p.x, p.y, p.z, p.w};
+    uint32_t bits = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) bits |= __float_as_uint(ga[k]) | __float_as_uint(ma[k]) | __float_as_uint(va[k]);
+    if (bits == 0u && a.lr < INFINITY) return false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        ma[k] = a.b1 * ma[k] + (1.0f - a.b1) * ga[k];
+        va[k] = a.b2 * va[k] + (1.0f - a.b2) * ga[k] * ga[k];
+        pa[k] -= a.lr * (ma[k] / a.c1) / (sqrtf(va[k] / a.c2) + a.eps);
+    }
+    m = make_float4(ma[0], ma[1], ma[2], ma[3]);
+    v = make_float4(va[0], va[1], va[2], va[3]);
+    p = make_float4(pa[0], pa[1], pa[2], pa[3]);
+    return true;
+}
+
+// host: the constants, false for arguments snerg_adam_step refuses
+bool adam_args(float lr, float beta1, float beta2, float eps, int32_t step, AdamArgs* a);
+
 struct PersistentParams {
     snerg_camera cams[kMaxCams];
     int32_t tile_start[kMaxCams + 1];   // prefix sum of work items per camera

@@ -79,25 +79,27 @@ __global__ void __launch_bounds__(256) block_copy_kernel(const float4* __restric
 }
 
 // The same update four parameters at a time (16-byte loads and stores) for the bulk of a
-// large parameter array.
+// large parameter array; a quad that does not change is not stored.
 __global__ void __launch_bounds__(256) adam4_kernel(float4* __restrict__ p, float4* __restrict__ m,
                                                     float4* __restrict__ v, const float4* __restrict__ g, int64_t n4,
-                                                    float lr, float b1, float b2, float eps, float c1, float c2) {
+                                                    const AdamArgs a) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 gi = g[i];
         float4 mi = m[i], vi = v[i], pi = p[i];
-        const float ga[4] = {gi.x, gi.y, gi.z, gi.w};
-        float ma[4] = {mi.x, mi.y, mi.z, mi.w}, va[4] = {vi.x, vi.y, vi.z, vi.w}, pa[4] = {pi.x, pi.y, pi.z, pi.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            ma[k] = b1 * ma[k] + (1.0f - b1) * ga[k];
-            va[k] = b2 * va[k] + (1.0f - b2) * ga[k] * ga[k];
-            pa[k] -= lr * (ma[k] / c1) / (sqrtf(va[k] / c2) + eps);
+        if (adam_quad(a, g[i], mi, vi, pi)) {
+            m[i] = mi;
+            v[i] = vi;
+            p[i] = pi;
         }
-        m[i] = make_float4(ma[0], ma[1], ma[2], ma[3]);
-        v[i] = make_float4(va[0], va[1], va[2], va[3]);
-        p[i] = make_float4(pa[0], pa[1], pa[2], pa[3]);
     }
+}
+
+bool adam_args(float lr, float beta1, float beta2, float eps, int32_t step, AdamArgs* a) {
+    if (step < 1 || !(lr >= 0.0f) || !(beta1 >= 0.0f && beta1 < 1.0f) || !(beta2 >= 0.0f && beta2 < 1.0f) ||
+        !(eps > 0.0f))
+        return false;
+    *a = AdamArgs{lr, beta1, beta2, eps, (float)(1.0 - std::pow((double)beta1, (double)step)),
+                  (float)(1.0 - std::pow((double)beta2, (double)step))};
+    return true;
 }
 
 static unsigned grid_1d(int64_t n) {
@@ -119,13 +121,10 @@ extern "C" snerg_status snerg_l2_loss(const float* d_rgb, const float* d_target,
 
 extern "C" snerg_status snerg_adam_step(float* d_param, float* d_m, float* d_v, const float* d_grad, int64_t n,
                                         float lr, float beta1, float beta2, float eps, int32_t step, void* stream) {
-    if (n < 0 || step < 1 || !(lr >= 0.0f) || !(beta1 >= 0.0f && beta1 < 1.0f) || !(beta2 >= 0.0f && beta2 < 1.0f) ||
-        !(eps > 0.0f))
-        return SNERG_E_INVAL;
+    AdamArgs a;
+    if (n < 0 || !adam_args(lr, beta1, beta2, eps, step, &a)) return SNERG_E_INVAL;
     if (n == 0) return SNERG_OK;
     if (!d_param || !d_m || !d_v || !d_grad) return SNERG_E_INVAL;
-    const float c1 = (float)(1.0 - std::pow((double)beta1, (double)step));
-    const float c2 = (float)(1.0 - std::pow((double)beta2, (double)step));
     cudaStream_t st = (cudaStream_t)stream;
     const bool aligned = (((uintptr_t)d_param | (uintptr_t)d_m | (uintptr_t)d_v | (uintptr_t)d_grad) & 15u) == 0;
     int64_t done = 0;
@@ -137,12 +136,12 @@ extern "C" snerg_status snerg_adam_step(float* d_param, float* d_m, float* d_v, 
         const int64_t want = (n4 + 255) / 256, cap = (int64_t)sms * 8;
         adam4_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(
             reinterpret_cast<float4*>(d_param), reinterpret_cast<float4*>(d_m), reinterpret_cast<float4*>(d_v),
-            reinterpret_cast<const float4*>(d_grad), n4, lr, beta1, beta2, eps, c1, c2);
+            reinterpret_cast<const float4*>(d_grad), n4, a);
         done = n4 * 4;
     }
     if (done < n)
         adam_kernel<<<grid_1d(n - done), 256, 0, st>>>(d_param + done, d_m + done, d_v + done, d_grad + done,
-                                                       n - done, lr, beta1, beta2, eps, c1, c2);
+                                                       n - done, lr, beta1, beta2, eps, a.c1, a.c2);
     return cudaGetLastError() == cudaSuccess ? SNERG_OK : SNERG_E_CUDA;
 }
 

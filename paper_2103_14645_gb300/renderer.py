@@ -31,7 +31,7 @@ EXPORTED = ["snerg_workspace_bytes", "snerg_create", "snerg_render", "snerg_rend
             "snerg_render_backward", "snerg_last_status", "snerg_launch_count",
             "snerg_persistent_config", "snerg_destroy", "snerg_status_str", "snerg_render_rays_noalloc",
             "snerg_set_mlp", "snerg_l2_loss", "snerg_adam_step", "snerg_bake_workspace_bytes", "snerg_bake",
-            "snerg_requantize_atlas", "snerg_grad_blocks_touched", "snerg_grad_blocks_gather",
+            "snerg_requantize_atlas", "snerg_adam_requantize_atlas", "snerg_grad_blocks_touched", "snerg_grad_blocks_gather",
             "snerg_grad_blocks_scatter", "snerg_render_to_host", "snerg_train_rays", "snerg_schedule_stats"]
 MAX_BAKE_BLOBS = 64
 
@@ -117,6 +117,9 @@ def load_library(path: str = LIB_PATH):
     lib.snerg_grad_blocks_scatter.restype = ctypes.c_int
     lib.snerg_requantize_atlas.argtypes = [P, P, P, P]
     lib.snerg_requantize_atlas.restype = ctypes.c_int
+    lib.snerg_adam_requantize_atlas.argtypes = [P, P, P, P, P, ctypes.c_float, ctypes.c_float, ctypes.c_float,
+                                                ctypes.c_float, i32, P, P]
+    lib.snerg_adam_requantize_atlas.restype = ctypes.c_int
     lib.snerg_bake_workspace_bytes.argtypes = [P]
     lib.snerg_bake_workspace_bytes.restype = ctypes.c_size_t
     lib.snerg_bake.argtypes = [P, P, P, P, i64, P, ctypes.c_size_t, P, P]
@@ -226,19 +229,35 @@ class Renderer:
         """Synchronise and raise if a kernel recorded a device-side error."""
         _check(self.lib.snerg_last_status(self.handle, _stream(self.device)), "device status")
 
+    def _require_atlas(self, atlas_out: torch.Tensor | None, **values: torch.Tensor):
+        shape = (self.nb, self.B, self.B, self.B, 8)
+        for name, t in values.items():
+            _require_cuda(t, name, torch.float32)
+            if tuple(t.shape) != shape:
+                raise ValueError(f"{name} must have the atlas shape [nb, B, B, B, 8]")
+        if atlas_out is not None:
+            _require_cuda(atlas_out, "atlas_out", torch.uint8)
+            if tuple(atlas_out.shape) != shape:
+                raise ValueError("atlas_out must have the atlas shape")
+
     def requantize_atlas(self, values: torch.Tensor, atlas_out: torch.Tensor | None = None):
         """Write fine-tuned colour/feature values (float32 [nb,B,B,B,8], channel 0 ignored)
         into the scene as 8-bit codes (snerg_requantize_atlas); optionally also into
         atlas_out (uint8, same shape, density codes in channel 0)."""
-        _require_cuda(values, "values", torch.float32)
-        if tuple(values.shape) != (self.nb, self.B, self.B, self.B, 8):
-            raise ValueError("values must have the atlas shape [nb, B, B, B, 8]")
-        if atlas_out is not None:
-            _require_cuda(atlas_out, "atlas_out", torch.uint8)
-            if atlas_out.shape != values.shape:
-                raise ValueError("atlas_out must have the atlas shape")
+        self._require_atlas(atlas_out, values=values)
         _check(self.lib.snerg_requantize_atlas(self.handle, _ptr(values), _ptr(atlas_out), _stream(self.device)),
                "snerg_requantize_atlas")
+
+    def adam_requantize_atlas(self, values: torch.Tensor, m: torch.Tensor, v: torch.Tensor, grad: torch.Tensor,
+                              step: int, lr: float = 3e-4, betas=(0.9, 0.999), eps: float = 1e-8,
+                              atlas_out: torch.Tensor | None = None):
+        """adam_step(values, m, v, grad, ...) and requantize_atlas(values, atlas_out) in one pass
+        over the values (snerg_adam_requantize_atlas)."""
+        self._require_atlas(atlas_out, values=values, m=m, v=v, grad=grad)
+        _check(self.lib.snerg_adam_requantize_atlas(self.handle, _ptr(values), _ptr(m), _ptr(v), _ptr(grad), float(lr),
+                                                    float(betas[0]), float(betas[1]), float(eps), int(step),
+                                                    _ptr(atlas_out), _stream(self.device)),
+               "snerg_adam_requantize_atlas")
 
     def _opts(self, n_pix, aux, counts, trace_cap, persistent, tile, ctas_per_sm):
         out = {}
@@ -572,8 +591,8 @@ class FineTuner:
         self.steps += 1
         adam_step(self.mlp, self.m, self.v, self.grad, self.steps, self.lr, self.betas, self.eps)
         if self.shadow is not None:
-            adam_step(self.shadow, self.ma, self.va, self.grad_atlas, self.steps, self.atlas_lr, self.betas, self.eps)
-            self.r.requantize_atlas(self.shadow, self.codes)
+            self.r.adam_requantize_atlas(self.shadow, self.ma, self.va, self.grad_atlas, self.steps, self.atlas_lr,
+                                         self.betas, self.eps, self.codes)
         return self.loss
 
 

@@ -24,7 +24,7 @@ def test_separable_bake_matches_oracle(N, B, n_blob, std):
 def test_alpha_codes_of_separable_blocks():
     f = synth.analytic_field(5, n_blob=9, std=(0.05, 0.1), peak=(20.0, 80.0))
     field = renderer.bake_field(f["blobs"], f["colors"], f["jitter"], TAU)
-    ind, atl = renderer.bake(96, 32, BMIN, EXTENT, 100.0, field, DEV, alpha_codes=True)
+    ind, atl = renderer.bake(96, 32, BMIN, EXTENT, 100.0, field, DEV, flags=renderer.FLAG_ALPHA_ATLAS)
     ind, atl = ind.cpu().numpy(), atl.cpu().numpy()
     blocks = np.flatnonzero((ind >= 0).ravel())
     _, content, raw = oracle.bake_blocks(96, 32, BMIN, EXTENT, 100.0, f["blobs"], f["colors"], f["jitter"], blocks,
