@@ -140,7 +140,7 @@ __device__ __forceinline__ void image_pixel(const DevScene& s, const snerg_camer
         march<false, false, PS>(s, r, st, nullptr, 0, nullptr, nullptr, 0, DBG ? &k_first : nullptr, pwp, sW);
     record_status(s, st);
     float c[3], aux[kAuxCh];
-    finish_ray(s, sW, nullptr, r, st, c, aux, pwp);
+    finish_ray(s, sW, r, st, c, aux, pwp);
     rgb[pix * 3 + 0] = c[0];
     rgb[pix * 3 + 1] = c[1];
     rgb[pix * 3 + 2] = c[2];
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(128, MINB) render_rays_kernel(const DevScene s
         march<false, false, false, true>(s, r, st, nullptr, 0, nullptr, nullptr, 0, DBG ? &k_first : nullptr);
     record_status(s, st);
     float c[3], aux[kAuxCh];
-    finish_ray(s, sW, nullptr, r, st, c, aux, PW ? &pw : nullptr);
+    finish_ray(s, sW, r, st, c, aux, PW ? &pw : nullptr);
     rgb[i * 3 + 0] = c[0];
     rgb[i * 3 + 1] = c[1];
     rgb[i * 3 + 2] = c[2];
@@ -260,7 +260,7 @@ __device__ __forceinline__ void persistent_pixel(const DevScene& s, const snerg_
     march<false, false>(s, r, st, nullptr, 0, nullptr, nullptr);
     record_status(s, st);
     float c[3], aux[kAuxCh];
-    finish_ray(s, sW, nullptr, r, st, c, aux, PW ? &pw : nullptr);
+    finish_ray(s, sW, r, st, c, aux, PW ? &pw : nullptr);
     out[0] = c[0];
     out[1] = c[1];
     out[2] = c[2];

@@ -216,7 +216,7 @@ __device__ __forceinline__ bool in_box(const Ray& r, float k, const Box& bx) {
     return true;
 }
 
-// The margin (in samples) of box_exit's unconfirmed estimate for ray r in a grid of N
+// The margin (in samples) of march_exit's unconfirmed estimate for ray r in a grid of N
 // voxels per axis, with t_m = max(t1, 1) bounding every lattice t the march compares:
 //  - the estimate K = fl(fl(te - t0) - 0.5) with te = fl(fl(face - o) * inv_d), inv_d
 //    within 2 ulp of 1/d: |K - K*| <= t_m (2^-22 + 2^-23 + 2^-24 + 2 * 2^-24) < t_m 2^-20;
@@ -236,21 +236,10 @@ __device__ __forceinline__ float exit_margin(const Ray& r, float fN) {
     return 4.0f * (tm * (1.0f / 1048576.0f) + lat + tm * (1.0f / 16777216.0f));
 }
 
-// First lattice index k' > k with in_box(k') false, given in_box(k). Each axis's
-// nearest voxel is a monotone function of k (every step of the lattice arithmetic is a
-// rounded monotone operation), so the samples inside a box form one contiguous run:
-// estimate its end from the ray/box exit distance, then confirm or correct it with an
-// exact search on the lattice itself.
-//
-// The estimate needs no confirmation when the real crossing index is at least `margin`
-// from every integer, margin bounding (a) the error of the estimate K (rounding of the
-// face distances, the approximate reciprocal, the two subtractions) and (b) how far in k
-// the binary32 lattice can place a sample across a face or past t1 from where exact
-// arithmetic would (see exit_margin). Then every sample before ceil(K) is inside on every
-// face still ahead (their crossings are no earlier than K's) and the sample at ceil(K)
-// is outside. A margin of 1 or more disables this.
-//
-// box_search: the exact search from an estimate n.
+// First lattice index k' > k with in_box(k') false, given in_box(k), by an exact search on the
+// lattice itself from an estimate n: each axis's nearest voxel is a monotone function of k
+// (every step of the lattice arithmetic is a rounded monotone operation), so the samples
+// inside a box form one contiguous run.
 __device__ __forceinline__ float box_search(const Ray& r, float kmax, float k, float n, const Box& bx) {
     // estimate clamped to [k + 1, kmax] (fminf/fmaxf also map a NaN estimate into range)
     const float ke = fmaxf(fminf(n, kmax), k + 1.0f);
@@ -277,36 +266,27 @@ __device__ __forceinline__ float box_search(const Ray& r, float kmax, float k, f
     return hi_k;
 }
 
-__device__ __forceinline__ float box_exit(const Ray& r, const float inv_d[3], float kmax, float k, const Box& bx,
-                                          float margin) {
-    float te = r.t1;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        if (r.d[i] > 0.0f) te = fminf(te, (bx.hi[i] - r.o[i]) * inv_d[i]);
-        else if (r.d[i] < 0.0f) te = fminf(te, (bx.lo[i] - r.o[i]) * inv_d[i]);
-    }
-    const float K = te - r.t0 - 0.5f;
-    const float n = ceil_small(K);        // |K| <= t1 - t0 + 1 (or NaN, kept)
-    // fr in [0, 1). n - K is exact for K >= 1/2 (Sterbenz) and for K <= 0; for K in
-    // (0, 1/2), n = 1 and 1 - K rounds by at most 2^-25, far inside the margin (at least
-    // 4 * 2^-20, four times the bound on the estimate's own error), so the test below
-    // decides the same way.
-    const float fr = n - K;
-    if (n >= k + 1.0f && n < kmax && fr >= margin && fr < 1.0f - margin) return n;
-    return box_search(r, kmax, k, n, bx);
-}
-
-// box_exit for the march's own boxes, from sample kh (= k + 1/2) of the voxel j: the blocks
-// within D - 1 (D >= 1) of j's block towards the ray's octant, so that on every axis only
-// the face ahead can be crossed. The estimate is box_exit's with two differences. A face on
-// or beyond the grid's border is not clipped to infinity: its crossing is at or behind t1 up
-// to the rounding that the margin covers, and t1 is in the minimum. And the margin test is
-// taken as |fr - 1/2| < half = 1/2 - margin. Lanes that stand in an empty box and in an
-// occupied block (D = 1) share this code. Returns k' + 1/2.
+// The march's own boxes: for sample kh (= k + 1/2) of the voxel j, the blocks within D - 1
+// (D >= 1) of j's block towards the ray's octant, so that on every axis only the face ahead can
+// be crossed. Returns k' + 1/2, k' the first sample outside the box.
 //
-// A block entry was about 100 instructions, issued once for a warp's empty lanes and again
-// for its occupied ones (the march is bound by issue in full launches, by the chain of
-// dependent steps in small ones); one shared copy with a face instead of a box per axis:
+// The run's end is estimated from the ray/box exit distance. The estimate needs no
+// confirmation when the real crossing index is at least `margin` from every integer, margin
+// bounding (a) the error of the estimate K (rounding of the face distances, the approximate
+// reciprocal, the two subtractions) and (b) how far in k the binary32 lattice can place a
+// sample across a face or past t1 from where exact arithmetic would (see exit_margin). Then
+// every sample before ceil(K) is inside on every face still ahead (their crossings are no
+// earlier than K's) and the sample at ceil(K) is outside. n - K = ceil(K) - K is exact for
+// K >= 1/2 (Sterbenz) and for K <= 0; for K in (0, 1/2), 1 - K rounds by at most 2^-25, far
+// inside the margin (at least 4 * 2^-20, four times the bound on the estimate's own error). The
+// test is |n - K - 1/2| < half = 1/2 - margin; a margin of 1/2 or more disables it. A face on
+// or beyond the grid's border bounds nothing (the nearest voxel is clamped there), yet is not
+// left out: its crossing is at or behind t1 up to rounding of the same kind, and t1 is in the
+// minimum. Otherwise the exact search decides.
+//
+// A block entry was about 100 instructions, issued once for a warp's lanes in empty boxes and
+// again for those in stored blocks (the march is bound by issue in full launches, by the chain
+// of dependent steps in small ones); one shared copy with a face instead of a box per axis:
 // 64 mixed views of a 1024^3 grid 6.01 -> 5.64 ms, one 800^2 view 190 -> 183 us, 262,147
 // scattered rays 283 -> 255 us.
 __device__ __forceinline__ float march_exit(const DevScene& s, const Ray& r, const float inv_d[3], float kh,
@@ -672,14 +652,12 @@ __device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchStat
 // view-dependence MLP (Eq. 7): x = [C_d, V, d, sin/cos(2^l d), l = 0..3] -> 16 ReLU ->
 // 16 ReLU -> 3 -> sigmoid, built to stay small in registers and code:
 // weights sit in shared memory with W1 and W2 transposed (rows of 16 outputs, read with
-// uniform 128-bit loads), the 34-float input row of each thread is staged in shared
-// memory and streamed through a rolled loop, and the direction encoding takes one
-// sincosf per axis and the double-angle identities for the higher octaves.
+// uniform 128-bit loads), the inputs are consumed from registers as they are made (the adjoint
+// keeps them in a row of shared memory), and the direction encoding takes one sincosf per
+// axis and the double-angle identities for the higher octaves.
 // Layout (floats): W1^T[34][16] | b1[16] | W2^T[16][16] | b2[16] | W3[3][16] | b3[3]
 // (the offsets kOff* are those of the flat layout; only W1 and W2 are transposed).
 // ---------------------------------------------------------------------------------
-constexpr int kXStride = 35;   // per-thread input row stride in shared memory (odd: no bank conflicts)
-
 __device__ __forceinline__ void load_mlp_smem_t(float* sW, const float* mlp) {
     const int nt = blockDim.x * blockDim.y;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
@@ -741,29 +719,7 @@ __device__ __forceinline__ void stage_mlp_input(float* xrow, const float cd[3], 
     }
 }
 
-__device__ __forceinline__ void mlp_residual(const float* sW, const float* xrow, float res[3]) {
-    float h[16];
-    load16(h, sW + kOffB1);
-#pragma unroll 2
-    for (int i = 0; i < kMlpIn; ++i) fma16(h, sW + kOffW1 + i * kMlpH, xrow[i]);
-#pragma unroll
-    for (int o = 0; o < 16; ++o) h[o] = fmaxf(h[o], 0.0f);
-    float h2[16];
-    load16(h2, sW + kOffB2);
-#pragma unroll
-    for (int i = 0; i < kMlpH; ++i) fma16(h2, sW + kOffW2 + i * kMlpH, h[i]);
-#pragma unroll
-    for (int o = 0; o < kMlpOut; ++o) {
-        float w3[16];
-        load16(w3, sW + kOffW3 + o * kMlpH);
-        float acc = sW[kOffB3 + o];
-#pragma unroll
-        for (int i = 0; i < kMlpH; ++i) acc = fmaf(w3[i], fmaxf(h2[i], 0.0f), acc);
-        res[o] = 1.0f / (1.0f + expf(-acc));
-    }
-}
-
-// The same MLP with its 34 inputs taken from registers: C_d, V and d directly, the
+// The MLP with its 34 inputs taken from registers: C_d, V and d directly, the
 // direction encoding generated in order (one sincosf per axis, double-angle identities
 // for the higher octaves) and consumed as produced. Needs no shared-memory row.
 __device__ __forceinline__ void mlp_residual_regs(const float* sW, const float cd[3], const float v[4],
@@ -870,10 +826,8 @@ __device__ __forceinline__ void per_sample_residual(const MlpWeights* pw, const 
 }
 
 // Finish one ray: colour = C_d + residual + T bg (residual only if something was
-// composited). sW: weights in the transposed layout of load_mlp_smem_t; xrow: this
-// thread's kXStride-float row of shared memory to stage the MLP input in, or nullptr to
-// evaluate the MLP from registers.
-__device__ __forceinline__ void finish_ray(const DevScene& s, const float* sW, float* xrow, const Ray& r,
+// composited). sW: weights in the transposed layout of load_mlp_smem_t, if pw is null.
+__device__ __forceinline__ void finish_ray(const DevScene& s, const float* sW, const Ray& r,
                                            const MarchState& st, float rgb[3], float aux[kAuxCh],
                                            const MlpWeights* pw = nullptr) {
     const float inv255 = 1.0f / 255.0f;
@@ -905,14 +859,8 @@ __device__ __forceinline__ void finish_ray(const DevScene& s, const float* sW, f
         for (int c = 0; c < 3; ++c) res[c] = cd[c];
     } else if (st.active > 0) {
         float m[3];
-        if (pw) {
-            mlp_residual_param(*pw, cd, v, r.d, m);
-        } else if (xrow) {
-            stage_mlp_input(xrow, cd, v, r.d);
-            mlp_residual(sW, xrow, m);
-        } else {
-            mlp_residual_regs(sW, cd, v, r.d, m);
-        }
+        if (pw) mlp_residual_param(*pw, cd, v, r.d, m);
+        else mlp_residual_regs(sW, cd, v, r.d, m);
 #pragma unroll
         for (int c = 0; c < 3; ++c) res[c] = cd[c] + m[c];
     }
@@ -980,10 +928,8 @@ cudaError_t launch_validate(const int32_t* ind, int64_t n_ind, int64_t nb, int32
 // that finds *err set does nothing
 cudaError_t launch_prep_blocks(const int32_t* ind, const int32_t* blk_of_slot, const int32_t* err, const uint8_t* atlas,
                                int64_t nb, int G, int lgB, uint2* patlas, uint8_t* vskip, cudaStream_t st);
-// Chebyshev distance maps over the G^3 indirection grid, distances capped at `cap`: the
-// two-sided one, and the render's (per octant of the ray direction, inside its cone).
-cudaError_t launch_block_distance(const int32_t* ind, int G, int cap, uint8_t* tmp0, uint8_t* tmp1,
-                                  uint8_t* bdist, cudaStream_t st);
+// Chebyshev distance maps over the G^3 indirection grid, distances capped at `cap`, per
+// octant of the ray direction inside its cone.
 cudaError_t launch_block_distance_octants(const int32_t* ind, int G, int cap, uint8_t* tmp0, uint8_t* tmp1,
                                           uint8_t* bdist, int32_t* ind_oct, int64_t* launches, cudaStream_t st);
 

@@ -113,12 +113,12 @@ __global__ void __launch_bounds__(256) requantize_kernel(const int32_t* __restri
 // over min, so the passes compose). The scan walks outwards from p and stops once the
 // offset reaches the best value found, so its cost is the distance itself.
 //
-// `side` restricts q to one half-line (bit 0: q <= p, bit 1: q >= p; 3 = both). With
-// one side per axis the result is the distance to the nearest occupied cell in the
+// `side` restricts q to one half-line (bit 0: q <= p, bit 1: q >= p). With one side per
+// axis the result is the distance to the nearest occupied cell in the
 // octant cone {q : q_i - p_i of the chosen sign}: the cone is a product of half-lines,
 // so the one-sided passes compose the same way.
 // ---------------------------------------------------------------------------------
-constexpr int kSideLow = 1, kSideHigh = 2, kSideBoth = 3;
+constexpr int kSideLow = 1, kSideHigh = 2;
 
 __device__ __forceinline__ int dt_line(const uint8_t* __restrict__ in, int64_t base, int64_t stride, int pos, int n,
                                        int cap, int side) {
@@ -505,13 +505,6 @@ static void block_distance(const int32_t* ind, int G, int cap, uint8_t* tmp0, ui
     dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp0, tmp1, G, 1, 0, cap, side[0]);
     dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp1, tmp0, G, 1, 1, cap, side[1]);
     dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp0, bdist, G, 1, 2, cap, side[2]);
-}
-
-cudaError_t launch_block_distance(const int32_t* ind, int G, int cap, uint8_t* tmp0, uint8_t* tmp1,
-                                  uint8_t* bdist, cudaStream_t st) {
-    const int both[3] = {kSideBoth, kSideBoth, kSideBoth};
-    block_distance(ind, G, cap, tmp0, tmp1, bdist, both, st);
-    return cudaGetLastError();
 }
 
 // For each octant o, ind_oct[o] = the indirection grid `ind` with every empty entry replaced by
