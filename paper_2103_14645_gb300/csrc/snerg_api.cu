@@ -218,6 +218,7 @@ extern "C" snerg_status snerg_create(const snerg_scene_desc* desc, const int32_t
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (h->num_sms < 1) h->num_sms = 1;
+    s.sms = h->num_sms;
     *out = h;
     return SNERG_OK;
 }
@@ -481,8 +482,10 @@ extern "C" snerg_status snerg_render(snerg_handle h, const snerg_camera* cams, i
         sa.cap = kSchedMaxTiles;
         sa.nt = tiles;
         sa.tiles_x = (cams[0].W + 15) / 16;
-        // sparse slots only with a previous frame to choose the slow tiles from
-        sa.smax = use ? std::min(kSchedMaxSparse, std::max(1, tiles / 8)) : 0;
+        // a small image's tiles take several CTAs each; sparse slots only beyond that, and with a
+        // previous frame to choose the slow tiles from
+        sa.parts = std::min(32 / image_lanes(h->ds, (int64_t)cams[0].W * cams[0].H), 8);
+        sa.smax = use && sa.parts < 4 ? std::min(kSchedMaxSparse, std::max(1, tiles / 8)) : 0;
         cudaError_t e = cudaMemsetAsync(wr, 0, kSchedCountBytes, st);
         if (e == cudaSuccess) e = launch_render_image(h->ds, cams[0], d_mlp, pw, d_rgb, dbg, st, 0, cams[0].H, &sa);
         if (e != cudaSuccess) return SNERG_E_CUDA;
@@ -591,7 +594,7 @@ extern "C" snerg_status snerg_render_rays(snerg_handle h, const snerg_camera* ca
     if (n == 0) { delete t; return SNERG_OK; }
     if (!d_pix || !d_rgb || (!d_mlp && !h->has_w)) { delete t; return SNERG_E_INVAL; }
     cudaError_t e = launch_render_rays(h->ds, *t, n_cams, d_pix, n, d_mlp, d_mlp ? nullptr : &h->host_w, d_rgb,
-                                       make_dbg(opts), h->num_sms, (cudaStream_t)stream);
+                                       make_dbg(opts), (cudaStream_t)stream);
     delete t;
     if (e != cudaSuccess) return SNERG_E_CUDA;
     h->launches++;

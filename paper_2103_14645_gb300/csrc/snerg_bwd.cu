@@ -25,7 +25,7 @@ constexpr int kRowX = 0, kRowH1 = 34, kRowH2 = 50, kRowG1 = 66, kRowG2 = 82, kRo
 constexpr int kWFloats = 884;      // transposed weights (883) rounded up to a 16-byte multiple
 constexpr int kMaxDevices = 64;     // devices whose shared-memory opt-in is remembered
 
-size_t backward_smem_bytes() { return (size_t)(kWFloats + kBwdThreads * kRow) * sizeof(float); }
+size_t backward_smem_bytes(int lanes) { return (size_t)(kWFloats + kBwdThreads / 32 * lanes * kRow) * sizeof(float); }
 
 // A recorded sample's lattice position, block origin (minus one), block slot and weight.
 struct RecSample {
@@ -187,7 +187,7 @@ __device__ __forceinline__ void mlp_forward_backward(const float* sW, float* row
 // register tiles (8 shared-memory loads per ray for 16 products, against 32 for one
 // product at a time): W1 (16 x 34) in 36 tiles, W2 (16 x 16) in 16, W3 (3 x 16) in 4;
 // threads 56..90 sum one bias each. Every sum runs over the rays in the same order.
-__device__ __forceinline__ void dphi_sums(const float* rows, float* grad_mlp) {
+__device__ __forceinline__ void dphi_sums(const float* rows, int n_rows, float* grad_mlp) {
     const int t = threadIdx.x;
     if (t < 56) {
         int a0, b0, out, lda, na, nb;    // rows of the two factors, output offset and stride
@@ -210,7 +210,7 @@ __device__ __forceinline__ void dphi_sums(const float* rows, float* grad_mlp) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) acc[u][v] = 0.0f;
 #pragma unroll 2
-        for (int r = 0; r < kBwdThreads; ++r) {
+        for (int r = 0; r < n_rows; ++r) {
             const float* row = rows + r * kRow;
             float a[4], b[4];
 #pragma unroll
@@ -235,7 +235,7 @@ __device__ __forceinline__ void dphi_sums(const float* rows, float* grad_mlp) {
         else { a = kRowGZ + (j - 2 * kMlpH); p = kOffB3 + (j - 2 * kMlpH); }
         float acc = 0.0f;
 #pragma unroll 4
-        for (int r = 0; r < kBwdThreads; ++r) acc += rows[r * kRow + a];
+        for (int r = 0; r < n_rows; ++r) acc += rows[r * kRow + a];
         if (acc != 0.0f) atomicAdd(grad_mlp + p, acc);
     }
 }
@@ -254,15 +254,17 @@ __global__ void __launch_bounds__(kBwdThreads, 4) backward_rays_kernel(
     int64_t n, const float* __restrict__ mlp, const float* __restrict__ grad_rgb,
     const float* __restrict__ fwd_aux, const int32_t* __restrict__ fwd_counts, const float* __restrict__ target,
     float* __restrict__ rgb_out, float* __restrict__ loss, float* __restrict__ grad_atlas,
-    float* __restrict__ grad_mlp) {
+    float* __restrict__ grad_mlp, int lanes) {
     extern __shared__ __align__(16) float smem[];
     __shared__ float s_loss[kBwdThreads / 32];
     float* sW = smem;
     float* rows = smem + kWFloats;
     load_mlp_smem_t(sW, mlp);
     __syncthreads();
-    float* row = rows + threadIdx.x * kRow;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool on = lane < lanes;
+    float* row = rows + (warp * lanes + (on ? lane : 0)) * kRow;
+    const int64_t i = on ? ((int64_t)blockIdx.x * (kBwdThreads / 32) + warp) * lanes + lane : n;
 
     Ray r;
     r.hit = false;
@@ -350,7 +352,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) backward_rays_kernel(
         } else {
             mlp_forward_backward(sW, row, g, gx);
         }
-    } else {
+    } else if (on) {
         for (int k = 0; k < kRow; ++k) row[k] = 0.0f;   // contributes nothing to the sums below
         if (TRAIN && i < n) {
             // nothing composited: C = T bg (T = 1 for a ray that composited nothing)
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) backward_rays_kernel(
     }
     // dL/dPhi: sums over the CTA's rays of outer products (one global atomic per parameter
     // per CTA): W1 <- g1 (x) x, W2 <- g2 (x) h1, W3 <- gz (x) h2, biases <- g.
-    if (grad_mlp) dphi_sums(rows, grad_mlp);
+    if (grad_mlp) dphi_sums(rows, kBwdThreads / 32 * lanes, grad_mlp);
 }
 
 template <bool TRAIN, bool STATE>
@@ -408,7 +410,10 @@ static cudaError_t backward_launch(const DevScene& s, const CamTable& cams, int3
                                    const int32_t* fwd_counts, const float* target, float* rgb_out, float* loss,
                                    float* grad_atlas, float* grad_mlp, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    const size_t smem = backward_smem_bytes();
+    // rays spread over one wave of 4 CTAs per SM: a step of 4,096 rays on a 1024^3 grid takes
+    // 132 us with 32 rays per warp and 89 with 2, 16,384: 140 and 110 with 8, 65,536: 155 with 32
+    const int lanes = lanes_per_warp(n, (int64_t)s.sms * 4 * (kBwdThreads / 32));
+    const size_t smem = backward_smem_bytes(lanes);
     // the opt-in for > 48 KB of dynamic shared memory, once per device
     static std::atomic<bool> attr_set[kMaxDevices];
     int dev = 0;
@@ -417,14 +422,15 @@ static cudaError_t backward_launch(const DevScene& s, const CamTable& cams, int3
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!attr_set[dev].load()) {
         e = cudaFuncSetAttribute(backward_rays_kernel<TRAIN, STATE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
+                                 (int)backward_smem_bytes(32));
         if (e != cudaSuccess) return e;
         attr_set[dev].store(true);
     }
-    const unsigned grid = (unsigned)((n + kBwdThreads - 1) / kBwdThreads);
+    const int rays = kBwdThreads / 32 * lanes;          // per CTA
+    const unsigned grid = (unsigned)((n + rays - 1) / rays);
     backward_rays_kernel<TRAIN, STATE><<<grid, kBwdThreads, smem, st>>>(s, cams, n_cams, pix, n, mlp, grad_rgb,
                                                                         fwd_aux, fwd_counts, target, rgb_out, loss,
-                                                                        grad_atlas, grad_mlp);
+                                                                        grad_atlas, grad_mlp, lanes);
     return cudaGetLastError();
 }
 

@@ -14,11 +14,14 @@ namespace snerg {
 // neighbouring voxels together. A CTA holds NW warps (1: 8x4, 2: 16x4, 4: 16x8 pixels);
 // small CTAs free their SM slot as soon as their own packets are done, which matters
 // because packets on the object take several times longer than background packets.
-template <int NW>
+//
+// L: rays per warp (the other lanes idle), see lanes_per_warp.
+template <int NW, int L = 32>
 struct ImageTile {
     static constexpr int WX = NW >= 2 ? 2 : 1;      // warps across
     static constexpr int WY = NW >= 4 ? 2 : 1;      // warps down
-    static constexpr int TW = 8 * WX, TH = 4 * WY;  // CTA tile in pixels
+    static constexpr int PX = L == 32 ? 8 : (L >= 8 ? 4 : (L >= 2 ? 2 : 1)), PY = L / PX;   // a warp's pixels
+    static constexpr int TW = PX * WX, TH = PY * WY;  // CTA tile in pixels
 };
 
 // SCHED: the launch's CTAs take the image's tiles in the order of the previous frame's
@@ -33,9 +36,13 @@ struct ImageTile {
 // kSchedSparseGain: about its dense cost, so that it stays sparse while it stays slow) and
 // the launch's start and end. The grid is nt + 4 smax CTAs: 4 smax sparse slots (S <= smax
 // used), then nt dense slots for the tiles S .. nt - 1 of the order (the last S idle).
+// A small image (lanes_per_warp) has `parts` CTAs per dense slot, each a band of the tile's rows
+// with 32 / parts rays per warp, and no sparse slots where that is as few; the first band's
+// duration stands for the tile's.
 struct SchedSlot {
     int tile;       // -1: idle
     int quarter;    // -1: dense
+    int part;       // dense: band of the tile's rows
 };
 
 __device__ __forceinline__ SchedSlot sched_map(const SchedArgs& sch, int c, unsigned long long* t0) {
@@ -75,11 +82,11 @@ __device__ __forceinline__ SchedSlot sched_map(const SchedArgs& sch, int c, unsi
                 q = c & 3;
             }
         } else {
-            item = S + (c - 4 * sch.smax);
+            item = S + (c - 4 * sch.smax) / sch.parts;
             if (item >= sch.nt) item = -1;
         }
         if (lane == 0) {
-            s_slot = SchedSlot{use ? -1 : item, q};
+            s_slot = SchedSlot{use ? -1 : item, q, q < 0 ? (c - 4 * sch.smax) % sch.parts : 0};
             if (c == 0) {           // what this launch did, for snerg_schedule_stats
                 sch.wr_count[kSchedHdrInfo] = S + 1;
                 sch.wr_count[kSchedHdrInfo + 1] = use ? 1 : 0;
@@ -103,7 +110,7 @@ __device__ __forceinline__ void sched_record(const SchedArgs& sch, const SchedSl
         atomicMax(tw, ~*t0);
         atomicMax(tw + 1, t1);
         float ns = (float)(t1 - *t0);
-        bool rec = sl.tile >= 0 && sl.quarter < 0;
+        bool rec = sl.tile >= 0 && sl.quarter < 0 && sl.part == 0;
         if (sl.tile >= 0 && sl.quarter >= 0) {
             // sparse: the last of the tile's four quarters records the slowest one
             const int j = (int)(blockIdx.x >> 2);
@@ -156,7 +163,7 @@ __device__ __forceinline__ void image_pixel(const DevScene& s, const snerg_camer
     }
 }
 
-template <bool DBG, bool PW, int NW, bool PS, bool SCHED = false>
+template <bool DBG, bool PW, int NW, bool PS, bool SCHED = false, int L = 32>
 __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const DevScene s, const snerg_camera cam,
                                                                         const float* __restrict__ mlp,
                                                                         const __grid_constant__ MlpWeights pw,
@@ -168,7 +175,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const De
         __syncthreads();
     }
     const MlpWeights* pwp = PW ? &pw : nullptr;
-    using T = ImageTile<NW>;
+    using T = ImageTile<NW, L>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if constexpr (SCHED) {
         static_assert(NW == 4, "the sparse mapping assumes 16x8 tiles of four 8x4 warps");
@@ -178,7 +185,12 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const De
             const int tx = sl.tile % sch.tiles_x, ty = sl.tile / sch.tiles_x;
             int px, py;
             bool on = true;
-            if (sl.quarter < 0) {
+            if (sl.quarter < 0 && sch.parts > 1) {
+                const int lanes = 32 / sch.parts, idx = warp * lanes + lane;     // 16 x (8 / parts) pixels
+                on = lane < lanes;
+                px = tx * T::TW + (idx & 15);
+                py = ty * T::TH + sl.part * (T::TH / sch.parts) + (idx >> 4);
+            } else if (sl.quarter < 0) {
                 px = tx * T::TW + (warp % T::WX) * 8 + (lane & 7);
                 py = ty * T::TH + (warp / T::WX) * 4 + (lane >> 3);
             } else {
@@ -191,27 +203,30 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const De
         }
         sched_record(sch, sl, &s_t0);
     } else {
-        const int px = blockIdx.x * T::TW + (warp % T::WX) * 8 + (lane & 7);
-        const int py = row0 + blockIdx.y * T::TH + (warp / T::WX) * 4 + (lane >> 3);
-        if (px >= cam.W || py >= row1) return;
+        const int px = blockIdx.x * T::TW + (warp % T::WX) * T::PX + lane % T::PX;
+        const int py = row0 + blockIdx.y * T::TH + (warp / T::WX) * T::PY + lane / T::PX;
+        if (lane >= L || px >= cam.W || py >= row1) return;
         image_pixel<DBG, PS>(s, cam, sW, pwp, rgb, dbg, px, py);
     }
 }
 
-// MINB: resident CTAs per SM the build is limited to (8: 64 registers; 4: up to 128)
+// MINB: resident CTAs per SM the build is limited to (8: 64 registers; 4: up to 128);
+// lanes: rays per warp (the other lanes idle)
 template <bool DBG, bool PW, int MINB>
 __global__ void __launch_bounds__(128, MINB) render_rays_kernel(const DevScene s, const __grid_constant__ CamTable cams,
                                                                 int32_t n_cams, const int32_t* __restrict__ pix,
                                                                 int64_t n, const float* __restrict__ mlp,
                                                                 const __grid_constant__ MlpWeights pw,
-                                                                float* __restrict__ rgb, const DebugOut dbg) {
+                                                                float* __restrict__ rgb, const DebugOut dbg,
+                                                                int lanes) {
     __shared__ __align__(16) float sW[PW ? 4 : kNParam + 1];
     if (!PW) {
         load_mlp_smem_t(sW, mlp);
         __syncthreads();
     }
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) * lanes + lane;
+    if (lane >= lanes || i >= n) return;
     const int ci = __ldg(pix + 3 * i), px = __ldg(pix + 3 * i + 1), py = __ldg(pix + 3 * i + 2);
     Ray r;
     if (ci >= 0 && ci < n_cams && px >= 0 && py >= 0 && px < cams.c[ci].W && py < cams.c[ci].H) {
@@ -319,6 +334,26 @@ static const MlpWeights& no_weights() {
     return z;
 }
 
+// Up to three waves of warps: 40,000 pixels of a 1024^3 grid take 202 us with 32 rays per warp,
+// 134 with 8 and 118 with 4 (2.1 waves); 160,000 take 201, 171 with 16 (2.1) and 164 with 8 (4.1),
+// but of a 512^3 grid 108, 102 and 111; from 470,000 on 32 is the best or within 5 % of it.
+int image_lanes(const DevScene& s, int64_t n) { return lanes_per_warp(n, (int64_t)s.sms * 8 * kImageWarps * 3); }
+
+template <int L>
+static void image_sparse(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
+                         float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1) {
+    using T = ImageTile<kImageWarps, L>;
+    const dim3 grid((cam.W + T::TW - 1) / T::TW, (row1 - row0 + T::TH - 1) / T::TH);
+    const SchedArgs none{nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 1};
+    const MlpWeights& w = pw ? *pw : no_weights();
+    if (pw)
+        render_image_kernel<false, true, kImageWarps, false, false, L><<<grid, 32 * kImageWarps, 0, st>>>(
+            s, cam, mlp, w, rgb, dbg, row0, row1, none);
+    else
+        render_image_kernel<false, false, kImageWarps, false, false, L><<<grid, 32 * kImageWarps, 0, st>>>(
+            s, cam, mlp, w, rgb, dbg, row0, row1, none);
+}
+
 template <bool PS>
 static void image_launch(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
                          float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1, const SchedArgs* sch) {
@@ -327,9 +362,18 @@ static void image_launch(const DevScene& s, const snerg_camera& cam, const float
     const int nt = 32 * kImageWarps;
     const bool d = dbg.aux || dbg.counts || dbg.trace;
     const MlpWeights& w = pw ? *pw : no_weights();
-    const SchedArgs none{nullptr, nullptr, nullptr, nullptr, 0};
+    const SchedArgs none{nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 1};
+    if (!PS && !d && !sch) {
+        switch (image_lanes(s, (int64_t)cam.W * (row1 - row0))) {
+            case 16: return image_sparse<16>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
+            case 8: return image_sparse<8>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
+            case 4: return image_sparse<4>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
+            case 2: return image_sparse<2>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
+            case 1: return image_sparse<1>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
+        }
+    }
     if (!PS && !d && sch) {
-        const dim3 g1((unsigned)(sch->nt + 4 * sch->smax));   // 4 smax sparse slots, then nt dense ones
+        const dim3 g1((unsigned)(sch->nt * sch->parts + 4 * sch->smax));   // 4 smax sparse slots, then nt dense ones
         if (pw) render_image_kernel<false, true, kImageWarps, false, true><<<g1, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg,
                                                                                             row0, row1, *sch);
         else render_image_kernel<false, false, kImageWarps, false, true><<<g1, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg,
@@ -359,28 +403,35 @@ cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, cons
 
 template <int MINB>
 static void rays_launch(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
-                        const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, cudaStream_t st) {
-    const unsigned grid = (unsigned)((n + 127) / 128);
+                        const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, int lanes,
+                        cudaStream_t st) {
+    const unsigned grid = (unsigned)((n + 4 * lanes - 1) / (4 * lanes));
     const bool d = dbg.aux || dbg.counts || dbg.trace;
     const MlpWeights& w = pw ? *pw : no_weights();
     if (pw) {
-        if (d) render_rays_kernel<true, true, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg);
-        else render_rays_kernel<false, true, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg);
+        if (d) render_rays_kernel<true, true, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg, lanes);
+        else render_rays_kernel<false, true, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg, lanes);
     } else {
-        if (d) render_rays_kernel<true, false, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg);
-        else render_rays_kernel<false, false, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg);
+        if (d) render_rays_kernel<true, false, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg, lanes);
+        else render_rays_kernel<false, false, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg, lanes);
     }
 }
 
-// A ray list that fits one wave of 4 CTAs per SM runs the build limited to 4 (the march
-// keeps its state in registers, and a single wave gains nothing from the 8-CTA
-// occupancy); longer lists keep 8 CTAs per SM to hide the march's latencies.
+// A list is spread over the warps of one wave of 8 CTAs per SM: scattered rays have less in
+// common than an image's, and a second wave costs as much as the first (4,096 rays of a 1024^3
+// grid 122 us with 32 rays per warp, 70 with 1; 16,384: 131 and, with 4, 102; 65,536: 143 with
+// 32, 145 with 16, 150 with 8; 262,144: 274, 324 with 16); with debug outputs, whose 8-CTA build
+// spills, over one wave of 4. If 4 CTAs per SM hold it, it
+// runs the build limited to 4 (the march keeps its state in registers, and a single wave gains
+// nothing from the 8-CTA occupancy); longer lists keep 8 CTAs per SM to hide the march's latencies.
 cudaError_t launch_render_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
                                int64_t n, const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg,
-                               int num_sms, cudaStream_t st) {
+                               cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    if ((n + 127) / 128 <= 4 * (int64_t)num_sms) rays_launch<4>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, st);
-    else rays_launch<8>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, st);
+    const bool d = dbg.aux || dbg.counts || dbg.trace;
+    const int lanes = lanes_per_warp(n, (int64_t)s.sms * (d ? 4 : 8) * 4);
+    if (n <= (int64_t)s.sms * 4 * 4 * lanes) rays_launch<4>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, lanes, st);
+    else rays_launch<8>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, lanes, st);
     return cudaGetLastError();
 }
 

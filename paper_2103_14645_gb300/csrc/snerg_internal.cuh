@@ -83,7 +83,19 @@ struct DevScene {
     float bg[3];
     int32_t kmax;     // lattice index cap (4N + 16)
     int32_t flags;    // SNERG_FLAG_*
+    int32_t sms;      // SMs of the device (host side: launch shapes)
 };
+
+// Rays per warp for n rays where `warps` warps are worth launching: 32, or as many lanes fewer
+// (a power of two) as still make no more than that many warps; the other lanes idle. A launch
+// that leaves the chip part empty is as slow as its slowest warps, whose lanes wait for one
+// another at every branch of their rays' chains of dependent loads: with fewer rays beside it a
+// ray's chain is shorter, and the warps it costs have room. The launches say how many they take.
+inline int lanes_per_warp(int64_t n, int64_t warps) {
+    int lanes = 32;
+    while (lanes > 1 && n <= warps * (lanes / 2)) lanes /= 2;
+    return lanes;
+}
 
 // App. C: the scale min(1, 1.5 a) / a applied after compositing to (C_d, alpha, V) when
 // un-premultiply is on and a = 1 - T > 0 (else 1). Depends on density only.
@@ -908,7 +920,11 @@ struct SchedArgs {
     int32_t nt;                // the image's tiles
     int32_t tiles_x;
     int32_t smax;              // sparse slots of this launch (0 without previous buckets)
+    int32_t parts;             // CTAs per dense tile (1, 2, 4, 8: bands of its rows)
 };
+
+// rays per warp of a one-camera launch of n pixels
+int image_lanes(const DevScene& s, int64_t n);
 
 // pw: weights as a kernel parameter (nullptr: read them from `mlp` in device memory)
 // sch: nullable; with it the launch takes its tile order from the previous frame's
@@ -918,7 +934,7 @@ cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, cons
                                 const SchedArgs* sch = nullptr);
 cudaError_t launch_render_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
                                int64_t n, const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg,
-                               int num_sms, cudaStream_t st);
+                               cudaStream_t st);
 cudaError_t launch_backward_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
                                  const float* mlp, const float* grad_rgb, const float* fwd_aux,
                                  const int32_t* fwd_counts, float* grad_atlas, float* grad_mlp, cudaStream_t st);

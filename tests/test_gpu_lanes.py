@@ -1,0 +1,89 @@
+"""Launches that leave the chip part empty run fewer rays per warp (1, 2, 4, 8 or 16 lanes). Which
+rays share a warp changes no ray: images, row ranges, scheduled frames and ray lists of every
+size class are compared bit for bit with launches of 32 rays per warp, and the adjoint's sums
+(which rows a thread block adds up depends on the lanes) with the same rays in many small calls."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2103_14645_gb300 import renderer, synth
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+@pytest.fixture(scope="module")
+def scene():
+    sc = synth.make_scene("gauss64")
+    r = renderer.Renderer.from_scene(sc, DEV)
+    r.set_mlp(sc.mlp)
+    return sc, r, torch.from_numpy(sc.mlp).to(DEV)
+
+
+def _camera(W, H):
+    return np.asarray([synth.look_at_camera((1.5, -1.1, 0.9), (0.0, 0.0, 0.0), W, H, 45.0, 0)])
+
+
+@pytest.mark.parametrize("W,H", [(1, 1), (7, 3), (61, 37), (123, 111), (199, 143), (283, 205), (401, 283), (640, 479),
+                                 (1021, 523)])
+def test_images_of_every_size_class(scene, W, H):
+    _, r, w = scene
+    cam = _camera(W, H)
+    want = r.render(cam, w, counts=True)["rgb"]            # debug outputs: 32 rays per warp
+    assert torch.equal(r.render(cam, w), want)
+    stored = r.render(cam, None, counts=True)["rgb"]
+    assert torch.equal(r.render(cam, None), stored)
+    for _ in range(2):
+        assert torch.equal(r.render(cam, None, schedule=True), stored)
+    rows = (H // 3, H - H // 4)
+    out = torch.full((W * H, 3), -1.0, device=DEV)
+    r.render(cam, w, out=out, rows=rows)
+    inside = torch.zeros(H, dtype=torch.bool, device=DEV)
+    inside[rows[0]:rows[1]] = True
+    inside = inside[:, None].expand(H, W).reshape(-1)
+    assert torch.equal(out[inside], want[inside]) and bool((out[~inside] == -1.0).all())
+    r.check_status()
+
+
+@pytest.mark.parametrize("n", [1, 33, 4864, 4865, 9729, 19457, 38913, 77825, 155649])
+def test_ray_lists_of_every_size_class(scene, n):
+    _, r, w = scene
+    cam = _camera(1021, 523)
+    image = r.render(cam, w, counts=True)["rgb"]
+    pix = synth.random_pixels(np.random.default_rng(n), cam, n)
+    t = torch.from_numpy(pix).to(DEV)
+    want = image[t[:, 2].long() * 1021 + t[:, 1].long()]
+    assert torch.equal(r.render_rays(cam, t, w), want)
+    out = r.render_rays(cam, t, w, aux=True, counts=True)
+    assert torch.equal(out["rgb"], want)
+    r.check_status()
+
+
+@pytest.mark.parametrize("n", [5, 2432, 2433, 4865, 9729, 19457, 38913])
+def test_adjoint_sums_of_every_size_class(scene, n):
+    sc, r, w = scene
+    cam = _camera(640, 479)
+    rng = np.random.default_rng(n)
+    pix = torch.from_numpy(synth.random_pixels(rng, cam, n)).to(DEV)
+    target = torch.from_numpy(rng.uniform(size=(n, 3)).astype(np.float32)).to(DEV)
+
+    def step(lots):
+        g_atlas = torch.zeros(sc.atlas.shape, device=DEV)
+        g_mlp, loss = torch.zeros(883, device=DEV), torch.zeros(1, device=DEV)
+        rgb = torch.empty((n, 3), device=DEV)
+        b_atlas, b_mlp = torch.zeros_like(g_atlas), torch.zeros_like(g_mlp)
+        for i in range(0, n, lots):
+            sl = slice(i, min(i + lots, n))
+            out = rgb[sl]
+            r.train_rays(cam, pix[sl].contiguous(), w, target[sl].contiguous(), g_atlas, g_mlp, loss=loss, out=out)
+            r.backward(cam, pix[sl].contiguous(), w, 2.0 * (out - target[sl]), b_atlas, b_mlp)
+        return rgb, loss, g_atlas, g_mlp, b_atlas, b_mlp
+
+    whole, small = step(n), step(2000)
+    assert torch.equal(whole[0], small[0])
+    # FP32 sums of up to n terms in another order
+    for a, b in zip(whole[1:], small[1:]):
+        scale = float(b.abs().max())
+        assert float((a - b).abs().max()) <= 2e-5 * scale + 1e-7
+    assert float((whole[2] - whole[4]).abs().max()) <= 2e-5 * float(whole[2].abs().max())
+    r.check_status()
