@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const De
     }
 }
 
-// MINB: resident CTAs per SM the build is limited to (8: 64 registers; 4: up to 128);
+// MINB: resident CTAs per SM the build is limited to (7: 72 registers; 4: up to 128);
 // lanes: rays per warp (the other lanes idle)
 template <bool DBG, bool PW, int MINB>
 __global__ void __launch_bounds__(128, MINB) render_rays_kernel(const DevScene s, const __grid_constant__ CamTable cams,
@@ -417,21 +417,23 @@ static void rays_launch(const DevScene& s, const CamTable& cams, int32_t n_cams,
     }
 }
 
-// A list is spread over the warps of one wave of 8 CTAs per SM: scattered rays have less in
+// A list is spread over the warps of one wave of 7 CTAs per SM: scattered rays have less in
 // common than an image's, and a second wave costs as much as the first (4,096 rays of a 1024^3
 // grid 122 us with 32 rays per warp, 70 with 1; 16,384: 131 and, with 4, 102; 65,536: 143 with
-// 32, 145 with 16, 150 with 8; 262,144: 274, 324 with 16); with debug outputs, whose 8-CTA build
-// spills, over one wave of 4. If 4 CTAs per SM hold it, it
-// runs the build limited to 4 (the march keeps its state in registers, and a single wave gains
-// nothing from the 8-CTA occupancy); longer lists keep 8 CTAs per SM to hide the march's latencies.
+// 32, 145 with 16, 150 with 8; 262,144: 274, 324 with 16); with debug outputs, which need more
+// registers, over one wave of 4. If 4 CTAs per SM hold it, it runs the build limited to 4 (the march
+// keeps its state in registers, and a single wave gains nothing from more CTAs); longer lists
+// keep 7 CTAs per SM to hide the march's latencies: 8 spill with the weights in device memory
+// (131,072 and 262,144 rays of a 1024^3 grid 163 and 277 us with 8, 153 and 268 with 7; 1,000,000
+// rays 731 and 747).
 cudaError_t launch_render_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
                                int64_t n, const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg,
                                cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const bool d = dbg.aux || dbg.counts || dbg.trace;
-    const int lanes = lanes_per_warp(n, (int64_t)s.sms * (d ? 4 : 8) * 4);
+    const int lanes = lanes_per_warp(n, (int64_t)s.sms * (d ? 4 : 7) * 4);
     if (n <= (int64_t)s.sms * 4 * 4 * lanes) rays_launch<4>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, lanes, st);
-    else rays_launch<8>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, lanes, st);
+    else rays_launch<7>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, lanes, st);
     return cudaGetLastError();
 }
 
