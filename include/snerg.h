@@ -242,6 +242,23 @@ snerg_status snerg_render_backward(snerg_handle h, const snerg_camera* cams, int
                                    const int32_t* d_fwd_counts, float* d_grad_atlas,
                                    float* d_grad_mlp, void* stream);
 
+/* snerg_render_rays and snerg_render_backward for a program that keeps state between the two:
+ * the render also stores what the adjoint needs of each ray (its composites and its first 32
+ * composited samples' lattice indices and weights), and the adjoint does not march again.
+ *   d_state : snerg_state_bytes(n) bytes (312 per ray), 16-byte aligned, not initialised;
+ *             opaque, valid for the same handle, cameras, rays and n;
+ *   d_grad_atlas, d_grad_mlp (either nullable) are WRITTEN, not accumulated into: with the
+ *             sums that snerg_render_backward would add to zeros.
+ * d_mlp must be device weights. */
+size_t snerg_state_bytes(int64_t n);
+snerg_status snerg_render_rays_recorded(snerg_handle h, const snerg_camera* cams, int32_t n_cams,
+                                        const int32_t* d_pix, int64_t n, const float* d_mlp, float* d_rgb,
+                                        void* d_state, void* stream);
+snerg_status snerg_render_backward_recorded(snerg_handle h, const snerg_camera* cams, int32_t n_cams,
+                                            const int32_t* d_pix, int64_t n, const float* d_mlp,
+                                            const float* d_grad_rgb, const void* d_state, float* d_grad_atlas,
+                                            float* d_grad_mlp, void* stream);
+
 /* Data-parallel fine-tuning (one exchange step per training step, Sec. 5.5 run on several
  * GPUs): every rank sums dL/dPhi and the atlas gradient of its own rays, and the ranks
  * all-reduce them before the optimiser step. The atlas gradient is exchanged only over the

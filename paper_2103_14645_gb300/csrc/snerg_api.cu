@@ -583,18 +583,71 @@ static bool make_table(const snerg_camera* cams, int32_t n_cams, CamTable* t) {
     return true;
 }
 
-extern "C" snerg_status snerg_render_rays(snerg_handle h, const snerg_camera* cams, int32_t n_cams,
-                                          const int32_t* d_pix, int64_t n, const float* d_mlp, float* d_rgb,
-                                          const snerg_render_opts* opts, void* stream) {
-    if (!h || n < 0) return SNERG_E_INVAL;
-    if (h->desc.flags & SNERG_FLAG_PER_SAMPLE_MLP) return SNERG_E_UNSUPPORTED;
+static snerg_status render_rays(snerg_handle h, const snerg_camera* cams, int32_t n_cams, const int32_t* d_pix,
+                                int64_t n, const float* d_mlp, float* d_rgb, const DebugOut& dbg, float2* record,
+                                cudaStream_t st) {
     CamTable* t = new (std::nothrow) CamTable;
     if (!t) return SNERG_E_NOMEM;
     if (!make_table(cams, n_cams, t)) { delete t; return SNERG_E_INVAL; }
     if (n == 0) { delete t; return SNERG_OK; }
     if (!d_pix || !d_rgb || (!d_mlp && !h->has_w)) { delete t; return SNERG_E_INVAL; }
-    cudaError_t e = launch_render_rays(h->ds, *t, n_cams, d_pix, n, d_mlp, d_mlp ? nullptr : &h->host_w, d_rgb,
-                                       make_dbg(opts), (cudaStream_t)stream);
+    cudaError_t e = launch_render_rays(h->ds, *t, n_cams, d_pix, n, d_mlp, d_mlp ? nullptr : &h->host_w, d_rgb, dbg, record,
+                                       st);
+    delete t;
+    if (e != cudaSuccess) return SNERG_E_CUDA;
+    h->launches++;
+    return SNERG_OK;
+}
+
+extern "C" snerg_status snerg_render_rays(snerg_handle h, const snerg_camera* cams, int32_t n_cams,
+                                          const int32_t* d_pix, int64_t n, const float* d_mlp, float* d_rgb,
+                                          const snerg_render_opts* opts, void* stream) {
+    if (!h || n < 0) return SNERG_E_INVAL;
+    if (h->desc.flags & SNERG_FLAG_PER_SAMPLE_MLP) return SNERG_E_UNSUPPORTED;
+    return render_rays(h, cams, n_cams, d_pix, n, d_mlp, d_rgb, make_dbg(opts), nullptr, (cudaStream_t)stream);
+}
+
+// snerg_render_rays_recorded's state: aux [n][8] | counts [n][4] | record [kRecCap + 1][n]
+struct RayState {
+    float* aux;
+    int32_t* counts;
+    float2* record;
+};
+static RayState ray_state(const void* d_state, int64_t n) {
+    uint8_t* p = (uint8_t*)d_state;
+    return RayState{(float*)p, (int32_t*)(p + n * kAuxCh * 4), (float2*)(p + n * (kAuxCh + 4) * 4)};
+}
+
+extern "C" size_t snerg_state_bytes(int64_t n) {
+    return n > 0 ? (size_t)n * ((kAuxCh + 4) * 4 + (kRecCap + 1) * sizeof(float2)) : 0;
+}
+
+extern "C" snerg_status snerg_render_rays_recorded(snerg_handle h, const snerg_camera* cams, int32_t n_cams,
+                                                   const int32_t* d_pix, int64_t n, const float* d_mlp, float* d_rgb,
+                                                   void* d_state, void* stream) {
+    if (!h || n < 0) return SNERG_E_INVAL;
+    if (h->desc.flags & SNERG_FLAG_PER_SAMPLE_MLP) return SNERG_E_UNSUPPORTED;
+    if (n > 0 && (!d_mlp || !d_state || ((uintptr_t)d_state & 15u))) return SNERG_E_INVAL;
+    const RayState s = ray_state(d_state, n);
+    return render_rays(h, cams, n_cams, d_pix, n, d_mlp, d_rgb, DebugOut{s.aux, s.counts, nullptr, 0}, s.record,
+                       (cudaStream_t)stream);
+}
+
+static snerg_status render_backward(snerg_handle h, const snerg_camera* cams, int32_t n_cams, const int32_t* d_pix,
+                                    int64_t n, const float* d_mlp, const float* d_grad_rgb, const float* d_fwd_aux,
+                                    const int32_t* d_fwd_counts, const float2* record, float* d_grad_atlas,
+                                    float* d_grad_mlp, cudaStream_t st) {
+    if (!h || n < 0) return SNERG_E_INVAL;
+    if (h->desc.flags & SNERG_FLAG_PER_SAMPLE_MLP) return SNERG_E_UNSUPPORTED;
+    CamTable* t = new (std::nothrow) CamTable;
+    if (!t) return SNERG_E_NOMEM;
+    if (!make_table(cams, n_cams, t)) { delete t; return SNERG_E_INVAL; }
+    if (n == 0 || (!d_grad_atlas && !d_grad_mlp)) { delete t; return SNERG_OK; }
+    if (!d_pix || !d_mlp || !d_grad_rgb) { delete t; return SNERG_E_INVAL; }
+    if (d_grad_atlas && ((uintptr_t)d_grad_atlas & 15u)) { delete t; return SNERG_E_INVAL; }
+    if ((d_fwd_aux == nullptr) != (d_fwd_counts == nullptr)) { delete t; return SNERG_E_INVAL; }
+    cudaError_t e = launch_backward_rays(h->ds, *t, n_cams, d_pix, n, d_mlp, d_grad_rgb, d_fwd_aux, d_fwd_counts, record,
+                                         d_grad_atlas, d_grad_mlp, st);
     delete t;
     if (e != cudaSuccess) return SNERG_E_CUDA;
     h->launches++;
@@ -606,21 +659,26 @@ extern "C" snerg_status snerg_render_backward(snerg_handle h, const snerg_camera
                                               const float* d_grad_rgb, const float* d_fwd_aux,
                                               const int32_t* d_fwd_counts, float* d_grad_atlas, float* d_grad_mlp,
                                               void* stream) {
+    return render_backward(h, cams, n_cams, d_pix, n, d_mlp, d_grad_rgb, d_fwd_aux, d_fwd_counts, nullptr, d_grad_atlas,
+                           d_grad_mlp, (cudaStream_t)stream);
+}
+
+extern "C" snerg_status snerg_render_backward_recorded(snerg_handle h, const snerg_camera* cams, int32_t n_cams,
+                                                       const int32_t* d_pix, int64_t n, const float* d_mlp,
+                                                       const float* d_grad_rgb, const void* d_state,
+                                                       float* d_grad_atlas, float* d_grad_mlp, void* stream) {
     if (!h || n < 0) return SNERG_E_INVAL;
     if (h->desc.flags & SNERG_FLAG_PER_SAMPLE_MLP) return SNERG_E_UNSUPPORTED;
-    CamTable* t = new (std::nothrow) CamTable;
-    if (!t) return SNERG_E_NOMEM;
-    if (!make_table(cams, n_cams, t)) { delete t; return SNERG_E_INVAL; }
-    if (n == 0 || (!d_grad_atlas && !d_grad_mlp)) { delete t; return SNERG_OK; }
-    if (!d_pix || !d_mlp || !d_grad_rgb) { delete t; return SNERG_E_INVAL; }
-    if (d_grad_atlas && ((uintptr_t)d_grad_atlas & 15u)) { delete t; return SNERG_E_INVAL; }
-    if ((d_fwd_aux == nullptr) != (d_fwd_counts == nullptr)) { delete t; return SNERG_E_INVAL; }
-    cudaError_t e = launch_backward_rays(h->ds, *t, n_cams, d_pix, n, d_mlp, d_grad_rgb, d_fwd_aux, d_fwd_counts,
-                                         d_grad_atlas, d_grad_mlp, (cudaStream_t)stream);
-    delete t;
+    if (n > 0 && (!d_state || ((uintptr_t)d_state & 15u))) return SNERG_E_INVAL;
+    cudaStream_t st = (cudaStream_t)stream;
+    cudaError_t e = cudaSuccess;
+    if (d_grad_atlas && h->nb > 0)
+        e = cudaMemsetAsync(d_grad_atlas, 0, (size_t)h->nb * h->ds.B * h->ds.B * h->ds.B * 8 * sizeof(float), st);
+    if (d_grad_mlp && e == cudaSuccess) e = cudaMemsetAsync(d_grad_mlp, 0, kNParam * sizeof(float), st);
     if (e != cudaSuccess) return SNERG_E_CUDA;
-    h->launches++;
-    return SNERG_OK;
+    const RayState s = ray_state(d_state, n);
+    return render_backward(h, cams, n_cams, d_pix, n, d_mlp, d_grad_rgb, s.aux, s.counts, s.record, d_grad_atlas,
+                           d_grad_mlp, st);
 }
 
 extern "C" snerg_status snerg_train_rays(snerg_handle h, const snerg_camera* cams, int32_t n_cams,

@@ -61,19 +61,19 @@ __device__ __forceinline__ void locate_recorded(const DevScene& s, const Ray& r,
 // slot loaded) before the current one's atomics, so that those loads overlap them. T and
 // tau after the kRecCap-th sample (rec[kRecCap]) go to st for a march that continues from
 // the next lattice index (CONT).
-__device__ __forceinline__ void scatter_recorded(const DevScene& s, const Ray& r, const float2* rec, int n,
-                                                 const float* gfeat, float* grad_atlas, MarchState& st) {
+__device__ __forceinline__ void scatter_recorded(const DevScene& s, const Ray& r, const float2* rec, int64_t stride,
+                                                 int n, const float* gfeat, float* grad_atlas, MarchState& st) {
     if (n > 0) {
         const int oct = (r.d[0] < 0.0f ? 1 : 0) | (r.d[1] < 0.0f ? 2 : 0) | (r.d[2] < 0.0f ? 4 : 0);
         const int32_t* ind = s.ind + oct * s.ind_oct;
         int bprev = -1, slot = -1;
         RecSample cur, nxt;
         locate_recorded(s, r, ind, rec[0], bprev, slot, cur);
-        float2 e = n > 1 ? rec[1] : make_float2(0.0f, 0.0f);
+        float2 e = n > 1 ? rec[stride] : make_float2(0.0f, 0.0f);
         for (int j = 0; j < n; ++j) {
             if (j + 1 < n) {
                 locate_recorded(s, r, ind, e, bprev, slot, nxt);
-                if (j + 2 < n) e = rec[j + 2];
+                if (j + 2 < n) e = rec[(j + 2) * stride];
             }
             // a block without samples is never recorded by a march
             if (cur.slot >= 0) {
@@ -86,8 +86,8 @@ __device__ __forceinline__ void scatter_recorded(const DevScene& s, const Ray& r
         }
     }
     if (n == kRecCap) {
-        st.T = rec[kRecCap].x;
-        st.tau = rec[kRecCap].y;
+        st.T = rec[kRecCap * stride].x;
+        st.tau = rec[kRecCap * stride].y;
     }
 }
 
@@ -243,17 +243,19 @@ __device__ __forceinline__ void dphi_sums(const float* rows, int n_rows, float* 
 // STATE: fwd_aux / fwd_counts hold the forward's per-ray outputs (C_d, V, opacity;
 // steps, composited samples, indirection reads, first composited lattice index); the
 // kernel then skips its own first march and scatters with one march from the first
-// composited sample.
+// composited sample. RECORDED (with STATE): record holds the forward's composited samples
+// (render_rays_kernel<..., REC>), and the scatter takes them from there: a step with the march
+// again from the first sample on takes 102 us for 65,536 rays of a 512^3 grid.
 // TRAIN: one fine-tuning step for the ray in one pass (Sec. 5.5, Eq. 3): the march and the
 // MLP give C, the L2 loss |C - C*|^2 is accumulated into *loss, dL/dC = 2 (C - C*) is taken
 // in the kernel, and the adjoint follows as for a given upstream gradient; C goes to
 // rgb_out (nullable). grad_rgb, fwd_aux and fwd_counts are not used.
-template <bool TRAIN, bool STATE>
+template <bool TRAIN, bool STATE, bool RECORDED = false>
 __global__ void __launch_bounds__(kBwdThreads, 4) backward_rays_kernel(
     const DevScene s, const __grid_constant__ CamTable cams, int32_t n_cams, const int32_t* __restrict__ pix,
     int64_t n, const float* __restrict__ mlp, const float* __restrict__ grad_rgb,
-    const float* __restrict__ fwd_aux, const int32_t* __restrict__ fwd_counts, const float* __restrict__ target,
-    float* __restrict__ rgb_out, float* __restrict__ loss, float* __restrict__ grad_atlas,
+    const float* __restrict__ fwd_aux, const int32_t* __restrict__ fwd_counts, const float2* __restrict__ record,
+    const float* __restrict__ target, float* __restrict__ rgb_out, float* __restrict__ loss, float* __restrict__ grad_atlas,
     float* __restrict__ grad_mlp, int lanes) {
     extern __shared__ __align__(16) float smem[];
     __shared__ float s_loss[kBwdThreads / 32];
@@ -374,12 +376,14 @@ __global__ void __launch_bounds__(kBwdThreads, 4) backward_rays_kernel(
 #pragma unroll
         for (int c = 0; c < 4; ++c) gf[3 + c] = sc * gx[3 + c];
         MarchState st2;
-        if (!STATE) {
-            scatter_recorded(s, r, rec, min(st.active, kRecCap), gf, grad_atlas, st2);
+        if (!STATE || RECORDED) {
+            const float2* list = RECORDED ? record + i : rec;
+            const int64_t stride = RECORDED ? n : 1;
+            scatter_recorded(s, r, list, stride, min(st.active, kRecCap), gf, grad_atlas, st2);
             // a ray with more composited samples marches on from the last recorded one
             if (st.active > kRecCap)
                 march<false, true, false, true, false, true>(s, r, st2, nullptr, 0, gf, grad_atlas,
-                                                             (int)rec[kRecCap - 1].x + 1);
+                                                             (int)list[(kRecCap - 1) * stride].x + 1);
         } else {
             // without a recording (the forward's per-ray state given) a second march starts
             // at the first composited sample: nothing before it contributes (T = 1 and
@@ -404,10 +408,10 @@ __global__ void __launch_bounds__(kBwdThreads, 4) backward_rays_kernel(
     if (grad_mlp) dphi_sums(rows, kBwdThreads / 32 * lanes, grad_mlp);
 }
 
-template <bool TRAIN, bool STATE>
+template <bool TRAIN, bool STATE, bool RECORDED = false>
 static cudaError_t backward_launch(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
                                    int64_t n, const float* mlp, const float* grad_rgb, const float* fwd_aux,
-                                   const int32_t* fwd_counts, const float* target, float* rgb_out, float* loss,
+                                   const int32_t* fwd_counts, const float2* record, const float* target, float* rgb_out, float* loss,
                                    float* grad_atlas, float* grad_mlp, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     // rays spread over one wave of 4 CTAs per SM: a step of 4,096 rays on a 1024^3 grid takes
@@ -421,34 +425,38 @@ static cudaError_t backward_launch(const DevScene& s, const CamTable& cams, int3
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!attr_set[dev].load()) {
-        e = cudaFuncSetAttribute(backward_rays_kernel<TRAIN, STATE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(backward_rays_kernel<TRAIN, STATE, RECORDED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)backward_smem_bytes(32));
         if (e != cudaSuccess) return e;
         attr_set[dev].store(true);
     }
     const int rays = kBwdThreads / 32 * lanes;          // per CTA
     const unsigned grid = (unsigned)((n + rays - 1) / rays);
-    backward_rays_kernel<TRAIN, STATE><<<grid, kBwdThreads, smem, st>>>(s, cams, n_cams, pix, n, mlp, grad_rgb,
-                                                                        fwd_aux, fwd_counts, target, rgb_out, loss,
-                                                                        grad_atlas, grad_mlp, lanes);
+    backward_rays_kernel<TRAIN, STATE, RECORDED><<<grid, kBwdThreads, smem, st>>>(
+        s, cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, record, target, rgb_out, loss, grad_atlas, grad_mlp,
+        lanes);
     return cudaGetLastError();
 }
 
 cudaError_t launch_backward_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
                                  int64_t n, const float* mlp, const float* grad_rgb, const float* fwd_aux,
-                                 const int32_t* fwd_counts, float* grad_atlas, float* grad_mlp, cudaStream_t st) {
+                                 const int32_t* fwd_counts, const float2* record, float* grad_atlas, float* grad_mlp,
+                                 cudaStream_t st) {
+    if (fwd_aux && record)
+        return backward_launch<false, true, true>(s, cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, record,
+                                                  nullptr, nullptr, nullptr, grad_atlas, grad_mlp, st);
     if (fwd_aux)
-        return backward_launch<false, true>(s, cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, nullptr,
+        return backward_launch<false, true>(s, cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, nullptr, nullptr,
                                             nullptr, nullptr, grad_atlas, grad_mlp, st);
     return backward_launch<false, false>(s, cams, n_cams, pix, n, mlp, grad_rgb, nullptr, nullptr, nullptr, nullptr,
-                                         nullptr, grad_atlas, grad_mlp, st);
+                                         nullptr, nullptr, grad_atlas, grad_mlp, st);
 }
 
 cudaError_t launch_train_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
                               const float* mlp, const float* target, float* rgb_out, float* loss, float* grad_atlas,
                               float* grad_mlp, cudaStream_t st) {
-    return backward_launch<true, false>(s, cams, n_cams, pix, n, mlp, nullptr, nullptr, nullptr, target, rgb_out, loss,
-                                 grad_atlas, grad_mlp, st);
+    return backward_launch<true, false>(s, cams, n_cams, pix, n, mlp, nullptr, nullptr, nullptr, nullptr, target, rgb_out,
+                                        loss, grad_atlas, grad_mlp, st);
 }
 
 }  // namespace snerg

@@ -211,14 +211,15 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const De
 }
 
 // MINB: resident CTAs per SM the build is limited to (7: 72 registers; 4: up to 128);
-// lanes: rays per warp (the other lanes idle)
-template <bool DBG, bool PW, int MINB>
+// lanes: rays per warp (the other lanes idle); REC: each ray's composited samples go to
+// record (entry j of ray i at record[j * n + i], see march) for the adjoint
+template <bool DBG, bool PW, int MINB, bool REC = false>
 __global__ void __launch_bounds__(128, MINB) render_rays_kernel(const DevScene s, const __grid_constant__ CamTable cams,
                                                                 int32_t n_cams, const int32_t* __restrict__ pix,
                                                                 int64_t n, const float* __restrict__ mlp,
                                                                 const __grid_constant__ MlpWeights pw,
                                                                 float* __restrict__ rgb, const DebugOut dbg,
-                                                                int lanes) {
+                                                                float2* __restrict__ record, int lanes) {
     __shared__ __align__(16) float sW[PW ? 4 : kNParam + 1];
     if (!PW) {
         load_mlp_smem_t(sW, mlp);
@@ -238,7 +239,10 @@ __global__ void __launch_bounds__(128, MINB) render_rays_kernel(const DevScene s
     }
     MarchState st;
     int k_first = 0;
-    if (DBG && dbg.trace)
+    if (REC)
+        march<false, false, false, true, true>(s, r, st, nullptr, 0, nullptr, nullptr, 0, &k_first, nullptr, nullptr,
+                                               record + i, n);
+    else if (DBG && dbg.trace)
         march<true, false>(s, r, st, dbg.trace + i * dbg.trace_cap, dbg.trace_cap, nullptr, nullptr, 0, &k_first);
     else
         march<false, false, false, true>(s, r, st, nullptr, 0, nullptr, nullptr, 0, DBG ? &k_first : nullptr);
@@ -403,18 +407,14 @@ cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, cons
 
 template <int MINB>
 static void rays_launch(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
-                        const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, int lanes,
+                        const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, float2* record, int lanes,
                         cudaStream_t st) {
     const unsigned grid = (unsigned)((n + 4 * lanes - 1) / (4 * lanes));
     const bool d = dbg.aux || dbg.counts || dbg.trace;
-    const MlpWeights& w = pw ? *pw : no_weights();
-    if (pw) {
-        if (d) render_rays_kernel<true, true, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg, lanes);
-        else render_rays_kernel<false, true, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg, lanes);
-    } else {
-        if (d) render_rays_kernel<true, false, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg, lanes);
-        else render_rays_kernel<false, false, MINB><<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, w, rgb, dbg, lanes);
-    }
+    auto* kernel = record ? render_rays_kernel<true, false, MINB, true>       // recorded: weights in device memory
+                   : pw   ? (d ? render_rays_kernel<true, true, MINB> : render_rays_kernel<false, true, MINB>)
+                          : (d ? render_rays_kernel<true, false, MINB> : render_rays_kernel<false, false, MINB>);
+    kernel<<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, pw ? *pw : no_weights(), rgb, dbg, record, lanes);
 }
 
 // A list is spread over the warps of one wave of 7 CTAs per SM: scattered rays have less in
@@ -428,12 +428,12 @@ static void rays_launch(const DevScene& s, const CamTable& cams, int32_t n_cams,
 // rays 731 and 747).
 cudaError_t launch_render_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
                                int64_t n, const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg,
-                               cudaStream_t st) {
+                               float2* record, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const bool d = dbg.aux || dbg.counts || dbg.trace;
     const int lanes = lanes_per_warp(n, (int64_t)s.sms * (d ? 4 : 7) * 4);
-    if (n <= (int64_t)s.sms * 4 * 4 * lanes) rays_launch<4>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, lanes, st);
-    else rays_launch<7>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, lanes, st);
+    if (n <= (int64_t)s.sms * 4 * 4 * lanes) rays_launch<4>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, record, lanes, st);
+    else rays_launch<7>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, record, lanes, st);
     return cudaGetLastError();
 }
 

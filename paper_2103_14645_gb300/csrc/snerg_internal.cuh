@@ -499,7 +499,7 @@ constexpr int kRecCap = 32;
 // the march. TRACE records visited voxels; GRAD scatters w_k * trilinear weight * g
 // into the gradient atlas (density frozen, so the weights are the forward ones); REC
 // stores the lattice index and weight of the first kRecCap composited samples in rec[j]
-// and T, tau after them in rec[kRecCap]; CONT starts from the T and tau already in st (a
+// and T, tau after them in rec[kRecCap] (entries rec_stride apart); CONT starts from the T and tau already in st (a
 // march resumed after recorded samples).
 // ---------------------------------------------------------------------------------
 // k_begin: first lattice index to consider (0, or a k known to precede every composited
@@ -518,7 +518,7 @@ __device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchStat
                                       const float* gfeat, float* grad_atlas,
                                       int k_begin = 0, int* k_first = nullptr,
                                       const MlpWeights* ps_w = nullptr, const float* ps_sw = nullptr,
-                                      float2* rec = nullptr) {
+                                      float2* rec = nullptr, int64_t rec_stride = 1) {
 #pragma unroll
     for (int c = 0; c < 7; ++c) st.acc[c] = 0.0f;
     st.rgb_ps[0] = st.rgb_ps[1] = st.rgb_ps[2] = 0.0f;
@@ -615,8 +615,8 @@ __device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchStat
             bool saturated;
             const float wk = composite(s, cv, f, g, st.T, st.tau, saturated);
             if (REC && st.active <= kRecCap) {
-                rec[st.active - 1] = make_float2(kk - 0.5f, wk);
-                if (st.active == kRecCap) rec[kRecCap] = make_float2(st.T, st.tau);
+                rec[(st.active - 1) * rec_stride] = make_float2(kk - 0.5f, wk);
+                if (st.active == kRecCap) rec[kRecCap * rec_stride] = make_float2(st.T, st.tau);
             }
             accumulate_colour(st, cv, wk, f, g);
             if (PS) {
@@ -934,10 +934,11 @@ cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, cons
                                 const SchedArgs* sch = nullptr);
 cudaError_t launch_render_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
                                int64_t n, const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg,
-                               cudaStream_t st);
+                               float2* record, cudaStream_t st);
 cudaError_t launch_backward_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
                                  const float* mlp, const float* grad_rgb, const float* fwd_aux,
-                                 const int32_t* fwd_counts, float* grad_atlas, float* grad_mlp, cudaStream_t st);
+                                 const int32_t* fwd_counts, const float2* record, float* grad_atlas, float* grad_mlp,
+                                 cudaStream_t st);
 cudaError_t launch_validate(const int32_t* ind, int64_t n_ind, int64_t nb, int32_t* blk_of_slot, int32_t* err,
                             cudaStream_t st);
 // the padded atlas and the 8 octants' voxel-distance planes of every stored block; a launch

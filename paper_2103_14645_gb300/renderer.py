@@ -32,7 +32,8 @@ EXPORTED = ["snerg_workspace_bytes", "snerg_create", "snerg_render", "snerg_rend
             "snerg_persistent_config", "snerg_destroy", "snerg_status_str", "snerg_render_rays_noalloc",
             "snerg_set_mlp", "snerg_l2_loss", "snerg_adam_step", "snerg_bake_workspace_bytes", "snerg_bake",
             "snerg_requantize_atlas", "snerg_adam_requantize_atlas", "snerg_grad_blocks_touched", "snerg_grad_blocks_gather",
-            "snerg_grad_blocks_scatter", "snerg_render_to_host", "snerg_train_rays", "snerg_schedule_stats"]
+            "snerg_grad_blocks_scatter", "snerg_render_to_host", "snerg_train_rays", "snerg_schedule_stats",
+            "snerg_state_bytes", "snerg_render_rays_recorded", "snerg_render_backward_recorded"]
 MAX_BAKE_BLOBS = 64
 
 
@@ -84,6 +85,12 @@ def load_library(path: str = LIB_PATH):
     lib.snerg_render_rays.restype = ctypes.c_int
     lib.snerg_render_backward.argtypes = [P, P, i32, P, i64, P, P, P, P, P, P, P]
     lib.snerg_render_backward.restype = ctypes.c_int
+    lib.snerg_state_bytes.argtypes = [i64]
+    lib.snerg_state_bytes.restype = ctypes.c_size_t
+    lib.snerg_render_rays_recorded.argtypes = [P, P, i32, P, i64, P, P, P, P]
+    lib.snerg_render_rays_recorded.restype = ctypes.c_int
+    lib.snerg_render_backward_recorded.argtypes = [P, P, i32, P, i64, P, P, P, P, P, P]
+    lib.snerg_render_backward_recorded.restype = ctypes.c_int
     lib.snerg_last_status.argtypes = [P, P]
     lib.snerg_last_status.restype = ctypes.c_int
     lib.snerg_launch_count.argtypes = [P]
@@ -362,6 +369,43 @@ class Renderer:
             return extra
         return out
 
+    def render_rays_recorded(self, cams, pix: torch.Tensor, mlp: torch.Tensor):
+        """render_rays, and the state that backward_recorded needs of each ray
+        (snerg_render_rays_recorded): (rgb, state)."""
+        c = _cams(cams)
+        _require_cuda(pix, "pix", torch.int32)
+        _require_cuda(mlp, "mlp", torch.float32)
+        n = int(pix.shape[0])
+        rgb = torch.empty((n, 3), dtype=torch.float32, device=self.device)
+        state = torch.empty(self.lib.snerg_state_bytes(n), dtype=torch.uint8, device=self.device)
+        _check(self.lib.snerg_render_rays_recorded(self.handle, c.ctypes.data, c.shape[0], pix.data_ptr(), n,
+                                                   mlp.data_ptr(), rgb.data_ptr(), state.data_ptr(),
+                                                   _stream(self.device)), "snerg_render_rays_recorded")
+        return rgb, state
+
+    def backward_recorded(self, cams, pix: torch.Tensor, mlp: torch.Tensor, grad_rgb: torch.Tensor,
+                          state: torch.Tensor, grad_atlas: torch.Tensor | None, grad_mlp: torch.Tensor | None):
+        """Write dL/d(atlas values) and dL/d(mlp) for dL/dC of a render_rays_recorded call
+        (snerg_render_backward_recorded; backward accumulates, this overwrites)."""
+        c = _cams(cams)
+        _require_cuda(pix, "pix", torch.int32)
+        _require_cuda(mlp, "mlp", torch.float32)
+        _require_cuda(grad_rgb, "grad_rgb", torch.float32)
+        _require_cuda(state, "state", torch.uint8)
+        n = int(pix.shape[0])
+        if state.numel() != self.lib.snerg_state_bytes(n) or grad_rgb.numel() != 3 * n:
+            raise ValueError("state and grad_rgb must be those of pix")
+        if grad_atlas is not None:
+            _require_cuda(grad_atlas, "grad_atlas", torch.float32)
+            if grad_atlas.numel() != self.nb * self.B ** 3 * 8:
+                raise ValueError("grad_atlas must have nb*B^3*8 elements")
+        if grad_mlp is not None:
+            _require_cuda(grad_mlp, "grad_mlp", torch.float32)
+        _check(self.lib.snerg_render_backward_recorded(self.handle, c.ctypes.data, c.shape[0], pix.data_ptr(), n,
+                                                       mlp.data_ptr(), grad_rgb.data_ptr(), state.data_ptr(),
+                                                       _ptr(grad_atlas), _ptr(grad_mlp), _stream(self.device)),
+               "snerg_render_backward_recorded")
+
     def backward(self, cams, pix: torch.Tensor, mlp: torch.Tensor, grad_rgb: torch.Tensor,
                  grad_atlas: torch.Tensor | None = None, grad_mlp: torch.Tensor | None = None,
                  fwd_aux: torch.Tensor | None = None, fwd_counts: torch.Tensor | None = None):
@@ -429,22 +473,31 @@ class SnergRenderFn(torch.autograd.Function):
         ctx.renderer = renderer
         ctx.cams = cams
         ctx.atlas_shape = atlas_values.shape
-        out = renderer.render_rays(cams, pix, mlp.detach().contiguous(), aux=True, counts=True)
-        # per-ray state (C_d, V, first composited index) for the backward's single march
+        w = mlp.detach().contiguous()
+        # per-ray state for the backward: with the composited samples if they are to be scattered
+        if ctx.needs_input_grad[1]:
+            rgb, state = renderer.render_rays_recorded(cams, pix, w)
+            ctx.save_for_backward(mlp, pix, state)
+            return rgb
+        out = renderer.render_rays(cams, pix, w, aux=True, counts=True)
         ctx.save_for_backward(mlp, pix, out["aux"], out["counts"])
         return out["rgb"]
 
     @staticmethod
     def backward(ctx, grad_rgb):
-        mlp, pix, aux, counts = ctx.saved_tensors
+        mlp, pix, *state = ctx.saved_tensors
         r = ctx.renderer
-        g_mlp = torch.zeros(MLP_PARAMS, dtype=torch.float32, device=r.device) if ctx.needs_input_grad[0] else None
-        g_atl = (torch.zeros(ctx.atlas_shape, dtype=torch.float32, device=r.device)
-                 if ctx.needs_input_grad[1] else None)
-        if g_mlp is not None or g_atl is not None:
-            r.backward(ctx.cams, pix, mlp.detach().contiguous(), grad_rgb.contiguous().float(), g_atl, g_mlp,
-                       fwd_aux=aux, fwd_counts=counts)
-        return g_mlp, g_atl, None, None, None
+        w, g = mlp.detach().contiguous(), grad_rgb.contiguous().float()
+        if ctx.needs_input_grad[1]:
+            g_atl = torch.empty(ctx.atlas_shape, dtype=torch.float32, device=r.device)
+            g_mlp = torch.empty(MLP_PARAMS, dtype=torch.float32, device=r.device) if ctx.needs_input_grad[0] else None
+            r.backward_recorded(ctx.cams, pix, w, g, state[0], g_atl, g_mlp)
+            return g_mlp, g_atl, None, None, None
+        g_mlp = None
+        if ctx.needs_input_grad[0]:
+            g_mlp = torch.zeros(MLP_PARAMS, dtype=torch.float32, device=r.device)
+            r.backward(ctx.cams, pix, w, g, None, g_mlp, fwd_aux=state[0], fwd_counts=state[1])
+        return g_mlp, None, None, None, None
 
 
 def render_rays_autograd(renderer: Renderer, cams, pix: torch.Tensor, mlp: torch.Tensor,
@@ -547,8 +600,8 @@ class FineTuner:
         self.mlp = torch.as_tensor(np.asarray(mlp, np.float32)).to(renderer.device).contiguous()
         self.m = torch.zeros_like(self.mlp)
         self.v = torch.zeros_like(self.mlp)
-        self.grad = torch.zeros_like(self.mlp)
-        self.loss = torch.zeros(1, dtype=torch.float32, device=renderer.device)
+        sums = torch.zeros(MLP_PARAMS + 1, dtype=torch.float32, device=renderer.device)
+        self.sums, self.grad, self.loss = sums, sums[:MLP_PARAMS], sums[MLP_PARAMS:]     # cleared together
         self.lr, self.betas, self.eps = lr, betas, eps
         self.steps = 0
         # 8 waves of the adjoint kernel (4 CTAs of 128 rays per SM): up to there the one-launch
@@ -570,22 +623,25 @@ class FineTuner:
     def step(self, cams, pix: torch.Tensor, target: torch.Tensor) -> torch.Tensor:
         """One Adam step on rays pix [n,3] with observed colours target [n,3]; returns the
         loss before the step (a device tensor [1])."""
-        self.loss.zero_()
-        self.grad.zero_()
-        ga = None
-        if self.shadow is not None:
-            self.grad_atlas.zero_()
-            ga = self.grad_atlas
+        self.sums.zero_()
+        ga = None if self.shadow is None else self.grad_atlas
         if pix.shape[0] <= self.fused_rays:
             # render, loss and adjoint of every ray in one launch: one launch tail replaces
             # two, and no per-ray forward state goes through memory
+            if ga is not None:
+                ga.zero_()
             self.r.train_rays(cams, pix, self.mlp, target, ga, self.grad, loss=self.loss)
-        else:
+        elif ga is not None:
             # larger batches: the forward at its own (higher) occupancy, keeping per-ray state
+            rgb, state = self.r.render_rays_recorded(cams, pix, self.mlp)
+            g = torch.empty_like(rgb)
+            l2_loss(rgb, target, g, self.loss)
+            self.r.backward_recorded(cams, pix, self.mlp, g, state, ga, self.grad)
+        else:
             fwd = self.r.render_rays(cams, pix, self.mlp, aux=True, counts=True)
             g = torch.empty_like(fwd["rgb"])
             l2_loss(fwd["rgb"], target, g, self.loss)
-            self.r.backward(cams, pix, self.mlp, g, ga, self.grad, fwd_aux=fwd["aux"], fwd_counts=fwd["counts"])
+            self.r.backward(cams, pix, self.mlp, g, None, self.grad, fwd_aux=fwd["aux"], fwd_counts=fwd["counts"])
         if _data_parallel(self.group):
             allreduce_gradients(self.grad, ga, self.group)
         self.steps += 1
