@@ -8,6 +8,8 @@
 // following samples are certainly empty. The 1-voxel apron makes every trilinear
 // stencil of a sample a fetch from one block: atlas neighbours are not spatial neighbours (Sec. 5.1), so without it a sample
 // near a block face would need up to 8 indirection lookups.
+#include <type_traits>
+
 #include "snerg_internal.cuh"
 
 namespace snerg {
@@ -169,13 +171,13 @@ __global__ void encode_distance_kernel(const int32_t* __restrict__ src, const ui
 }
 
 // ---------------------------------------------------------------------------------
-// The device layout of the stored blocks, one CTA of 8 warps for one block (B >= 32) or
-// for 32 / B blocks side by side in a warp's lanes:
-//   1. the block's voxels are read once, row by row, copied into the padded atlas, and each
-//      row's non-zero density codes kept as a bit mask in shared memory;
-//   2. the apron: padded coordinate p in [0, B+2) is the global voxel block_origin + p - 1,
-//      clamped to the grid (clamp-to-edge); its owner block supplies the value, 0 if empty;
-//   3. warp o computes octant o's voxel distances from the masks, with no pass over memory
+// The device layout of the stored blocks, one CTA for one block (B >= 32) or for 32 / B blocks
+// side by side in a warp's lanes:
+//   1. the padded copy row by row, and each of the block's own rows' non-zero density codes as a
+//      bit mask in shared memory: padded coordinate p in [0, B+2) is the global voxel
+//      block_origin + p - 1, clamped to the grid (clamp-to-edge); its owner block supplies the
+//      value, 0 if empty (one owner for a row, two more for its ends);
+//   2. the warps compute the octants' voxel distances from the masks, with no pass over memory
 //      but the store of the result. The distance to the nearest set voxel in the cone obeys
 //          D(p) = 0 if p is set, else 1 + min over the 7 neighbours p + {0, 1}^3 \ 0
 //      (steps in the cone's directions). Along x, D(x) <= 1 + D(x + 1) in the rows already
@@ -187,72 +189,73 @@ __global__ void encode_distance_kernel(const int32_t* __restrict__ src, const ui
 // Apron cells of the distance planes hold 255, or, outside the grid, the value of the voxel
 // that they clamp to, so that a sample which rounding puts a hair outside the grid finds its
 // clamped nearest voxel's value without a clamp.
-// Bound by issue and by the latency of the first two parts: 0.77 ms for 2,144 blocks of 32^3,
-// whose 1.8 GB read and written would take 0.27 ms at the copy rate. Separate seed, x, y, z,
-// apron and border passes with a scan per voxel took 25.4 ms.
+// 2,144 blocks of 32^3 take 0.53 ms: the first part 0.22, bound by memory (1.35 GB at 6 TB/s), the
+// second 0.30, bound by issue. Separate seed, x, y, z, apron and border passes with a scan per
+// voxel took 25.4 ms; one octant per warp and the apron gathered voxel by voxel 0.77 ms.
 // ---------------------------------------------------------------------------------
-constexpr int kPrepThreads = 256;
-
 template <int LGB>
 struct PrepShape {
     static constexpr int B = 1 << LGB, P = B + 2, P2 = P * P, P3 = P2 * P, B2 = B * B, B3 = B2 * B;
     static constexpr int LX = B < 32 ? B : 32;      // lanes along x
     static constexpr int NB = 32 / LX;              // blocks per CTA
     static constexpr int VPL = B / LX;              // voxels per lane along x (2 for B = 64)
-    static constexpr int kApron = P3 - B3;
-    static constexpr int kMinCtas = VPL == 2 ? 2 : 4;
-    static constexpr int kSmem = 2 * VPL * B2 * 4 + kPrepThreads / 32 * NB * P2;    // row masks, slices
+    static constexpr int OPW = VPL == 2 ? 1 : 2;    // octants per warp: the two sides along y
+    static constexpr int kWarps = 8 / OPW, kThreads = 32 * kWarps;
+    static constexpr int kMinCtas = VPL == 2 ? 2 : 8;
+    static constexpr int kSmem = 2 * VPL * B2 * 4 + 8 * NB * P2;    // row masks, the octants' slices
 };
 
-// the cone distance of one row: prev / pprev the z + 1 slice's rows y and y + 1, cur the row
-// y + 1 (16-bit pairs for two voxels per lane); wa, wb the row's masks in lane order
+// The cone distance of one row: prev / pprev the z + 1 slice's rows y and y + 1, cur the row
+// y + 1, all as 16-bit pairs. VPL 1: the row y of the octant with the cone towards lower y and
+// the row B - 1 - y of the other, wa and wb their masks in lane order. VPL 2: the lane's two
+// voxels of one octant's row, wa and wb the masks of the first and of the second.
 template <int VPL>
 __device__ __forceinline__ uint32_t prep_row(uint32_t cur, uint32_t prev, uint32_t pprev, uint32_t wa, uint32_t wb,
                                              int lane, uint32_t le, uint32_t lt, int lx) {
-    if (VPL == 1) {
-        const int m = (int)min(min(cur, prev), pprev);
-        const int mx = __shfl_up_sync(0xffffffffu, m, 1, lx);     // the first lane of a block gets its own m back
-        int D = __viaddmin_s32(min(m, mx), 1, 255);
-        if (wa) {                                                 // the same for all lanes
-            const uint32_t t = wa & le;
-            if (t) D = min(D, lane - (31 - __clz(t)));
+    const uint32_t m = __vimin3_u16x2(cur, prev, pprev);
+    // x + 1: the lane before's (the first lane of a block gets its own m back), or for VPL 2
+    // (low: the lane before's high; high: own low)
+    uint32_t mx = __shfl_up_sync(0xffffffffu, m, 1, lx);
+    if (VPL == 2) mx = __byte_perm(m, lane == 0 ? 0x00ff00ffu : mx, 0x1076);
+    uint32_t D = __viaddmin_u16x2(__vminu2(m, mx), 0x00010001u, 0x00ff00ffu);
+    if (wa | wb) {                                                // the same for all lanes
+        const uint32_t ta = wa & le, tb = wb & le;
+        const int la = 31 - __clz(ta), lb = 31 - __clz(tb);
+        int da, db;
+        if (VPL == 1) {
+            da = ta ? lane - la : 255;
+            db = tb ? lane - lb : 255;
+        } else {
+            const uint32_t ua = wb & lt;
+            const int lu = 31 - __clz(ua);
+            da = min(ta ? 2 * (lane - la) : 255, ua ? 2 * (lane - lu) - 1 : 255);
+            db = min(tb ? 2 * (lane - lb) : 255, ta ? 2 * (lane - la) + 1 : 255);
         }
-        return (uint32_t)D;
-    }
-    const uint32_t m = __vminu2(__vminu2(cur, prev), pprev);
-    uint32_t up = __shfl_up_sync(0xffffffffu, m, 1);
-    if (lane == 0) up = 0x00ff00ffu;
-    const uint32_t mx = __byte_perm(m, up, 0x1076);               // (low: the lane before's high; high: own low)
-    uint32_t D = __vminu2(__vadd2(__vminu2(m, mx), 0x00010001u), 0x00ff00ffu);
-    if (wa | wb) {
-        const uint32_t ta = wa & le, tb = wb & le, ua = wb & lt;
-        const int la = 31 - __clz(ta), lb = 31 - __clz(tb), lu = 31 - __clz(ua);
-        const int da = min(ta ? 2 * (lane - la) : 255, ua ? 2 * (lane - lu) - 1 : 255);
-        const int db = min(tb ? 2 * (lane - lb) : 255, ta ? 2 * (lane - la) + 1 : 255);
         D = __vminu2(D, (uint32_t)da | ((uint32_t)db << 16));
     }
     return D;
 }
 
-// one slice (z) of one octant's plane into shared memory; SY: the cone's side along y
+// One slice (z) into shared memory: VPL 1 of both octants of a pair (out_a, out_b), VPL 2 of one
+// (SY: the cone's side along y), its voxels at out_a and out_b.
 template <int LGB, bool SY>
 __device__ __forceinline__ void prep_slice(uint32_t (&prev)[1 << LGB], const uint32_t* ma, const uint32_t* mb,
                                            uint8_t* out_a, uint8_t* out_b, int lane, uint32_t le, uint32_t lt) {
     using S = PrepShape<LGB>;
-    uint32_t cur = S::VPL == 1 ? 255u : 0x00ff00ffu, pprev = cur;
+    uint32_t cur = 0x00ff00ffu, pprev = cur;
 #pragma unroll
     for (int yi = 0; yi < S::B; ++yi) {
-        const int y = SY ? yi : S::B - 1 - yi;
-        cur = prep_row<S::VPL>(cur, prev[yi], pprev, ma[y], S::VPL == 2 ? mb[y] : 0u, lane, le, lt, S::LX);
+        const int ya = SY ? yi : S::B - 1 - yi, yb = S::VPL == 2 ? ya : S::B - 1 - ya;
+        cur = prep_row<S::VPL>(cur, prev[yi], pprev, ma[ya], mb[yb], lane, le, lt, S::LX);
         pprev = prev[yi];
         prev[yi] = cur;
-        out_a[(y + 1) * S::P] = (uint8_t)cur;
-        if (S::VPL == 2) out_b[(y + 1) * S::P] = (uint8_t)(cur >> 16);
+        out_a[(ya + 1) * S::P] = (uint8_t)cur;
+        out_b[(yb + 1) * S::P] = (uint8_t)(cur >> 16);
     }
 }
 
 template <int LGB>
-__global__ void __launch_bounds__(kPrepThreads, PrepShape<LGB>::kMinCtas) prep_blocks_kernel(
+__global__ void __launch_bounds__(PrepShape<LGB>::kThreads, PrepShape<LGB>::kMinCtas) prep_blocks_kernel(
     const int32_t* __restrict__ ind, const int32_t* __restrict__ blk_of_slot, const int32_t* __restrict__ err,
     const uint2* __restrict__ atlas, int64_t nb, int G, uint2* __restrict__ patlas, uint8_t* __restrict__ vskip) {
     using S = PrepShape<LGB>;
@@ -260,14 +263,14 @@ __global__ void __launch_bounds__(kPrepThreads, PrepShape<LGB>::kMinCtas) prep_b
     extern __shared__ __align__(16) uint32_t s_mem[];
     // a row's mask: bit g * LX + x (VPL 2: one word for even, one for odd x), and bit-reversed
     uint32_t(*s_mask)[S::VPL][S::B2] = reinterpret_cast<uint32_t(*)[S::VPL][S::B2]>(s_mem);
-    // a warp's slice of its plane
+    // the octants' slices
     uint8_t(*s_slice)[S::NB][S::P2] = reinterpret_cast<uint8_t(*)[S::NB][S::P2]>(s_mem + 2 * S::VPL * S::B2);
     __shared__ int s_own[S::NB][27];             // slots of the 3^3 blocks around, -1 empty
     __shared__ int s_edge[S::NB];                // bit 2 a (+ 1): first (last) block along axis a
     if (*err) return;                            // an invalid indirection grid: the host reports it
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t slot0 = (int64_t)blockIdx.x * S::NB;
-    for (int i = tid; i < S::NB * 27; i += kPrepThreads) {
+    for (int i = tid; i < S::NB * 27; i += S::kThreads) {
         const int g = i / 27, k = i % 27;
         const int blk = slot0 + g < nb ? blk_of_slot[slot0 + g] : -1;
         int own = -1;
@@ -286,95 +289,66 @@ __global__ void __launch_bounds__(kPrepThreads, PrepShape<LGB>::kMinCtas) prep_b
     }
     __syncthreads();
 
-    // 1. the blocks' own voxels (an unreferenced slot is stored as zeros)
+    // 1. the padded copy, a z slice per warp, kRows rows' loads in flight (the votes keep them from
+    // being moved up); an unreferenced slot is stored as zeros
     {
         const int g = lane / LX, x = lane % LX;
         const int64_t slot = slot0 + g;
-        const bool in = slot < nb, used = in && s_own[g][13] >= 0;
-        const uint2* src = atlas + slot * S::B3;
-        uint2* dst = patlas + slot * S::P3 + S::P2 + P + 1;
-        // kRows rows' loads in flight (the votes keep them from being moved up)
-        constexpr int kRows = 8, kWarps = kPrepThreads / 32;
-        for (int r0 = warp; r0 < S::B2; r0 += kRows * kWarps) {
-            uint2 v[kRows][S::VPL];
+        const bool in = slot < nb, first = x == 0, last = x == LX - 1;
+        const int edge = s_edge[g];
+        // the x apron's voxel beside a block's first and last: of the neighbour, or the clamped one
+        const int side = first ? 0 : 2;
+        const int side_x = first ? (edge & 1 ? 0 : B - 1) : (edge & 2 ? B - 1 : 0);
+        const int side_px = first ? 0 : P - 1;
+        uint2* dst = patlas + slot * S::P3 + 1 + S::VPL * x;
+        constexpr int kRows = B < 8 / S::VPL ? B : 8 / S::VPL;
+        for (int pz = warp; pz < P; pz += S::kWarps) {
+            const int nz = pz == 0 ? 0 : (pz == P - 1 ? 2 : 1);
+            const int lz = nz == 1 ? pz - 1 : (nz == 0 ? (edge & 16 ? 0 : B - 1) : (edge & 32 ? B - 1 : 0));
+            // n rows from py on, of the neighbours ny along y, from their row ly on
+            auto rows = [&](auto n, int ny, int ly, int py) {
+                constexpr int kN = decltype(n)::value;
+                const int* own = s_own[g] + (nz * 3 + ny) * 3;
+                const int mid = in ? own[1] : -1, beside = in && (first || last) ? own[side] : -1;
+                const int64_t line = (int64_t)(lz * B + ly) * B;
+                const uint2* src = atlas + (int64_t)mid * S::B3 + line + S::VPL * x;
+                const uint2* end = atlas + (int64_t)beside * S::B3 + line + side_x;
+                uint2* d = dst + (pz * P + py) * P;
+                uint2 v[kN][S::VPL], e[kN];
 #pragma unroll
-            for (int u = 0; u < kRows; ++u)
+                for (int u = 0; u < kN; ++u) {
 #pragma unroll
-                for (int q = 0; q < S::VPL; ++q) {
-                    const int row = r0 + u * kWarps;
-                    const bool on = used && (S::B2 % (kRows * kWarps) == 0 || row < S::B2);
-                    // 8-byte loads: the atlas need not be aligned to more
-                    v[u][q] = on ? __ldg(src + row * B + S::VPL * x + q) : make_uint2(0u, 0u);
+                    for (int q = 0; q < S::VPL; ++q)  // 8-byte loads: the atlas need not be aligned to more
+                        v[u][q] = mid >= 0 ? __ldg(src + u * B + q) : make_uint2(0u, 0u);
+                    e[u] = beside >= 0 ? __ldg(end + u * B) : make_uint2(0u, 0u);
                 }
 #pragma unroll
-            for (int u = 0; u < kRows; ++u) {
-                const int row = r0 + u * kWarps;
-                if (S::B2 % (kRows * kWarps) != 0 && row >= S::B2) break;
-                uint2* d = dst + ((row >> LGB) * P + (row & (B - 1))) * P + S::VPL * x;
+                for (int u = 0; u < kN; ++u) {
 #pragma unroll
-                for (int q = 0; q < S::VPL; ++q) {
-                    if (in) d[q] = v[u][q];
-                    const uint32_t m = __ballot_sync(0xffffffffu, (v[u][q].x & 0xffu) != 0u);
-                    if (lane == 0) {
-                        s_mask[0][S::VPL - 1 - q][row] = __brev(m);
-                        s_mask[1][q][row] = m;
+                    for (int q = 0; q < S::VPL; ++q) {
+                        if (in) d[u * P + q] = v[u][q];
+                        if (nz == 1 && ny == 1) {
+                            const uint32_t m = __ballot_sync(0xffffffffu, (v[u][q].x & 0xffu) != 0u);
+                            if (lane == 0) {
+                                s_mask[0][S::VPL - 1 - q][lz * B + ly + u] = __brev(m);
+                                s_mask[1][q][lz * B + ly + u] = m;
+                            }
+                        }
                     }
+                    if (in && (first || last)) d[u * P + side_px - 1 - S::VPL * x] = e[u];
                 }
-            }
+            };
+            rows(std::integral_constant<int, 1>{}, 0, edge & 4 ? 0 : B - 1, 0);
+            for (int y = 0; y < B; y += kRows) rows(std::integral_constant<int, kRows>{}, 1, y, y + 1);
+            rows(std::integral_constant<int, 1>{}, 2, edge & 8 ? B - 1 : 0, P - 1);
         }
-    }
-    // 2. the apron: two z faces of P x P, two y faces of P x B, two x faces of B x B
-    constexpr int kCells = 4;       // loads in flight per thread
-    for (int i0 = tid; i0 < S::NB * S::kApron; i0 += kCells * kPrepThreads) {
-        uint2 v[kCells];
-        int64_t at[kCells];
-#pragma unroll
-        for (int u = 0; u < kCells; ++u) {
-            const int i = i0 + u * kPrepThreads, g = i / S::kApron;
-            int a = i % S::kApron, px, py, pz;
-            at[u] = -1;
-            if (i >= S::NB * S::kApron || slot0 + g >= nb) continue;
-            if (a < 2 * S::P2) {
-                pz = a < S::P2 ? 0 : P - 1;
-                a %= S::P2;
-                py = a / P;
-                px = a % P;
-            } else if (a < 2 * S::P2 + 2 * P * B) {
-                a -= 2 * S::P2;
-                py = a < P * B ? 0 : P - 1;
-                a %= P * B;
-                pz = 1 + a / P;
-                px = a % P;
-            } else {
-                a -= 2 * S::P2 + 2 * P * B;
-                px = a < S::B2 ? 0 : P - 1;
-                a %= S::B2;
-                pz = 1 + a / B;
-                py = 1 + a % B;
-            }
-            const int p[3] = {px, py, pz};
-            int l[3], k = 0;
-            const int edge = s_edge[g];
-#pragma unroll
-            for (int c = 2; c >= 0; --c) {
-                const int n = p[c] == 0 ? 0 : (p[c] == P - 1 ? 2 : 1);
-                k = k * 3 + n;
-                // the neighbour's facing voxel, or the clamped one of this block's
-                l[c] = n == 1 ? p[c] - 1 : (n == 0 ? ((edge >> (2 * c)) & 1 ? 0 : B - 1) : ((edge >> (2 * c + 1)) & 1 ? B - 1 : 0));
-            }
-            const int own = s_own[g][k];
-            at[u] = (slot0 + g) * S::P3 + (pz * P + py) * P + px;
-            v[u] = own >= 0 ? __ldg(atlas + (int64_t)own * S::B3 + (l[2] * B + l[1]) * B + l[0]) : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int u = 0; u < kCells; ++u)
-            if (at[u] >= 0) patlas[at[u]] = v[u];
     }
     __syncthreads();
 
-    // 3. warp o: octant o's distance plane
-    const int o = warp;
-    const bool sx = o & 1, sy = o & 2, sz = o & 4;        // set: the cone runs towards lower coordinates
+    // 2. the octants' distance planes, two per warp (B = 64: one): o0 and, with VPL 1, the octant
+    // o0 + 2 whose cone runs towards lower y
+    const int o0 = S::OPW == 2 ? (warp & 1) | (warp & 2) << 1 : warp;
+    const bool sx = o0 & 1, sy = S::OPW == 2 || (o0 & 2), sz = o0 & 4;    // set: the cone runs towards lower coordinates
     const int bit = sx ? lane : 31 - lane;                // this lane's bit in a row's mask
     const int g = S::VPL == 1 ? bit / LX : 0;
     const uint32_t le = (2u << lane) - 1u, lt = le >> 1;
@@ -384,40 +358,73 @@ __global__ void __launch_bounds__(kPrepThreads, PrepShape<LGB>::kMinCtas) prep_b
     const int xb = S::VPL == 1 ? xa : xa ^ 1;
     uint32_t prev[B];
 #pragma unroll
-    for (int y = 0; y < B; ++y) prev[y] = S::VPL == 1 ? 255u : 0x00ff00ffu;
+    for (int y = 0; y < B; ++y) prev[y] = 0x00ff00ffu;
     const uint32_t* mask_a = s_mask[sx][0];
     const uint32_t* mask_b = s_mask[sx][S::VPL - 1];
-    uint8_t* out_a = s_slice[warp][g] + 1 + xa;
-    uint8_t* out_b = s_slice[warp][g] + 1 + xb;
+    const int oa = S::OPW == 2 ? o0 + 2 : o0;
+    uint8_t* out_a = s_slice[oa][g] + 1 + xa;
+    uint8_t* out_b = s_slice[o0][g] + 1 + xb;
 #pragma unroll 1
     for (int zi = 0; zi < B; ++zi) {
         const int z = sz ? zi : B - 1 - zi;
         if (sy) prep_slice<LGB, true>(prev, mask_a + z * B, mask_b + z * B, out_a, out_b, lane, own_le, lt);
         else prep_slice<LGB, false>(prev, mask_a + z * B, mask_b + z * B, out_a, out_b, lane, own_le, lt);
         __syncwarp();
-        // the x and then the y apron: 255, or outside the grid the voxel that they clamp to
-        for (int i = lane; i < S::NB * 2 * B; i += 32) {
-            const int gi = i / (2 * B), hi = i & 1, py = 1 + ((i % (2 * B)) >> 1);
-            uint8_t* sl = s_slice[warp][gi] + py * P;
-            sl[hi ? P - 1 : 0] = (s_edge[gi] >> hi) & 1 ? sl[hi ? B : 1] : (uint8_t)255;
-        }
-        __syncwarp();
-        for (int i = lane; i < S::NB * 2 * P; i += 32) {
-            const int gi = i / (2 * P), q = i % (2 * P), hi = q >= P, px = hi ? q - P : q;
-            uint8_t* sl = s_slice[warp][gi];
-            sl[(hi ? P - 1 : 0) * P + px] = (s_edge[gi] >> (2 + hi)) & 1 ? sl[(hi ? B : 1) * P + px] : (uint8_t)255;
-        }
-        __syncwarp();
-        // the slice goes out in words (P^2 and P^3 are multiples of 4), and once more where it
-        // is beside the z apron: there as 255, or outside the grid as it is
-        for (int i = lane; i < S::NB * (S::P2 / 4); i += 32) {
-            const int gi = i / (S::P2 / 4), q = i % (S::P2 / 4);
-            if (slot0 + gi >= nb) break;
-            const uint32_t w = reinterpret_cast<const uint32_t*>(s_slice[warp][gi])[q];
-            uint32_t* d = reinterpret_cast<uint32_t*>(vskip + ((int64_t)o * nb + slot0 + gi) * S::P3 + (z + 1) * S::P2) + q;
-            *d = w;
-            if (z == 0) d[-(S::P2 / 4)] = (s_edge[gi] & 16) ? w : 0xffffffffu;
-            if (z == B - 1) d[S::P2 / 4] = (s_edge[gi] & 32) ? w : 0xffffffffu;
+#pragma unroll
+        for (int p = 0; p < S::OPW; ++p) {
+            const int o = o0 + 2 * p;
+            uint32_t* plane = reinterpret_cast<uint32_t*>(vskip + ((int64_t)o * nb + slot0) * S::P3) + (z + 1) * (S::P2 / 4);
+            if constexpr (S::NB == 1) {
+                // the x and then the y apron: 255, or outside the grid the voxel that they clamp to
+                const int edge = s_edge[0];
+                uint8_t* sl = s_slice[o][0];
+#pragma unroll
+                for (int q = 0; q < S::VPL; ++q) {
+                    uint8_t* row = sl + (1 + lane + 32 * q) * P;
+                    row[0] = (edge & 1) ? row[1] : (uint8_t)255;
+                    row[P - 1] = (edge & 2) ? row[B] : (uint8_t)255;
+                }
+                __syncwarp();
+                for (int px = lane; px < P; px += 32) {
+                    sl[px] = (edge & 4) ? sl[P + px] : (uint8_t)255;
+                    sl[(P - 1) * P + px] = (edge & 8) ? sl[B * P + px] : (uint8_t)255;
+                }
+                __syncwarp();
+                // the slice goes out in words (P^2 and P^3 are multiples of 4), and once more where
+                // it is beside the z apron: there as 255, or outside the grid as it is
+                const uint32_t* w = reinterpret_cast<const uint32_t*>(sl);
+#pragma unroll
+                for (int i = 0; i < S::P2 / 4 / 32; ++i) plane[lane + 32 * i] = w[lane + 32 * i];
+                if (lane < S::P2 / 4 % 32) plane[lane + S::P2 / 4 / 32 * 32] = w[lane + S::P2 / 4 / 32 * 32];
+                if (z == 0 || z == B - 1)
+                    for (int i = lane; i < S::P2 / 4; i += 32) {
+                        if (z == 0) plane[i - S::P2 / 4] = (edge & 16) ? w[i] : 0xffffffffu;
+                        if (z == B - 1) plane[i + S::P2 / 4] = (edge & 32) ? w[i] : 0xffffffffu;
+                    }
+            } else {
+                // the same for the blocks beside one another
+                for (int i = lane; i < S::NB * 2 * B; i += 32) {
+                    const int gi = i / (2 * B), hi = i & 1, py = 1 + ((i % (2 * B)) >> 1);
+                    uint8_t* sl = s_slice[o][gi] + py * P;
+                    sl[hi ? P - 1 : 0] = (s_edge[gi] >> hi) & 1 ? sl[hi ? B : 1] : (uint8_t)255;
+                }
+                __syncwarp();
+                for (int i = lane; i < S::NB * 2 * P; i += 32) {
+                    const int gi = i / (2 * P), q = i % (2 * P), hi = q >= P, px = hi ? q - P : q;
+                    uint8_t* sl = s_slice[o][gi];
+                    sl[(hi ? P - 1 : 0) * P + px] = (s_edge[gi] >> (2 + hi)) & 1 ? sl[(hi ? B : 1) * P + px] : (uint8_t)255;
+                }
+                __syncwarp();
+                for (int i = lane; i < S::NB * (S::P2 / 4); i += 32) {
+                    const int gi = i / (S::P2 / 4), q = i % (S::P2 / 4);
+                    if (slot0 + gi >= nb) break;
+                    const uint32_t w = reinterpret_cast<const uint32_t*>(s_slice[o][gi])[q];
+                    uint32_t* d = plane + (int64_t)gi * (S::P3 / 4) + q;
+                    *d = w;
+                    if (z == 0) d[-(S::P2 / 4)] = (s_edge[gi] & 16) ? w : 0xffffffffu;
+                    if (z == B - 1) d[S::P2 / 4] = (s_edge[gi] & 32) ? w : 0xffffffffu;
+                }
+            }
         }
         __syncwarp();
     }
@@ -546,7 +553,7 @@ static cudaError_t prep_blocks(const int32_t* ind, const int32_t* blk_of_slot, c
                                                    smem);
         if (e != cudaSuccess) return e;
     }
-    prep_blocks_kernel<LGB><<<(unsigned)((nb + n - 1) / n), kPrepThreads, smem, st>>>(
+    prep_blocks_kernel<LGB><<<(unsigned)((nb + n - 1) / n), PrepShape<LGB>::kThreads, smem, st>>>(
         ind, blk_of_slot, err, reinterpret_cast<const uint2*>(atlas), nb, G, patlas, vskip);
     return cudaGetLastError();
 }
