@@ -406,6 +406,13 @@ snerg_status snerg_bake(const snerg_scene_desc* desc, const snerg_bake_field* fi
                         int32_t* d_indirection, uint8_t* d_atlas, int64_t max_blocks,
                         void* d_workspace, size_t ws_bytes, int64_t* num_blocks, void* stream);
 
+/* The second half of a bake whose first call had no room: writes the atlas of the *num_blocks
+ * blocks that snerg_bake (SNERG_E_NOMEM, with its d_indirection complete) found, without
+ * looking for them again. d_workspace as that call left it, desc and field the same; num_blocks
+ * of the blocks, in slot order, are written. SYNCHRONISES `stream`. */
+snerg_status snerg_bake_atlas(const snerg_scene_desc* desc, const snerg_bake_field* field, uint8_t* d_atlas,
+                              int64_t num_blocks, const void* d_workspace, size_t ws_bytes, void* stream);
+
 /* SYNCHRONISES `stream`, returns and clears the device status word (SNERG_OK or the
  * first device error recorded since the last call); SNERG_E_DEVICE_FAULT if the stream
  * reports a sticky device fault (the context is unusable afterwards), SNERG_E_CUDA for

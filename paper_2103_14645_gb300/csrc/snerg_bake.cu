@@ -746,23 +746,15 @@ extern "C" size_t snerg_bake_workspace_bytes(const snerg_scene_desc* desc) {
     return ws_layout(G * G * G).total;
 }
 
-extern "C" snerg_status snerg_bake(const snerg_scene_desc* desc, const snerg_bake_field* field,
-                                   int32_t* d_indirection, uint8_t* d_atlas, int64_t max_blocks, void* d_workspace,
-                                   size_t ws_bytes, int64_t* num_blocks, void* stream) {
-    if (!desc_ok(desc) || !field_ok(field) || !d_indirection || !num_blocks || max_blocks < 0) return SNERG_E_INVAL;
-    if (max_blocks > 0 && (!d_atlas || ((uintptr_t)d_atlas & 7u))) return SNERG_E_INVAL;
-    if (!d_workspace || ((uintptr_t)d_workspace & (kAlign - 1))) return SNERG_E_INVAL;
-    const int64_t G = desc->N / desc->B, G3 = G * G * G;
-    const WsLayout L = ws_layout(G3);
-    if (ws_bytes < L.total) return SNERG_E_NOMEM;
-    *num_blocks = 0;
+namespace bake_gpu {
 
+BakeParams make_params(const snerg_scene_desc* desc, const snerg_bake_field* field) {
     BakeParams P;
     std::memset(&P, 0, sizeof(P));
     P.N = desc->N;
     P.B = desc->B;
     P.lgB = ilog2_exact(desc->B);
-    P.G = (int32_t)G;
+    P.G = desc->N / desc->B;
     P.n_blob = field->n_blob;
     const int B3 = desc->B * desc->B * desc->B;
     P.item_voxels = B3 < kThreads ? B3 : kThreads;
@@ -814,7 +806,23 @@ extern "C" snerg_status snerg_bake(const snerg_scene_desc* desc, const snerg_bak
         P.cbar[c] = (float)(cs / 16.0);
         P.sbar[c] = (float)(sn / 16.0);
     }
+    return P;
+}
 
+}  // namespace bake_gpu
+
+extern "C" snerg_status snerg_bake(const snerg_scene_desc* desc, const snerg_bake_field* field,
+                                   int32_t* d_indirection, uint8_t* d_atlas, int64_t max_blocks, void* d_workspace,
+                                   size_t ws_bytes, int64_t* num_blocks, void* stream) {
+    if (!desc_ok(desc) || !field_ok(field) || !d_indirection || !num_blocks || max_blocks < 0) return SNERG_E_INVAL;
+    if (max_blocks > 0 && (!d_atlas || ((uintptr_t)d_atlas & 7u))) return SNERG_E_INVAL;
+    if (!d_workspace || ((uintptr_t)d_workspace & (kAlign - 1))) return SNERG_E_INVAL;
+    const int64_t G = desc->N / desc->B, G3 = G * G * G;
+    const WsLayout L = ws_layout(G3);
+    if (ws_bytes < L.total) return SNERG_E_NOMEM;
+    *num_blocks = 0;
+
+    const BakeParams P = make_params(desc, field);
     cudaStream_t st = (cudaStream_t)stream;
     uint8_t* ws = (uint8_t*)d_workspace;
     int64_t* d_count = (int64_t*)(ws + L.count);
@@ -841,4 +849,22 @@ extern "C" snerg_status snerg_bake(const snerg_scene_desc* desc, const snerg_bak
         if (e != cudaSuccess) return SNERG_E_CUDA;
     }
     return SNERG_OK;
+}
+
+extern "C" snerg_status snerg_bake_atlas(const snerg_scene_desc* desc, const snerg_bake_field* field, uint8_t* d_atlas,
+                                         int64_t num_blocks, const void* d_workspace, size_t ws_bytes, void* stream) {
+    if (!desc_ok(desc) || !field_ok(field) || num_blocks < 0) return SNERG_E_INVAL;
+    if (num_blocks > 0 && (!d_atlas || ((uintptr_t)d_atlas & 7u))) return SNERG_E_INVAL;
+    if (!d_workspace || ((uintptr_t)d_workspace & (kAlign - 1))) return SNERG_E_INVAL;
+    const int64_t G = desc->N / desc->B;
+    const WsLayout L = ws_layout(G * G * G);
+    if (ws_bytes < L.total) return SNERG_E_NOMEM;
+    if (num_blocks == 0) return SNERG_OK;
+    if (num_blocks > G * G * G) return SNERG_E_INVAL;
+    cudaStream_t st = (cudaStream_t)stream;
+    const uint8_t* ws = (const uint8_t*)d_workspace;
+    cudaError_t e = launch_fill(make_params(desc, field), (const int32_t*)(ws + L.list), (const int64_t*)(ws + L.count),
+                                num_blocks, num_blocks, (uint2*)d_atlas, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e == cudaSuccess ? SNERG_OK : SNERG_E_CUDA;
 }

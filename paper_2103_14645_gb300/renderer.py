@@ -30,7 +30,7 @@ STATUS = {0: "ok", 1: "invalid argument", 2: "buffer too small", 3: "CUDA error"
 EXPORTED = ["snerg_workspace_bytes", "snerg_create", "snerg_render", "snerg_render_rays",
             "snerg_render_backward", "snerg_last_status", "snerg_launch_count",
             "snerg_persistent_config", "snerg_destroy", "snerg_status_str", "snerg_render_rays_noalloc",
-            "snerg_set_mlp", "snerg_l2_loss", "snerg_adam_step", "snerg_bake_workspace_bytes", "snerg_bake",
+            "snerg_set_mlp", "snerg_l2_loss", "snerg_adam_step", "snerg_bake_workspace_bytes", "snerg_bake", "snerg_bake_atlas",
             "snerg_requantize_atlas", "snerg_adam_requantize_atlas", "snerg_grad_blocks_touched", "snerg_grad_blocks_gather",
             "snerg_grad_blocks_scatter", "snerg_render_to_host", "snerg_train_rays", "snerg_schedule_stats",
             "snerg_state_bytes", "snerg_render_rays_recorded", "snerg_render_backward_recorded"]
@@ -131,6 +131,8 @@ def load_library(path: str = LIB_PATH):
     lib.snerg_bake_workspace_bytes.restype = ctypes.c_size_t
     lib.snerg_bake.argtypes = [P, P, P, P, i64, P, ctypes.c_size_t, P, P]
     lib.snerg_bake.restype = ctypes.c_int
+    lib.snerg_bake_atlas.argtypes = [P, P, P, i64, P, ctypes.c_size_t, P]
+    lib.snerg_bake_atlas.restype = ctypes.c_int
     _LIB = lib
     return lib
 
@@ -676,7 +678,7 @@ def bake(N: int, B: int, bmin, extent: float, sigma_max: float, field: BakeField
          max_blocks: int | None = None, flags: int = 0):
     """Bake an analytic field into (indirection int32 [G,G,G], atlas uint8 [nb,B,B,B,8]) on
     the GPU with snerg_bake (Sec. 5.3-5.4). With max_blocks None the atlas is sized by a
-    first call that only counts the kept blocks. flags = FLAG_ALPHA_ATLAS stores alpha
+    first call that only finds the kept blocks, and written by snerg_bake_atlas. flags = FLAG_ALPHA_ATLAS stores alpha
     codes in channel 0."""
     lib = load_library()
     device = torch.device(device)
@@ -698,9 +700,11 @@ def bake(N: int, B: int, bmin, extent: float, sigma_max: float, field: BakeField
                                   ctypes.byref(nb), st)
             if code not in (0, 2):
                 _check(code, "snerg_bake")
-            max_blocks = nb.value
-        atlas = torch.empty((max_blocks, B, B, B, 8), dtype=torch.uint8, device=device)
-        code = lib.snerg_bake(ctypes.byref(desc), ctypes.byref(field), _ptr(ind), _ptr(atlas) if max_blocks else None,
-                              int(max_blocks), _ptr(ws), nbytes, ctypes.byref(nb), st)
+            atlas = torch.empty((nb.value, B, B, B, 8), dtype=torch.uint8, device=device)
+            code = lib.snerg_bake_atlas(ctypes.byref(desc), ctypes.byref(field), _ptr(atlas), nb, _ptr(ws), nbytes, st)
+        else:
+            atlas = torch.empty((max_blocks, B, B, B, 8), dtype=torch.uint8, device=device)
+            code = lib.snerg_bake(ctypes.byref(desc), ctypes.byref(field), _ptr(ind), _ptr(atlas) if max_blocks else None,
+                                  int(max_blocks), _ptr(ws), nbytes, ctypes.byref(nb), st)
     _check(code, "snerg_bake")
     return ind, atlas[:nb.value]

@@ -38,3 +38,14 @@ def test_blobs_below_the_threshold_keep_nothing():
     field = renderer.bake_field(f["blobs"], f["colors"], f["jitter"], TAU)
     ind, atl = renderer.bake(64, 16, BMIN, EXTENT, 10.0, field, DEV)
     assert bool((ind == -1).all()) and atl.shape[0] == 0
+
+
+def test_atlas_of_a_counted_bake():
+    """max_blocks None counts first and then only writes the atlas: the same scene as one call
+    with room, for blocks on both sides of 8^3."""
+    for N, B in ((64, 4), (64, 8), (96, 32)):
+        f = synth.analytic_field(N, n_blob=12, std=(0.05, 0.1), peak=(20.0, 80.0))
+        field = renderer.bake_field(f["blobs"], f["colors"], f["jitter"], TAU)
+        ind, atl = renderer.bake(N, B, BMIN, EXTENT, 100.0, field, DEV)
+        ind1, atl1 = renderer.bake(N, B, BMIN, EXTENT, 100.0, field, DEV, max_blocks=atl.shape[0] + 3)
+        assert atl.shape[0] > 0 and bool((ind == ind1).all()) and bool((atl == atl1).all())
