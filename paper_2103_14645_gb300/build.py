@@ -1,6 +1,7 @@
 """Build the in-tree renderer library libsnerg.so for sm_103a with nvcc.
 
-Each translation unit compiles in parallel into _build/, then nvcc links the shared
+Each translation unit compiles in parallel into _build/ (the kernels of the march once per
+block build), then nvcc links the shared
 library next to this file. Only the sm_103a target is emitted (one -gencode).
 """
 from __future__ import annotations
@@ -16,8 +17,12 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libsnerg.so")
-SOURCES = ["snerg_api.cu", "snerg_fwd.cu", "snerg_bwd.cu", "snerg_prep.cu", "snerg_noalloc.cu", "snerg_train.cu",
-           "snerg_bake.cu"]
+SOURCES = ["snerg_api.cu", "snerg_prep.cu", "snerg_noalloc.cu", "snerg_train.cu", "snerg_bake.cu"]
+# compiled once per block build: log2 of the block edge as a constant (0: any edge), and whether
+# channel 0 holds alpha (2: by the scene's flags)
+PER_BLOCK_SOURCES = ["snerg_fwd.cu", "snerg_bwd.cu"]
+BLOCK_BUILDS = [(0, 2)] + [(lgb, alpha) for lgb in (3, 4, 5, 6) for alpha in (0, 1)]
+UNITS = [(f, b) for f in PER_BLOCK_SOURCES for b in BLOCK_BUILDS] + [(f, None) for f in SOURCES]
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -33,9 +38,11 @@ def _flags(extra=()):
             "-I", INCLUDE, "-I", CSRC, *extra]
 
 
-def _compile(src: str, extra, verbose: bool) -> str:
-    obj = os.path.join(BUILD, os.path.splitext(src)[0] + ".o")
-    cmd = [nvcc(), *_flags(extra), "-c", os.path.join(CSRC, src), "-o", obj]
+def _compile(unit, extra, verbose: bool) -> str:
+    src, block = unit
+    obj = os.path.join(BUILD, os.path.splitext(src)[0] + ("" if block is None else "_%d_%d" % block) + ".o")
+    define = [] if block is None else ["-DSNERG_LGB=%d" % block[0], "-DSNERG_ALPHA=%d" % block[1]]
+    cmd = [nvcc(), *_flags(extra), *define, "-c", os.path.join(CSRC, src), "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if verbose or r.returncode:
         sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
@@ -46,8 +53,8 @@ def _compile(src: str, extra, verbose: bool) -> str:
 
 def build(verbose: bool = False, extra=()) -> str:
     os.makedirs(BUILD, exist_ok=True)
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(lambda s: _compile(s, extra, verbose), SOURCES))
+    with cf.ThreadPoolExecutor(max_workers=os.cpu_count() or 4) as ex:
+        objs = list(ex.map(lambda u: _compile(u, extra, verbose), UNITS))
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc(), *GENCODE, "-shared", "-cudart", "static", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)

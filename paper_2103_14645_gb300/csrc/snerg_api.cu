@@ -224,10 +224,24 @@ extern "C" snerg_status snerg_create(const snerg_scene_desc* desc, const int32_t
 }
 
 namespace snerg {
-// snerg_bwd.cu: one fine-tuning step per ray (render, L2 loss and adjoint in one launch)
-cudaError_t launch_train_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
-                              const float* mlp, const float* target, float* rgb_out, float* loss, float* grad_atlas,
-                              float* grad_mlp, cudaStream_t st);
+// debug outputs and the per-sample model are in build 0
+cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
+                                float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1,
+                                const SchedArgs* sch) {
+    row0 = std::max(row0, 0);
+    row1 = std::min(row1, cam.H);
+    if (cam.W <= 0 || row1 <= row0) return cudaSuccess;
+    if (dbg.aux || dbg.counts || dbg.trace || (s.flags & SNERG_FLAG_PER_SAMPLE_MLP))
+        return Forward<0, kAnyAlpha>::image(s, cam, mlp, pw, rgb, dbg, st, row0, row1, nullptr);
+    return with_block_build(s, [&](auto b) {
+        return Forward<decltype(b)::lgB, decltype(b)::alpha>::image(s, cam, mlp, pw, rgb, dbg, st, row0, row1, sch);
+    });
+}
+
+static const void* persistent_fn(const DevScene& s, bool param_weights, bool multi) {
+    return with_block_build(s, [&](auto b) { return Forward<decltype(b)::lgB, decltype(b)::alpha>::persistent_fn(param_weights, multi); });
+}
+
 // snerg_prep.cu; adam: nullable, an optimiser step on the values first (m, v, g)
 cudaError_t launch_requantize(const int32_t* ind, const int32_t* blk_of_slot, float* values, float* m, float* v,
                               const float* g, const AdamArgs* adam, int64_t nb, int N, int B, int lgB, uint2* patlas,
@@ -305,13 +319,21 @@ static void fill_params(PersistentParams& p, const snerg_camera* cams, int32_t n
     p.total_items = acc;
 }
 
+static cudaError_t launch_persistent(const DevScene& s, const PersistentParams& p, const float* mlp, const MlpWeights* pw,
+                                     float* rgb, int32_t* queue, int grid, int block, cudaStream_t st) {
+    const bool multi = p.tile_w != p.warp_w || p.tile_h != p.warp_h;
+    const MlpWeights& w = pw ? *pw : no_weights();
+    void* args[] = {(void*)&s, (void*)&p, (void*)&mlp, (void*)&w, (void*)&rgb, (void*)&queue};
+    return cudaLaunchKernel(persistent_fn(s, pw != nullptr, multi), dim3(grid), dim3(block), args, 0, st);
+}
+
 static cudaError_t launch_persistent_direct(snerg_scene* h, const PersistentParams& p, const PersistentConfig& c,
                                             const float* mlp, const MlpWeights* pw, float* rgb, cudaStream_t st) {
     int32_t* queue = h->hdr + kHdrQueue;
     cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     h->launches++;
-    return launch_render_persistent(h->ds, p, mlp, pw, rgb, queue, h->num_sms * c.ctas_per_sm, c.block, st);
+    return launch_persistent(h->ds, p, mlp, pw, rgb, queue, h->num_sms * c.ctas_per_sm, c.block, st);
 }
 
 // Work items of one warp pass only: items of several passes (the kernel build with a pass
@@ -390,7 +412,7 @@ static snerg_status render_persistent(snerg_scene* h, const snerg_camera* cams, 
         if (e == cudaSuccess) e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             cudaMemsetAsync(queue, 0, sizeof(int32_t), h->cap_stream);
-            launch_render_persistent(h->ds, *p, mlp, pw, rgb, queue, grid, cfg.block, h->cap_stream);
+            launch_persistent(h->ds, *p, mlp, pw, rgb, queue, grid, cfg.block, h->cap_stream);
             e = cudaStreamEndCapture(h->cap_stream, &ge.graph);
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ge.exec, ge.graph, 0);
@@ -418,11 +440,10 @@ static snerg_status render_persistent(snerg_scene* h, const snerg_camera* cams, 
     DevScene ds = h->ds;
     const float* mlp_arg = mlp;
     float* rgb_arg = rgb;
-    static const MlpWeights zero_w = {};
-    const MlpWeights* w_arg = pw ? pw : &zero_w;
+    const MlpWeights* w_arg = pw ? pw : &no_weights();
     void* args[] = {(void*)&ds, (void*)p, (void*)&mlp_arg, (void*)w_arg, (void*)&rgb_arg, (void*)&queue};
     cudaKernelNodeParams kp = {};
-    kp.func = const_cast<void*>(persistent_kernel_fn(pw != nullptr, cfg.passes > 1));
+    kp.func = const_cast<void*>(persistent_fn(ds, pw != nullptr, cfg.passes > 1));
     kp.gridDim = dim3(grid);
     kp.blockDim = dim3(cfg.block);
     kp.sharedMemBytes = 0;
@@ -591,8 +612,13 @@ static snerg_status render_rays(snerg_handle h, const snerg_camera* cams, int32_
     if (!make_table(cams, n_cams, t)) { delete t; return SNERG_E_INVAL; }
     if (n == 0) { delete t; return SNERG_OK; }
     if (!d_pix || !d_rgb || (!d_mlp && !h->has_w)) { delete t; return SNERG_E_INVAL; }
-    cudaError_t e = launch_render_rays(h->ds, *t, n_cams, d_pix, n, d_mlp, d_mlp ? nullptr : &h->host_w, d_rgb, dbg, record,
-                                       st);
+    const MlpWeights* pw = d_mlp ? nullptr : &h->host_w;
+    const bool debug = !record && (dbg.aux || dbg.counts || dbg.trace);      // in build 0
+    const cudaError_t e = debug ? Forward<0, kAnyAlpha>::rays(h->ds, *t, n_cams, d_pix, n, d_mlp, pw, d_rgb, dbg, nullptr, st)
+                                : with_block_build(h->ds, [&](auto b) {
+                                      return Forward<decltype(b)::lgB, decltype(b)::alpha>::rays(h->ds, *t, n_cams, d_pix, n, d_mlp, pw,
+                                                                                 d_rgb, dbg, record, st);
+                                  });
     delete t;
     if (e != cudaSuccess) return SNERG_E_CUDA;
     h->launches++;
@@ -646,8 +672,10 @@ static snerg_status render_backward(snerg_handle h, const snerg_camera* cams, in
     if (!d_pix || !d_mlp || !d_grad_rgb) { delete t; return SNERG_E_INVAL; }
     if (d_grad_atlas && ((uintptr_t)d_grad_atlas & 15u)) { delete t; return SNERG_E_INVAL; }
     if ((d_fwd_aux == nullptr) != (d_fwd_counts == nullptr)) { delete t; return SNERG_E_INVAL; }
-    cudaError_t e = launch_backward_rays(h->ds, *t, n_cams, d_pix, n, d_mlp, d_grad_rgb, d_fwd_aux, d_fwd_counts, record,
-                                         d_grad_atlas, d_grad_mlp, st);
+    const cudaError_t e = with_block_build(h->ds, [&](auto b) {
+        return Adjoint<decltype(b)::lgB, decltype(b)::alpha>::backward(h->ds, *t, n_cams, d_pix, n, d_mlp, d_grad_rgb, d_fwd_aux,
+                                                       d_fwd_counts, record, d_grad_atlas, d_grad_mlp, st);
+    });
     delete t;
     if (e != cudaSuccess) return SNERG_E_CUDA;
     h->launches++;
@@ -693,8 +721,10 @@ extern "C" snerg_status snerg_train_rays(snerg_handle h, const snerg_camera* cam
     if (n == 0) { delete t; return SNERG_OK; }
     if (!d_pix || !d_mlp || !d_target) { delete t; return SNERG_E_INVAL; }
     if (d_grad_atlas && ((uintptr_t)d_grad_atlas & 15u)) { delete t; return SNERG_E_INVAL; }
-    cudaError_t e = launch_train_rays(h->ds, *t, n_cams, d_pix, n, d_mlp, d_target, d_rgb, d_loss, d_grad_atlas,
-                                      d_grad_mlp, (cudaStream_t)stream);
+    const cudaError_t e = with_block_build(h->ds, [&](auto b) {
+        return Adjoint<decltype(b)::lgB, decltype(b)::alpha>::train(h->ds, *t, n_cams, d_pix, n, d_mlp, d_target, d_rgb, d_loss,
+                                                    d_grad_atlas, d_grad_mlp, (cudaStream_t)stream);
+    });
     delete t;
     if (e != cudaSuccess) return SNERG_E_CUDA;
     h->launches++;

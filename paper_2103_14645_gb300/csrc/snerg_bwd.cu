@@ -11,9 +11,15 @@
 // ray that composited more. MLP weight gradients are
 // summed over the CTA's rays from activations staged in shared memory and reach global
 // memory with one atomic per parameter per CTA.
+//
+// Compiled once per block build (BlockScene): SNERG_LGB and SNERG_ALPHA are the build's LGB and A.
 #include <atomic>
 
 #include "snerg_internal.cuh"
+
+#if !defined(SNERG_LGB) || !defined(SNERG_ALPHA)
+#error "SNERG_LGB: log2 of the block edge of this build, 0 for any; SNERG_ALPHA: 0, 1 or 2 for any"
+#endif
 
 namespace snerg {
 
@@ -25,7 +31,7 @@ constexpr int kRowX = 0, kRowH1 = 34, kRowH2 = 50, kRowG1 = 66, kRowG2 = 82, kRo
 constexpr int kWFloats = 884;      // transposed weights (883) rounded up to a 16-byte multiple
 constexpr int kMaxDevices = 64;     // devices whose shared-memory opt-in is remembered
 
-size_t backward_smem_bytes(int lanes) { return (size_t)(kWFloats + kBwdThreads / 32 * lanes * kRow) * sizeof(float); }
+static size_t backward_smem_bytes(int lanes) { return (size_t)(kWFloats + kBwdThreads / 32 * lanes * kRow) * sizeof(float); }
 
 // A recorded sample's lattice position, block origin (minus one), block slot and weight.
 struct RecSample {
@@ -34,7 +40,8 @@ struct RecSample {
     int slot;
 };
 
-__device__ __forceinline__ void locate_recorded(const DevScene& s, const Ray& r, const int32_t* ind, float2 e,
+template <class SC>
+__device__ __forceinline__ void locate_recorded(const SC& s, const Ray& r, const int32_t* ind, float2 e,
                                                 int& bprev, int& slot, RecSample& x) {
     const float t = lattice_t(r, e.x);
     int b[3];
@@ -61,7 +68,8 @@ __device__ __forceinline__ void locate_recorded(const DevScene& s, const Ray& r,
 // slot loaded) before the current one's atomics, so that those loads overlap them. T and
 // tau after the kRecCap-th sample (rec[kRecCap]) go to st for a march that continues from
 // the next lattice index (CONT).
-__device__ __forceinline__ void scatter_recorded(const DevScene& s, const Ray& r, const float2* rec, int64_t stride,
+template <class SC>
+__device__ __forceinline__ void scatter_recorded(const SC& s, const Ray& r, const float2* rec, int64_t stride,
                                                  int n, const float* gfeat, float* grad_atlas, MarchState& st) {
     if (n > 0) {
         const int oct = (r.d[0] < 0.0f ? 1 : 0) | (r.d[1] < 0.0f ? 2 : 0) | (r.d[2] < 0.0f ? 4 : 0);
@@ -250,9 +258,9 @@ __device__ __forceinline__ void dphi_sums(const float* rows, int n_rows, float* 
 // MLP give C, the L2 loss |C - C*|^2 is accumulated into *loss, dL/dC = 2 (C - C*) is taken
 // in the kernel, and the adjoint follows as for a given upstream gradient; C goes to
 // rgb_out (nullable). grad_rgb, fwd_aux and fwd_counts are not used.
-template <bool TRAIN, bool STATE, bool RECORDED = false>
+template <int LGB, int A, bool TRAIN, bool STATE, bool RECORDED = false>
 __global__ void __launch_bounds__(kBwdThreads, 4) backward_rays_kernel(
-    const DevScene s, const __grid_constant__ CamTable cams, int32_t n_cams, const int32_t* __restrict__ pix,
+    const BlockScene<LGB, A> s, const __grid_constant__ CamTable cams, int32_t n_cams, const int32_t* __restrict__ pix,
     int64_t n, const float* __restrict__ mlp, const float* __restrict__ grad_rgb,
     const float* __restrict__ fwd_aux, const int32_t* __restrict__ fwd_counts, const float2* __restrict__ record,
     const float* __restrict__ target, float* __restrict__ rgb_out, float* __restrict__ loss, float* __restrict__ grad_atlas,
@@ -408,7 +416,7 @@ __global__ void __launch_bounds__(kBwdThreads, 4) backward_rays_kernel(
     if (grad_mlp) dphi_sums(rows, kBwdThreads / 32 * lanes, grad_mlp);
 }
 
-template <bool TRAIN, bool STATE, bool RECORDED = false>
+template <int LGB, int A, bool TRAIN, bool STATE, bool RECORDED = false>
 static cudaError_t backward_launch(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
                                    int64_t n, const float* mlp, const float* grad_rgb, const float* fwd_aux,
                                    const int32_t* fwd_counts, const float2* record, const float* target, float* rgb_out, float* loss,
@@ -425,38 +433,39 @@ static cudaError_t backward_launch(const DevScene& s, const CamTable& cams, int3
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!attr_set[dev].load()) {
-        e = cudaFuncSetAttribute(backward_rays_kernel<TRAIN, STATE, RECORDED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(backward_rays_kernel<LGB, A, TRAIN, STATE, RECORDED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)backward_smem_bytes(32));
         if (e != cudaSuccess) return e;
         attr_set[dev].store(true);
     }
     const int rays = kBwdThreads / 32 * lanes;          // per CTA
     const unsigned grid = (unsigned)((n + rays - 1) / rays);
-    backward_rays_kernel<TRAIN, STATE, RECORDED><<<grid, kBwdThreads, smem, st>>>(
-        s, cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, record, target, rgb_out, loss, grad_atlas, grad_mlp,
+    backward_rays_kernel<LGB, A, TRAIN, STATE, RECORDED><<<grid, kBwdThreads, smem, st>>>(
+        BlockScene<LGB, A>(s), cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, record, target, rgb_out, loss, grad_atlas, grad_mlp,
         lanes);
     return cudaGetLastError();
 }
 
-cudaError_t launch_backward_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
-                                 int64_t n, const float* mlp, const float* grad_rgb, const float* fwd_aux,
-                                 const int32_t* fwd_counts, const float2* record, float* grad_atlas, float* grad_mlp,
-                                 cudaStream_t st) {
-    if (fwd_aux && record)
-        return backward_launch<false, true, true>(s, cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, record,
-                                                  nullptr, nullptr, nullptr, grad_atlas, grad_mlp, st);
-    if (fwd_aux)
-        return backward_launch<false, true>(s, cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, nullptr, nullptr,
-                                            nullptr, nullptr, grad_atlas, grad_mlp, st);
-    return backward_launch<false, false>(s, cams, n_cams, pix, n, mlp, grad_rgb, nullptr, nullptr, nullptr, nullptr,
-                                         nullptr, nullptr, grad_atlas, grad_mlp, st);
+template <int LGB, int A>
+cudaError_t Adjoint<LGB, A>::backward(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
+                                   const float* mlp, const float* grad_rgb, const float* fwd_aux,
+                                   const int32_t* fwd_counts, const float2* record, float* grad_atlas, float* grad_mlp,
+                                   cudaStream_t st) {
+    auto* launch = fwd_aux && record ? backward_launch<LGB, A, false, true, true>
+                   : fwd_aux         ? backward_launch<LGB, A, false, true>
+                                     : backward_launch<LGB, A, false, false>;
+    return launch(s, cams, n_cams, pix, n, mlp, grad_rgb, fwd_aux, fwd_counts, record, nullptr, nullptr, nullptr, grad_atlas,
+                  grad_mlp, st);
 }
 
-cudaError_t launch_train_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
-                              const float* mlp, const float* target, float* rgb_out, float* loss, float* grad_atlas,
-                              float* grad_mlp, cudaStream_t st) {
-    return backward_launch<true, false>(s, cams, n_cams, pix, n, mlp, nullptr, nullptr, nullptr, nullptr, target, rgb_out,
-                                        loss, grad_atlas, grad_mlp, st);
+template <int LGB, int A>
+cudaError_t Adjoint<LGB, A>::train(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
+                                const float* mlp, const float* target, float* rgb_out, float* loss, float* grad_atlas,
+                                float* grad_mlp, cudaStream_t st) {
+    return backward_launch<LGB, A, true, false>(s, cams, n_cams, pix, n, mlp, nullptr, nullptr, nullptr, nullptr, target,
+                                             rgb_out, loss, grad_atlas, grad_mlp, st);
 }
+
+template struct Adjoint<SNERG_LGB, SNERG_ALPHA>;
 
 }  // namespace snerg

@@ -6,7 +6,14 @@
 // reads the weights from the kernel parameter `pw` (constant-bank operands; set with
 // snerg_set_mlp), PW = false stages them from device memory into shared memory (the
 // form the autograd path uses, where the weights live in a tensor).
+//
+// Compiled once per block build (BlockScene): SNERG_LGB and SNERG_ALPHA are the build's LGB and A. Debug outputs and
+// the per-sample model are in build 0 only.
 #include "snerg_internal.cuh"
+
+#if !defined(SNERG_LGB) || !defined(SNERG_ALPHA)
+#error "SNERG_LGB: log2 of the block edge of this build, 0 for any; SNERG_ALPHA: 0, 1 or 2 for any"
+#endif
 
 namespace snerg {
 
@@ -15,14 +22,17 @@ namespace snerg {
 // small CTAs free their SM slot as soon as their own packets are done, which matters
 // because packets on the object take several times longer than background packets.
 //
-// L: rays per warp (the other lanes idle), see lanes_per_warp.
-template <int NW, int L = 32>
+// With fewer rays per warp (lanes, see lanes_per_warp) the packet shrinks to 4x4, 4x2, 2x2, 2x1
+// or one pixel, and the CTA's tile with it.
+template <int NW>
 struct ImageTile {
     static constexpr int WX = NW >= 2 ? 2 : 1;      // warps across
     static constexpr int WY = NW >= 4 ? 2 : 1;      // warps down
-    static constexpr int PX = L == 32 ? 8 : (L >= 8 ? 4 : (L >= 2 ? 2 : 1)), PY = L / PX;   // a warp's pixels
-    static constexpr int TW = PX * WX, TH = PY * WY;  // CTA tile in pixels
+    static constexpr int TW = 8 * WX, TH = 4 * WY;  // CTA tile in pixels
 };
+__host__ __device__ __forceinline__ int packet_width_log2(int lanes) {
+    return lanes == 32 ? 3 : (lanes >= 8 ? 2 : (lanes >= 2 ? 1 : 0));
+}
 
 // SCHED: the launch's CTAs take the image's tiles in the order of the previous frame's
 // cost buckets (slowest first). The slowest tiles -- those whose recorded cost is at least
@@ -132,8 +142,8 @@ __device__ __forceinline__ void sched_record(const SchedArgs& sch, const SchedSl
 }
 
 // one pixel of render_image_kernel: march, MLP, store (and the debug outputs)
-template <bool DBG, bool PS>
-__device__ __forceinline__ void image_pixel(const DevScene& s, const snerg_camera& cam, const float* sW,
+template <bool DBG, bool PS, class SC>
+__device__ __forceinline__ void image_pixel(const SC& s, const snerg_camera& cam, const float* sW,
                                             const MlpWeights* pwp, float* __restrict__ rgb, const DebugOut& dbg,
                                             int px, int py) {
     const Ray r = make_ray(s, cam, px, py);
@@ -163,19 +173,20 @@ __device__ __forceinline__ void image_pixel(const DevScene& s, const snerg_camer
     }
 }
 
-template <bool DBG, bool PW, int NW, bool PS, bool SCHED = false, int L = 32>
-__global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const DevScene s, const snerg_camera cam,
+template <int LGB, int A, bool DBG, bool PW, int NW, bool PS, bool SCHED = false>
+__global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const BlockScene<LGB, A> s, const snerg_camera cam,
                                                                         const float* __restrict__ mlp,
                                                                         const __grid_constant__ MlpWeights pw,
                                                                         float* __restrict__ rgb, const DebugOut dbg,
-                                                                        int row0, int row1, const SchedArgs sch) {
+                                                                        int row0, int row1, int lanes,
+                                                                        const SchedArgs sch) {
     __shared__ __align__(16) float sW[PW ? 4 : kNParam + 1];
     if (!PW) {
         load_mlp_smem_t(sW, mlp);
         __syncthreads();
     }
     const MlpWeights* pwp = PW ? &pw : nullptr;
-    using T = ImageTile<NW, L>;
+    using T = ImageTile<NW>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if constexpr (SCHED) {
         static_assert(NW == 4, "the sparse mapping assumes 16x8 tiles of four 8x4 warps");
@@ -203,9 +214,10 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const De
         }
         sched_record(sch, sl, &s_t0);
     } else {
-        const int px = blockIdx.x * T::TW + (warp % T::WX) * T::PX + lane % T::PX;
-        const int py = row0 + blockIdx.y * T::TH + (warp / T::WX) * T::PY + lane / T::PX;
-        if (lane >= L || px >= cam.W || py >= row1) return;
+        const int lgx = packet_width_log2(lanes), h = lanes >> lgx;      // a warp's packet: (1 << lgx) x h
+        const int px = (((int)blockIdx.x * T::WX + warp % T::WX) << lgx) + (lane & ((1 << lgx) - 1));
+        const int py = row0 + ((int)blockIdx.y * T::WY + warp / T::WX) * h + (lane >> lgx);
+        if (lane >= lanes || px >= cam.W || py >= row1) return;
         image_pixel<DBG, PS>(s, cam, sW, pwp, rgb, dbg, px, py);
     }
 }
@@ -213,8 +225,8 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const De
 // MINB: resident CTAs per SM the build is limited to (7: 72 registers; 4: up to 128);
 // lanes: rays per warp (the other lanes idle); REC: each ray's composited samples go to
 // record (entry j of ray i at record[j * n + i], see march) for the adjoint
-template <bool DBG, bool PW, int MINB, bool REC = false>
-__global__ void __launch_bounds__(128, MINB) render_rays_kernel(const DevScene s, const __grid_constant__ CamTable cams,
+template <int LGB, int A, bool DBG, bool PW, int MINB, bool REC = false>
+__global__ void __launch_bounds__(128, MINB) render_rays_kernel(const BlockScene<LGB, A> s, const __grid_constant__ CamTable cams,
                                                                 int32_t n_cams, const int32_t* __restrict__ pix,
                                                                 int64_t n, const float* __restrict__ mlp,
                                                                 const __grid_constant__ MlpWeights pw,
@@ -269,8 +281,8 @@ __global__ void __launch_bounds__(128, MINB) render_rays_kernel(const DevScene s
 // and renders each item in warp_w x warp_h packets of 32 rays. The counter is zeroed by
 // the launch sequence (a memset node of the captured graph) before every launch.
 // One pixel of the persistent launch: march, shade and store.
-template <bool PW>
-__device__ __forceinline__ void persistent_pixel(const DevScene& s, const snerg_camera& cam, const float* sW,
+template <bool PW, class SC>
+__device__ __forceinline__ void persistent_pixel(const SC& s, const snerg_camera& cam, const float* sW,
                                                  const MlpWeights& pw, float* rgb, int px, int py) {
     // the output row before the march, so that only it stays live across it
     float* out = rgb + (cam.out_offset + (int64_t)py * cam.W + px) * 3;
@@ -288,8 +300,8 @@ __device__ __forceinline__ void persistent_pixel(const DevScene& s, const snerg_
 // MULTI: a work item is several warp passes (tile_w x tile_h larger than warp_w x
 // warp_h); without it an item is exactly one warp pass and no pass loop stays live across
 // the march.
-template <bool PW, bool MULTI>
-__global__ void __launch_bounds__(128, 8) render_persistent_kernel(const DevScene s,
+template <int LGB, int A, bool PW, bool MULTI>
+__global__ void __launch_bounds__(128, 8) render_persistent_kernel(const BlockScene<LGB, A> s,
                                                                    const __grid_constant__ PersistentParams p,
                                                                    const float* __restrict__ mlp,
                                                                    const __grid_constant__ MlpWeights pw,
@@ -331,90 +343,46 @@ __global__ void __launch_bounds__(128, 8) render_persistent_kernel(const DevScen
     }
 }
 
-constexpr int kImageWarps = 4;     // warps per CTA of the one-camera launch
-
-static const MlpWeights& no_weights() {
-    static const MlpWeights z = {};
-    return z;
-}
-
-// Up to three waves of warps: 40,000 pixels of a 1024^3 grid take 202 us with 32 rays per warp,
-// 134 with 8 and 118 with 4 (2.1 waves); 160,000 take 201, 171 with 16 (2.1) and 164 with 8 (4.1),
-// but of a 512^3 grid 108, 102 and 111; from 470,000 on 32 is the best or within 5 % of it.
-int image_lanes(const DevScene& s, int64_t n) { return lanes_per_warp(n, (int64_t)s.sms * 8 * kImageWarps * 3); }
-
-template <int L>
-static void image_sparse(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
-                         float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1) {
-    using T = ImageTile<kImageWarps, L>;
-    const dim3 grid((cam.W + T::TW - 1) / T::TW, (row1 - row0 + T::TH - 1) / T::TH);
-    const SchedArgs none{nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 1};
-    const MlpWeights& w = pw ? *pw : no_weights();
-    if (pw)
-        render_image_kernel<false, true, kImageWarps, false, false, L><<<grid, 32 * kImageWarps, 0, st>>>(
-            s, cam, mlp, w, rgb, dbg, row0, row1, none);
-    else
-        render_image_kernel<false, false, kImageWarps, false, false, L><<<grid, 32 * kImageWarps, 0, st>>>(
-            s, cam, mlp, w, rgb, dbg, row0, row1, none);
-}
-
-template <bool PS>
-static void image_launch(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
-                         float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1, const SchedArgs* sch) {
-    using T = ImageTile<kImageWarps>;
-    dim3 grid((cam.W + T::TW - 1) / T::TW, (row1 - row0 + T::TH - 1) / T::TH);
-    const int nt = 32 * kImageWarps;
-    const bool d = dbg.aux || dbg.counts || dbg.trace;
-    const MlpWeights& w = pw ? *pw : no_weights();
-    const SchedArgs none{nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 1};
-    if (!PS && !d && !sch) {
-        switch (image_lanes(s, (int64_t)cam.W * (row1 - row0))) {
-            case 16: return image_sparse<16>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
-            case 8: return image_sparse<8>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
-            case 4: return image_sparse<4>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
-            case 2: return image_sparse<2>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
-            case 1: return image_sparse<1>(s, cam, mlp, pw, rgb, dbg, st, row0, row1);
-        }
-    }
-    if (!PS && !d && sch) {
-        const dim3 g1((unsigned)(sch->nt * sch->parts + 4 * sch->smax));   // 4 smax sparse slots, then nt dense ones
-        if (pw) render_image_kernel<false, true, kImageWarps, false, true><<<g1, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg,
-                                                                                            row0, row1, *sch);
-        else render_image_kernel<false, false, kImageWarps, false, true><<<g1, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg,
-                                                                                              row0, row1, *sch);
-        return;
-    }
-    if (pw) {
-        if (d) render_image_kernel<true, true, kImageWarps, PS><<<grid, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg, row0, row1, none);
-        else render_image_kernel<false, true, kImageWarps, PS><<<grid, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg, row0, row1, none);
-    } else {
-        if (d) render_image_kernel<true, false, kImageWarps, PS><<<grid, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg, row0, row1, none);
-        else render_image_kernel<false, false, kImageWarps, PS><<<grid, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg, row0, row1, none);
-    }
-}
-
-// rows [row0, row1) of the camera (clamped to [0, H]); all rows when row1 <= row0 after clamping
-cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
+// rows [row0, row1) of the camera
+template <int LGB, int A>
+cudaError_t Forward<LGB, A>::image(const DevScene& ds, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
                                 float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1,
                                 const SchedArgs* sch) {
-    row0 = max(row0, 0);
-    row1 = min(row1, cam.H);
-    if (cam.W <= 0 || row1 <= row0) return cudaSuccess;
-    if (s.flags & SNERG_FLAG_PER_SAMPLE_MLP) image_launch<true>(s, cam, mlp, pw, rgb, dbg, st, row0, row1, nullptr);
-    else image_launch<false>(s, cam, mlp, pw, rgb, dbg, st, row0, row1, sch);
+    using T = ImageTile<kImageWarps>;
+    const BlockScene<LGB, A> s(ds);
+    const int nt = 32 * kImageWarps;
+    const bool ps = (ds.flags & SNERG_FLAG_PER_SAMPLE_MLP) != 0, d = dbg.aux || dbg.counts || dbg.trace;
+    const MlpWeights& w = pw ? *pw : no_weights();
+    const SchedArgs none{nullptr, nullptr, nullptr, nullptr, 0, 0, 0, 0, 1};
+    if (sch && !ps && !d) {
+        // 4 smax sparse slots, then nt dense ones of `parts` CTAs
+        auto* kernel = pw ? render_image_kernel<LGB, A, false, true, kImageWarps, false, true>
+                          : render_image_kernel<LGB, A, false, false, kImageWarps, false, true>;
+        kernel<<<(unsigned)(sch->nt * sch->parts + 4 * sch->smax), nt, 0, st>>>(s, cam, mlp, w, rgb, dbg, row0, row1, 32,
+                                                                               *sch);
+        return cudaGetLastError();
+    }
+    const int lanes = ps || d ? 32 : image_lanes(ds, (int64_t)cam.W * (row1 - row0));
+    const int tw = T::WX << packet_width_log2(lanes), th = T::WY * (lanes >> packet_width_log2(lanes));
+    const dim3 grid((cam.W + tw - 1) / tw, (row1 - row0 + th - 1) / th);
+    auto* kernel = pw ? render_image_kernel<LGB, A, false, true, kImageWarps, false>
+                      : render_image_kernel<LGB, A, false, false, kImageWarps, false>;
+    if (ps || d) {
+        if constexpr (LGB == 0) {
+            if (ps)
+                kernel = pw ? (d ? render_image_kernel<LGB, A, true, true, kImageWarps, true>
+                                 : render_image_kernel<LGB, A, false, true, kImageWarps, true>)
+                            : (d ? render_image_kernel<LGB, A, true, false, kImageWarps, true>
+                                 : render_image_kernel<LGB, A, false, false, kImageWarps, true>);
+            else
+                kernel = pw ? render_image_kernel<LGB, A, true, true, kImageWarps, false>
+                            : render_image_kernel<LGB, A, true, false, kImageWarps, false>;
+        } else {
+            return cudaErrorInvalidValue;
+        }
+    }
+    kernel<<<grid, nt, 0, st>>>(s, cam, mlp, w, rgb, dbg, row0, row1, lanes, none);
     return cudaGetLastError();
-}
-
-template <int MINB>
-static void rays_launch(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
-                        const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, float2* record, int lanes,
-                        cudaStream_t st) {
-    const unsigned grid = (unsigned)((n + 4 * lanes - 1) / (4 * lanes));
-    const bool d = dbg.aux || dbg.counts || dbg.trace;
-    auto* kernel = record ? render_rays_kernel<true, false, MINB, true>       // recorded: weights in device memory
-                   : pw   ? (d ? render_rays_kernel<true, true, MINB> : render_rays_kernel<false, true, MINB>)
-                          : (d ? render_rays_kernel<true, false, MINB> : render_rays_kernel<false, false, MINB>);
-    kernel<<<grid, 128, 0, st>>>(s, cams, n_cams, pix, n, mlp, pw ? *pw : no_weights(), rgb, dbg, record, lanes);
 }
 
 // A list is spread over the warps of one wave of 7 CTAs per SM: scattered rays have less in
@@ -426,32 +394,38 @@ static void rays_launch(const DevScene& s, const CamTable& cams, int32_t n_cams,
 // keep 7 CTAs per SM to hide the march's latencies: 8 spill with the weights in device memory
 // (131,072 and 262,144 rays of a 1024^3 grid 163 and 277 us with 8, 153 and 268 with 7; 1,000,000
 // rays 731 and 747).
-cudaError_t launch_render_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
-                               int64_t n, const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg,
-                               float2* record, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
+template <int LGB, int A>
+cudaError_t Forward<LGB, A>::rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
+                               const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, float2* record,
+                               cudaStream_t st) {
     const bool d = dbg.aux || dbg.counts || dbg.trace;
     const int lanes = lanes_per_warp(n, (int64_t)s.sms * (d ? 4 : 7) * 4);
-    if (n <= (int64_t)s.sms * 4 * 4 * lanes) rays_launch<4>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, record, lanes, st);
-    else rays_launch<7>(s, cams, n_cams, pix, n, mlp, pw, rgb, dbg, record, lanes, st);
+    const bool one_wave = n <= (int64_t)s.sms * 4 * 4 * lanes;
+    auto* kernel = pw ? (one_wave ? render_rays_kernel<LGB, A, false, true, 4> : render_rays_kernel<LGB, A, false, true, 7>)
+                      : (one_wave ? render_rays_kernel<LGB, A, false, false, 4> : render_rays_kernel<LGB, A, false, false, 7>);
+    if (record) {                       // weights in device memory
+        kernel = one_wave ? render_rays_kernel<LGB, A, true, false, 4, true> : render_rays_kernel<LGB, A, true, false, 7, true>;
+    } else if (d) {
+        if constexpr (LGB == 0)
+            kernel = pw ? (one_wave ? render_rays_kernel<LGB, A, true, true, 4> : render_rays_kernel<LGB, A, true, true, 7>)
+                        : (one_wave ? render_rays_kernel<LGB, A, true, false, 4> : render_rays_kernel<LGB, A, true, false, 7>);
+        else
+            return cudaErrorInvalidValue;
+    }
+    kernel<<<(unsigned)((n + 4 * lanes - 1) / (4 * lanes)), 128, 0, st>>>(
+        BlockScene<LGB, A>(s), cams, n_cams, pix, n, mlp, pw ? *pw : no_weights(), rgb, dbg, record, lanes);
     return cudaGetLastError();
 }
 
-static bool persistent_multi(const PersistentParams& p) { return p.tile_w != p.warp_w || p.tile_h != p.warp_h; }
-
-cudaError_t launch_render_persistent(const DevScene& s, const PersistentParams& p, const float* mlp,
-                                     const MlpWeights* pw, float* rgb, int32_t* queue, int grid, int block,
-                                     cudaStream_t st) {
-    const void* fn = persistent_kernel_fn(pw != nullptr, persistent_multi(p));
-    const MlpWeights& w = pw ? *pw : no_weights();
-    void* args[] = {(void*)&s, (void*)&p, (void*)&mlp, (void*)&w, (void*)&rgb, (void*)&queue};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, 0, st);
-}
-
-const void* persistent_kernel_fn(bool param_weights, bool multi) {
+template <int LGB, int A>
+const void* Forward<LGB, A>::persistent_fn(bool param_weights, bool multi) {
     if (param_weights)
-        return multi ? (const void*)render_persistent_kernel<true, true> : (const void*)render_persistent_kernel<true, false>;
-    return multi ? (const void*)render_persistent_kernel<false, true> : (const void*)render_persistent_kernel<false, false>;
+        return multi ? (const void*)render_persistent_kernel<LGB, A, true, true>
+                     : (const void*)render_persistent_kernel<LGB, A, true, false>;
+    return multi ? (const void*)render_persistent_kernel<LGB, A, false, true>
+                 : (const void*)render_persistent_kernel<LGB, A, false, false>;
 }
+
+template struct Forward<SNERG_LGB, SNERG_ALPHA>;
 
 }  // namespace snerg

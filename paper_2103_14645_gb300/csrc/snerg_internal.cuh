@@ -86,6 +86,47 @@ struct DevScene {
     int32_t sms;      // SMs of the device (host side: launch shapes)
 };
 
+// The scene as the kernels take it, with the block edge (1 << LGB) and what follows from it as
+// compile-time constants that stand before the members of the same name (LGB 0: as members),
+// and whether channel 0 holds alpha (A 0 or 1; 2: by the scene's flags). The march's padded
+// indices, face distances and stencil addresses then take immediate operands, and a composited
+// sample has one arithmetic: 64 mixed views of a 1024^3 grid of 32^3 blocks 5.60 -> 5.18 ms, one
+// 800^2 view 168 -> 158 us (the edge alone: 4.5 and 2 %). Edges of 8 to 64 have builds of their own; smaller blocks, and debug
+// outputs and the per-sample model on any edge, run the build with members.
+template <int LGB>
+struct BlockEdge : DevScene {
+    static constexpr int32_t lgB = LGB, B = 1 << LGB, P = B + 2, P3 = P * P * P;
+};
+template <>
+struct BlockEdge<0> : DevScene {};
+
+constexpr int kAnyAlpha = 2;
+template <int LGB, int A>
+struct BlockScene : BlockEdge<LGB> {
+    explicit BlockScene(const DevScene& s) : BlockEdge<LGB>{s} {}
+    __device__ __forceinline__ bool alpha() const {
+        if constexpr (A == kAnyAlpha) return (this->flags & SNERG_FLAG_ALPHA_ATLAS) != 0;
+        else return A == 1;
+    }
+};
+
+// f(Build<LGB, A>) for the build of scene s
+template <int L, int A>
+struct Build {
+    static constexpr int lgB = L, alpha = A;
+};
+template <class F>
+inline auto with_block_build(const DevScene& s, F&& f) {
+    const bool alpha = (s.flags & SNERG_FLAG_ALPHA_ATLAS) != 0;
+    switch (s.lgB) {
+        case 3: return alpha ? f(Build<3, 1>{}) : f(Build<3, 0>{});
+        case 4: return alpha ? f(Build<4, 1>{}) : f(Build<4, 0>{});
+        case 5: return alpha ? f(Build<5, 1>{}) : f(Build<5, 0>{});
+        case 6: return alpha ? f(Build<6, 1>{}) : f(Build<6, 0>{});
+    }
+    return f(Build<0, kAnyAlpha>{});
+}
+
 // Rays per warp for n rays where `warps` warps are worth launching: 32, or as many lanes fewer
 // (a power of two) as still make no more than that many warps; the other lanes idle. A launch
 // that leaves the chip part empty is as slow as its slowest warps, whose lanes wait for one
@@ -205,7 +246,8 @@ struct Box {
     float lo[3], hi[3];
 };
 
-__device__ __forceinline__ Box make_box(const DevScene& s, const int lo[3], const int hi[3]) {
+template <class SC>
+__device__ __forceinline__ Box make_box(const SC& s, const int lo[3], const int hi[3]) {
     Box bx;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -301,7 +343,8 @@ __device__ __forceinline__ float box_search(const Ray& r, float kmax, float k, f
 // of dependent steps in small ones); one shared copy with a face instead of a box per axis:
 // 64 mixed views of a 1024^3 grid 6.01 -> 5.64 ms, one 800^2 view 190 -> 183 us, 262,147
 // scattered rays 283 -> 255 us.
-__device__ __forceinline__ float march_exit(const DevScene& s, const Ray& r, const float inv_d[3], float kh,
+template <class SC>
+__device__ __forceinline__ float march_exit(const SC& s, const Ray& r, const float inv_d[3], float kh,
                                             const int j[3], int D, float half) {
     const int DB = D << s.lgB, BD = s.B - DB;
     float te = r.t1;
@@ -373,7 +416,8 @@ __device__ __forceinline__ uint32_t floor_raw(float x) { return (uint32_t)__floa
 
 // For the block of voxel j: padded index = (v2 P + v1) P + v0 - base, v raw coordinates
 // (floor_raw) and (j & -B) - 1 the origin of the block's padded copy.
-__device__ __forceinline__ uint32_t padded_base(const DevScene& s, const int j[3]) {
+template <class SC>
+__device__ __forceinline__ uint32_t padded_base(const SC& s, const int j[3]) {
     const uint32_t P = (uint32_t)s.P, B = (uint32_t)-s.B, c = (uint32_t)kMagicBits - 1u;
     return (((uint32_t)j[2] & B) * P + ((uint32_t)j[1] & B)) * P + ((uint32_t)j[0] & B) + c * (P * P + P + 1u);
 }
@@ -420,7 +464,8 @@ __device__ __forceinline__ void load_stencil(const float u[3], uint32_t base, in
 // Density trilinear of one composited sample (binary32, x then y then z) and its
 // compositing (Eqs. 2, 5, 6): returns w_k and advances T (and tau); saturated once the
 // ray's remaining transmittance is below the early-exit bound.
-__device__ __forceinline__ float composite(const DevScene& s, const uint2 cv[8], const float f[3], const float g[3],
+template <class SC>
+__device__ __forceinline__ float composite(const SC& s, const uint2 cv[8], const float f[3], const float g[3],
                                            float& T, float& tau, bool& saturated) {
     const float e00 = __fadd_rn(__fmul_rn(code(cv[0].x, 0), g[0]), __fmul_rn(code(cv[1].x, 0), f[0]));
     const float e10 = __fadd_rn(__fmul_rn(code(cv[2].x, 0), g[0]), __fmul_rn(code(cv[3].x, 0), f[0]));
@@ -430,7 +475,7 @@ __device__ __forceinline__ float composite(const DevScene& s, const uint2 cv[8],
     const float e1 = __fadd_rn(__fmul_rn(e01, g[1]), __fmul_rn(e11, f[1]));
     const float sq = __fadd_rn(__fmul_rn(e0, g[2]), __fmul_rn(e1, f[2]));
     float wk;
-    if (s.flags & SNERG_FLAG_ALPHA_ATLAS) {
+    if (s.alpha()) {
         // channel 0 holds alpha: a = s * binary32(1/255), T <- T (1 - a) in binary32,
         // stop once T < binary32(1e-3)
         const float a = __fmul_rn(sq, s.inv255);
@@ -452,7 +497,8 @@ __device__ __forceinline__ float composite(const DevScene& s, const uint2 cv[8],
 // gfeat into the eight corners' gradient entries ([slot][B^3][8], channel 0 unused) with
 // vector atomics. o: the sample's block origin minus one, fi its stencil's lower corner
 // (integer voxel coordinates).
-__device__ __forceinline__ void scatter_sample(const DevScene& s, int slot, const int fi[3], const int o[3],
+template <class SC>
+__device__ __forceinline__ void scatter_sample(const SC& s, int slot, const int fi[3], const int o[3],
                                                const float f[3], const float g[3], float wk, const float* gfeat,
                                                float* grad_atlas) {
     const int B = s.B, N = s.N;
@@ -512,8 +558,8 @@ __device__ __forceinline__ void per_sample_residual(const MlpWeights* pw, const 
 // PS: the non-deferred comparison model (SNERG_FLAG_PER_SAMPLE_MLP): every composited
 // sample also evaluates the view-dependence MLP on its own (c_d, v) (weights from pw, else
 // from sW) and adds w_k (c_d,k + residual_k) to st.rgb_ps.
-template <bool TRACE, bool GRAD, bool PS = false, bool SPEC = false, bool REC = false, bool CONT = false>
-__device__ __forceinline__ void march(const DevScene& s, const Ray& r, MarchState& st,
+template <bool TRACE, bool GRAD, bool PS = false, bool SPEC = false, bool REC = false, bool CONT = false, class SC>
+__device__ __forceinline__ void march(const SC& s, const Ray& r, MarchState& st,
                                       uint64_t* trace, int trace_cap,
                                       const float* gfeat, float* grad_atlas,
                                       int k_begin = 0, int* k_first = nullptr,
@@ -923,22 +969,49 @@ struct SchedArgs {
     int32_t parts;             // CTAs per dense tile (1, 2, 4, 8: bands of its rows)
 };
 
-// rays per warp of a one-camera launch of n pixels
-int image_lanes(const DevScene& s, int64_t n);
+// Rays per warp of a one-camera launch of n pixels: up to three waves of warps. 40,000 pixels of a
+// 1024^3 grid take 202 us with 32 rays per warp, 134 with 8 and 118 with 4 (2.1 waves); 160,000 take
+// 201, 171 with 16 (2.1) and 164 with 8 (4.1), but of a 512^3 grid 108, 102 and 111; from 470,000
+// on 32 is the best or within 5 % of it.
+constexpr int kImageWarps = 4;     // warps per CTA of the one-camera launch
+inline int image_lanes(const DevScene& s, int64_t n) { return lanes_per_warp(n, (int64_t)s.sms * 8 * kImageWarps * 3); }
 
-// pw: weights as a kernel parameter (nullptr: read them from `mlp` in device memory)
-// sch: nullable; with it the launch takes its tile order from the previous frame's
-// buckets and records its own tile costs (deferred model, all rows, no debug outputs)
+inline const MlpWeights& no_weights() {
+    static const MlpWeights z = {};
+    return z;
+}
+
+// The kernels of one block build (snerg_fwd.cu and snerg_bwd.cu are compiled once per build).
+// pw: weights as a kernel parameter (nullptr: read them from `mlp` in device memory).
+// image: rows [row0, row1); sch: nullable; with it the launch takes its tile order from the
+// previous frame's buckets and records its own tile costs (deferred model, all rows, no debug
+// outputs). rays: record: nullable, with debug outputs and device weights.
+struct PersistentParams;
+template <int LGB, int A>
+struct Forward {
+    static cudaError_t image(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw, float* rgb,
+                             const DebugOut& dbg, cudaStream_t st, int row0, int row1, const SchedArgs* sch);
+    static cudaError_t rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
+                            const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, float2* record,
+                            cudaStream_t st);
+    // the persistent kernel for weights as parameters or in device memory, and for work items
+    // of one warp pass or several (multi)
+    static const void* persistent_fn(bool param_weights, bool multi);
+};
+template <int LGB, int A>
+struct Adjoint {
+    static cudaError_t backward(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
+                                const float* mlp, const float* grad_rgb, const float* fwd_aux, const int32_t* fwd_counts,
+                                const float2* record, float* grad_atlas, float* grad_mlp, cudaStream_t st);
+    static cudaError_t train(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
+                             const float* mlp, const float* target, float* rgb_out, float* loss, float* grad_atlas,
+                             float* grad_mlp, cudaStream_t st);
+};
+
+// snerg_api.cu: the build for the scene
 cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
                                 float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1,
                                 const SchedArgs* sch = nullptr);
-cudaError_t launch_render_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix,
-                               int64_t n, const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg,
-                               float2* record, cudaStream_t st);
-cudaError_t launch_backward_rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
-                                 const float* mlp, const float* grad_rgb, const float* fwd_aux,
-                                 const int32_t* fwd_counts, const float2* record, float* grad_atlas, float* grad_mlp,
-                                 cudaStream_t st);
 cudaError_t launch_validate(const int32_t* ind, int64_t n_ind, int64_t nb, int32_t* blk_of_slot, int32_t* err,
                             cudaStream_t st);
 // the padded atlas and the 8 octants' voxel-distance planes of every stored block; a launch
@@ -991,12 +1064,5 @@ struct PersistentParams {
     int32_t tile_w, tile_h;             // pixels per work item (tile_w * tile_h % 32 == 0)
     int32_t warp_w, warp_h;             // pixels per warp pass (warp_w * warp_h == 32)
 };
-
-cudaError_t launch_render_persistent(const DevScene& s, const PersistentParams& p, const float* mlp,
-                                     const MlpWeights* pw, float* rgb, int32_t* queue, int grid, int block,
-                                     cudaStream_t st);
-// the persistent kernel for weights as parameters or in device memory, and for work items
-// of one warp pass or several (multi)
-const void* persistent_kernel_fn(bool param_weights, bool multi);
 
 }  // namespace snerg

@@ -129,6 +129,7 @@ __device__ __forceinline__ uint2 raw_voxel(const DevScene& s, const uint2* atlas
 }
 
 constexpr int kProbes = 8;
+using RawScene = BlockScene<0, 0>;      // any block edge, density codes
 
 // The march of snerg_internal.cuh on the caller's unpadded atlas: empty blocks are
 // skipped through the block distance map, every lattice sample of an occupied block
@@ -141,7 +142,7 @@ constexpr int kProbes = 8;
 // other is a chain of memory latencies: kProbes samples' codes are loaded together, and those
 // with density composited in order. 65,537 scattered rays of a 768^3 grid: 294 us one by one,
 // 150 us for 8 together (the whole call 301 -> 169 us; 174 for 4, 192 for 16).
-__device__ __forceinline__ void march_raw(const DevScene& s, const uint2* atlas, int64_t nb, const Ray& r,
+__device__ __forceinline__ void march_raw(const RawScene& s, const uint2* atlas, int64_t nb, const Ray& r,
                                           MarchState& st) {
 #pragma unroll
     for (int c = 0; c < 7; ++c) st.acc[c] = 0.0f;
@@ -222,7 +223,7 @@ __device__ __forceinline__ void march_raw(const DevScene& s, const uint2* atlas,
 
 // MINB and lanes as for render_rays_kernel
 template <int MINB>
-__global__ void __launch_bounds__(128, MINB) render_rays_noalloc_kernel(const DevScene s, const uint2* __restrict__ atlas,
+__global__ void __launch_bounds__(128, MINB) render_rays_noalloc_kernel(const RawScene s, const uint2* __restrict__ atlas,
                                                                         int64_t nb,
                                                                         const __grid_constant__ CamTable cams,
                                                                         int32_t n_cams, const int32_t* __restrict__ pix,
@@ -338,7 +339,7 @@ extern "C" snerg_status snerg_render_rays_noalloc(const snerg_scene_desc* desc, 
         const int lanes = lanes_per_warp(n, (int64_t)sms * 4 * 4);
         const int64_t ctas = (n + 4 * lanes - 1) / (4 * lanes);
         auto* kernel = ctas <= 4 * (int64_t)sms ? render_rays_noalloc_kernel<4> : render_rays_noalloc_kernel<8>;
-        kernel<<<(unsigned)ctas, 128, 0, st>>>(s, reinterpret_cast<const uint2*>(d_atlas), num_blocks, table, n_cams, d_pix,
+        kernel<<<(unsigned)ctas, 128, 0, st>>>(RawScene(s), reinterpret_cast<const uint2*>(d_atlas), num_blocks, table, n_cams, d_pix,
                                                n, d_mlp, d_rgb, lanes);
         e = cudaGetLastError();
     }
