@@ -91,8 +91,9 @@ struct DevScene {
 // and whether channel 0 holds alpha (A 0 or 1; 2: by the scene's flags). The march's padded
 // indices, face distances and stencil addresses then take immediate operands, and a composited
 // sample has one arithmetic: 64 mixed views of a 1024^3 grid of 32^3 blocks 5.60 -> 5.18 ms, one
-// 800^2 view 168 -> 158 us (the edge alone: 4.5 and 2 %). Edges of 8 to 64 have builds of their own; smaller blocks, and debug
-// outputs and the per-sample model on any edge, run the build with members.
+// 800^2 view 168 -> 158 us (the edge alone: 4.5 and 2 %). Edges of 8 to 64 have builds of their
+// own; smaller blocks, and debug outputs and the per-sample model on any edge, run the build
+// with members.
 template <int LGB>
 struct BlockEdge : DevScene {
     static constexpr int32_t lgB = LGB, B = 1 << LGB, P = B + 2, P3 = P * P * P;

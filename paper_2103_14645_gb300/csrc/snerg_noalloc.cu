@@ -117,7 +117,8 @@ __global__ void __launch_bounds__(256) noalloc_map_z_kernel(const uint8_t* __res
 
 // value of channel 0..7 of voxel (x, y, z) of the virtual grid, clamped to the grid;
 // 0 in empty blocks (Sec. 5.1)
-__device__ __forceinline__ uint2 raw_voxel(const DevScene& s, const uint2* atlas, int64_t nb, int x, int y, int z) {
+template <class SC>
+__device__ __forceinline__ uint2 raw_voxel(const SC& s, const uint2* atlas, int64_t nb, int x, int y, int z) {
     x = min(max(x, 0), s.N - 1);
     y = min(max(y, 0), s.N - 1);
     z = min(max(z, 0), s.N - 1);
@@ -129,7 +130,6 @@ __device__ __forceinline__ uint2 raw_voxel(const DevScene& s, const uint2* atlas
 }
 
 constexpr int kProbes = 8;
-using RawScene = BlockScene<0, 0>;      // any block edge, density codes
 
 // The march of snerg_internal.cuh on the caller's unpadded atlas: empty blocks are
 // skipped through the block distance map, every lattice sample of an occupied block
@@ -141,8 +141,10 @@ using RawScene = BlockScene<0, 0>;      // any block edge, density codes
 // Without a voxel distance map a ray meets every sample of a block, and one probe after the
 // other is a chain of memory latencies: kProbes samples' codes are loaded together, and those
 // with density composited in order. 65,537 scattered rays of a 768^3 grid: 294 us one by one,
-// 150 us for 8 together (the whole call 301 -> 169 us; 174 for 4, 192 for 16).
-__device__ __forceinline__ void march_raw(const RawScene& s, const uint2* atlas, int64_t nb, const Ray& r,
+// 150 us for 8 together (the whole call 301 -> 169 us; 174 for 4, 192 for 16), 165 with the block
+// edge as a constant.
+template <class SC>
+__device__ __forceinline__ void march_raw(const SC& s, const uint2* atlas, int64_t nb, const Ray& r,
                                           MarchState& st) {
 #pragma unroll
     for (int c = 0; c < 7; ++c) st.acc[c] = 0.0f;
@@ -221,9 +223,9 @@ __device__ __forceinline__ void march_raw(const RawScene& s, const uint2* atlas,
     }
 }
 
-// MINB and lanes as for render_rays_kernel
-template <int MINB>
-__global__ void __launch_bounds__(128, MINB) render_rays_noalloc_kernel(const RawScene s, const uint2* __restrict__ atlas,
+// LGB: see BlockScene (density codes only); MINB and lanes as for render_rays_kernel
+template <int LGB, int MINB>
+__global__ void __launch_bounds__(128, MINB) render_rays_noalloc_kernel(const BlockScene<LGB, 0> s, const uint2* __restrict__ atlas,
                                                                         int64_t nb,
                                                                         const __grid_constant__ CamTable cams,
                                                                         int32_t n_cams, const int32_t* __restrict__ pix,
@@ -338,9 +340,12 @@ extern "C" snerg_status snerg_render_rays_noalloc(const snerg_scene_desc* desc, 
         // one wave of 4 CTAs per SM: 65,537 rays 169 us with 32 rays per warp, 179 with 16
         const int lanes = lanes_per_warp(n, (int64_t)sms * 4 * 4);
         const int64_t ctas = (n + 4 * lanes - 1) / (4 * lanes);
-        auto* kernel = ctas <= 4 * (int64_t)sms ? render_rays_noalloc_kernel<4> : render_rays_noalloc_kernel<8>;
-        kernel<<<(unsigned)ctas, 128, 0, st>>>(RawScene(s), reinterpret_cast<const uint2*>(d_atlas), num_blocks, table, n_cams, d_pix,
-                                               n, d_mlp, d_rgb, lanes);
+        with_block_build(s, [&](auto build) {
+            constexpr int L = decltype(build)::lgB;
+            auto* kernel = ctas <= 4 * (int64_t)sms ? render_rays_noalloc_kernel<L, 4> : render_rays_noalloc_kernel<L, 8>;
+            kernel<<<(unsigned)ctas, 128, 0, st>>>(BlockScene<L, 0>(s), reinterpret_cast<const uint2*>(d_atlas), num_blocks,
+                                                   table, n_cams, d_pix, n, d_mlp, d_rgb, lanes);
+        });
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && d_status) e = cudaMemcpyAsync(d_status, status, sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
