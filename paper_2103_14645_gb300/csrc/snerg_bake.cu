@@ -441,12 +441,14 @@ __device__ __forceinline__ uint32_t pack4(uint32_t a, uint32_t b, uint32_t c, ui
 }
 
 // 2^(-k d^2) of the binary32 k and d, the rounding errors of the exponent carried into the
-// result (three factors are multiplied where one exponential was)
+// result (three factors are multiplied where one exponential was). Where the exponential is 0
+// its correction is not taken: an exponent beyond binary32 (blobs of s below 1e-19) has an
+// infinite or undefined one.
 __device__ __forceinline__ float gauss_factor(float k, float d) {
     const float p = k * d, e = p * d;
     const float low = fmaf(fmaf(k, d, -p), d, fmaf(p, d, -e));
     const float r = ex2(-e);
-    return fmaf(r * -0.69314718f, low, r);
+    return r > 0.0f ? fmaf(r * -0.69314718f, low, r) : r;
 }
 
 // the centre of voxel i along an axis, rounded, and what the rounding left

@@ -49,3 +49,17 @@ def test_atlas_of_a_counted_bake():
         ind, atl = renderer.bake(N, B, BMIN, EXTENT, 100.0, field, DEV)
         ind1, atl1 = renderer.bake(N, B, BMIN, EXTENT, 100.0, field, DEV, max_blocks=atl.shape[0] + 3)
         assert atl.shape[0] > 0 and bool((ind == ind1).all()) and bool((atl == atl1).all())
+
+
+@pytest.mark.parametrize("B", [8, 16, 32, 64])
+def test_a_blob_narrower_than_any_voxel_adds_nothing(B):
+    """A finite blob whose exponent leaves binary32 a voxel away (s = 5e-20: k = 2.9e38) contributes
+    exactly 0 between the voxel centres: the codes of the field without it."""
+    f = synth.analytic_field(B, n_blob=3, std=(0.3, 0.6), peak=(20.0, 80.0))
+    out = []
+    for blobs in (f["blobs"], np.concatenate([f["blobs"], [[-1.7031, -1.7011, -1.7057, 5e-20, 10.0]]]).astype(np.float32)):
+        field = renderer.bake_field(blobs, f["colors"], f["jitter"], TAU)
+        out.append(renderer.bake(B, B, (-2.0,) * 3, 4.0, 100.0, field, DEV))
+    (ind, atl), (ind_n, atl_n) = out
+    assert bool((ind == ind_n).all()) and bool((atl == atl_n).all())
+    assert float((atl[..., 0] > 0).float().mean()) > 0.1
