@@ -244,11 +244,13 @@ snerg_status snerg_render_backward(snerg_handle h, const snerg_camera* cams, int
 
 /* snerg_render_rays and snerg_render_backward for a program that keeps state between the two:
  * the render also stores what the adjoint needs of each ray (its composites and its first 32
- * composited samples' lattice indices and weights), and the adjoint does not march again.
+ * composited samples' lattice indices and weights), and the adjoint marches only the rays that
+ * composited more, on from the last recorded sample.
  *   d_state : snerg_state_bytes(n) bytes (312 per ray), 16-byte aligned, not initialised;
  *             opaque, valid for the same handle, cameras, rays and n;
  *   d_grad_atlas, d_grad_mlp (either nullable) are WRITTEN, not accumulated into: with the
- *             sums that snerg_render_backward would add to zeros.
+ *             sums that snerg_render_backward would add to zeros; a call that returns
+ *             SNERG_E_INVAL leaves them as they were.
  * d_mlp must be device weights. */
 size_t snerg_state_bytes(int64_t n);
 snerg_status snerg_render_rays_recorded(snerg_handle h, const snerg_camera* cams, int32_t n_cams,

@@ -659,20 +659,26 @@ extern "C" snerg_status snerg_render_rays_recorded(snerg_handle h, const snerg_c
                        (cudaStream_t)stream);
 }
 
+// overwrite: the gradients are cleared first (once the arguments are known to be valid)
 static snerg_status render_backward(snerg_handle h, const snerg_camera* cams, int32_t n_cams, const int32_t* d_pix,
                                     int64_t n, const float* d_mlp, const float* d_grad_rgb, const float* d_fwd_aux,
                                     const int32_t* d_fwd_counts, const float2* record, float* d_grad_atlas,
-                                    float* d_grad_mlp, cudaStream_t st) {
+                                    float* d_grad_mlp, bool overwrite, cudaStream_t st) {
     if (!h || n < 0) return SNERG_E_INVAL;
     if (h->desc.flags & SNERG_FLAG_PER_SAMPLE_MLP) return SNERG_E_UNSUPPORTED;
     CamTable* t = new (std::nothrow) CamTable;
     if (!t) return SNERG_E_NOMEM;
     if (!make_table(cams, n_cams, t)) { delete t; return SNERG_E_INVAL; }
-    if (n == 0 || (!d_grad_atlas && !d_grad_mlp)) { delete t; return SNERG_OK; }
-    if (!d_pix || !d_mlp || !d_grad_rgb) { delete t; return SNERG_E_INVAL; }
-    if (d_grad_atlas && ((uintptr_t)d_grad_atlas & 15u)) { delete t; return SNERG_E_INVAL; }
-    if ((d_fwd_aux == nullptr) != (d_fwd_counts == nullptr)) { delete t; return SNERG_E_INVAL; }
-    const cudaError_t e = with_block_build(h->ds, [&](auto b) {
+    const bool work = n > 0 && (d_grad_atlas || d_grad_mlp);
+    if (work && (!d_pix || !d_mlp || !d_grad_rgb)) { delete t; return SNERG_E_INVAL; }
+    if (work && d_grad_atlas && ((uintptr_t)d_grad_atlas & 15u)) { delete t; return SNERG_E_INVAL; }
+    if (work && (d_fwd_aux == nullptr) != (d_fwd_counts == nullptr)) { delete t; return SNERG_E_INVAL; }
+    cudaError_t e = cudaSuccess;
+    if (overwrite && d_grad_atlas && h->nb > 0)
+        e = cudaMemsetAsync(d_grad_atlas, 0, (size_t)h->nb * h->ds.B * h->ds.B * h->ds.B * 8 * sizeof(float), st);
+    if (overwrite && d_grad_mlp && e == cudaSuccess) e = cudaMemsetAsync(d_grad_mlp, 0, kNParam * sizeof(float), st);
+    if (e != cudaSuccess || !work) { delete t; return e == cudaSuccess ? SNERG_OK : SNERG_E_CUDA; }
+    e = with_block_build(h->ds, [&](auto b) {
         return Adjoint<decltype(b)::lgB, decltype(b)::alpha>::backward(h->ds, *t, n_cams, d_pix, n, d_mlp, d_grad_rgb, d_fwd_aux,
                                                        d_fwd_counts, record, d_grad_atlas, d_grad_mlp, st);
     });
@@ -688,7 +694,7 @@ extern "C" snerg_status snerg_render_backward(snerg_handle h, const snerg_camera
                                               const int32_t* d_fwd_counts, float* d_grad_atlas, float* d_grad_mlp,
                                               void* stream) {
     return render_backward(h, cams, n_cams, d_pix, n, d_mlp, d_grad_rgb, d_fwd_aux, d_fwd_counts, nullptr, d_grad_atlas,
-                           d_grad_mlp, (cudaStream_t)stream);
+                           d_grad_mlp, false, (cudaStream_t)stream);
 }
 
 extern "C" snerg_status snerg_render_backward_recorded(snerg_handle h, const snerg_camera* cams, int32_t n_cams,
@@ -698,15 +704,9 @@ extern "C" snerg_status snerg_render_backward_recorded(snerg_handle h, const sne
     if (!h || n < 0) return SNERG_E_INVAL;
     if (h->desc.flags & SNERG_FLAG_PER_SAMPLE_MLP) return SNERG_E_UNSUPPORTED;
     if (n > 0 && (!d_state || ((uintptr_t)d_state & 15u))) return SNERG_E_INVAL;
-    cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaSuccess;
-    if (d_grad_atlas && h->nb > 0)
-        e = cudaMemsetAsync(d_grad_atlas, 0, (size_t)h->nb * h->ds.B * h->ds.B * h->ds.B * 8 * sizeof(float), st);
-    if (d_grad_mlp && e == cudaSuccess) e = cudaMemsetAsync(d_grad_mlp, 0, kNParam * sizeof(float), st);
-    if (e != cudaSuccess) return SNERG_E_CUDA;
     const RayState s = ray_state(d_state, n);
     return render_backward(h, cams, n_cams, d_pix, n, d_mlp, d_grad_rgb, s.aux, s.counts, s.record, d_grad_atlas,
-                           d_grad_mlp, st);
+                           d_grad_mlp, true, (cudaStream_t)stream);
 }
 
 extern "C" snerg_status snerg_train_rays(snerg_handle h, const snerg_camera* cams, int32_t n_cams,

@@ -86,6 +86,13 @@ def test_no_rays_and_arguments():
     assert lib.snerg_render_rays_recorded(r.handle, P, 2, pix.data_ptr(), 4, w.data_ptr(), rgb.data_ptr(), none, none) == 1
     assert lib.snerg_render_backward_recorded(r.handle, P, 2, pix.data_ptr(), 4, w.data_ptr(), rgb.data_ptr(), none, none,
                                               gm.data_ptr(), none) == 1
+    # a refused call leaves the gradients alone: no rays' pixels, weights or upstream gradient, no
+    # cameras, an unaligned atlas gradient
+    ga = torch.ones(sc.atlas.size + 1, device=DEV)
+    args = [r.handle, P, 2, pix.data_ptr(), 4, w.data_ptr(), rgb.data_ptr(), state.data_ptr(), ga.data_ptr(), gm.data_ptr(), none]
+    for i, v in ((3, none), (5, none), (6, none), (1, none), (2, 0), (8, ga.data_ptr() + 4)):
+        assert lib.snerg_render_backward_recorded(*args[:i], v, *args[i + 1:]) == 1
+        assert bool((ga == 1).all()) and bool((gm == 1).all()), i
     rgb, state = r.render_rays_recorded(sc.cameras, pix[:0], w)
     ga = torch.ones(sc.atlas.shape, device=DEV)
     r.backward_recorded(sc.cameras, pix[:0], w, rgb, state, ga, gm)
