@@ -403,6 +403,8 @@ class Renderer:
                 raise ValueError("grad_atlas must have nb*B^3*8 elements")
         if grad_mlp is not None:
             _require_cuda(grad_mlp, "grad_mlp", torch.float32)
+            if grad_mlp.numel() < MLP_PARAMS:
+                raise ValueError(f"grad_mlp must have {MLP_PARAMS} elements")
         _check(self.lib.snerg_render_backward_recorded(self.handle, c.ctypes.data, c.shape[0], pix.data_ptr(), n,
                                                        mlp.data_ptr(), grad_rgb.data_ptr(), state.data_ptr(),
                                                        _ptr(grad_atlas), _ptr(grad_mlp), _stream(self.device)),

@@ -93,6 +93,8 @@ def test_no_rays_and_arguments():
     for i, v in ((3, none), (5, none), (6, none), (1, none), (2, 0), (8, ga.data_ptr() + 4)):
         assert lib.snerg_render_backward_recorded(*args[:i], v, *args[i + 1:]) == 1
         assert bool((ga == 1).all()) and bool((gm == 1).all()), i
+    with pytest.raises(ValueError):                        # too short for the sums
+        r.backward_recorded(sc.cameras, pix, w, rgb, state, None, gm[:882])
     rgb, state = r.render_rays_recorded(sc.cameras, pix[:0], w)
     ga = torch.ones(sc.atlas.shape, device=DEV)
     r.backward_recorded(sc.cameras, pix[:0], w, rgb, state, ga, gm)
