@@ -348,9 +348,10 @@ snerg_status snerg_adam_step(float* d_param, float* d_m, float* d_v, const float
  * SNERG_FLAG_UNPREMULTIPLY is accepted (others return SNERG_E_INVAL).
  * Scratch: a status word and the block-level empty-space distance map live in one static
  * device array of 786,688 bytes that every GPU loading this library holds until the
- * process exits. The first call on each device looks up that array's device address
- * (cudaGetSymbolAddress, with the device current): make that first call before any
- * stream capture. The address is kept for the life of the process, so do not use this
+ * process exits. The first call on each device, with rays or without (n = 0), looks up that
+ * array's device address and loads every kernel that later calls can launch, for all block
+ * edges and ray counts (with the device current): make that first call before any stream
+ * capture and before device memory runs out. The address is kept for the life of the process, so do not use this
  * entry point after a device reset (cudaDeviceReset or a primary-context reset may move
  * the array). All calls share the array and each call rewrites it, so calls whose
  * work overlaps on the GPU (different streams or host threads) race; serialise them.

@@ -11,11 +11,12 @@
 // size that every GPU loading the library holds until the process exits.
 //
 // The array's host-side name is only a stand-in; its device address is fetched with
-// cudaGetSymbolAddress once per device (with that device current) on the first call
-// made on that device, so that first call should happen before any stream capture. The
-// address is kept for the life of the process: a device reset (cudaDeviceReset, or a
-// reset of the primary context) reloads the module and may move the array, after which
-// the kept address is stale, so this entry point must not be used across a reset.
+// cudaGetSymbolAddress, and every kernel a call can launch is loaded, once per device (with
+// that device current) on the first call made on that device, so that first call should
+// happen before any stream capture. The address is kept for the life of the process: a
+// device reset (cudaDeviceReset, or a reset of the primary context) reloads the module and
+// may move the array, after which the kept address is stale, so this entry point must not be
+// used across a reset.
 // Every call shares the array: calls whose work overlaps on the GPU (two streams, or two
 // host threads) race on it and must be serialised by the caller.
 #include <cuda_runtime.h>
@@ -37,26 +38,6 @@ constexpr int kNoAllocMaxDevices = 64;
 
 // [0, 256): status word | bdist [G^3] | two G^3 temporaries of the distance transform
 __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocBytes];
-
-std::mutex g_setup_mu;
-void* g_scratch_dev[kNoAllocMaxDevices] = {};
-
-// device address of g_noalloc_scratch on the current device (set up once per device)
-cudaError_t scratch_address(void** out) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kNoAllocMaxDevices) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(g_setup_mu);
-    if (!g_scratch_dev[dev]) {
-        void* p = nullptr;
-        e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-        if (e != cudaSuccess) return e;
-        g_scratch_dev[dev] = p;
-    }
-    *out = g_scratch_dev[dev];
-    return cudaSuccess;
-}
 
 // ---------------------------------------------------------------------------------
 // The two-sided block map in two launches: the x and y passes of one z slice per CTA in
@@ -254,6 +235,47 @@ __global__ void __launch_bounds__(128, MINB) render_rays_noalloc_kernel(const Bl
     rgb[i * 3 + 0] = c[0];
     rgb[i * 3 + 1] = c[1];
     rgb[i * 3 + 2] = c[2];
+}
+
+std::mutex g_setup_mu;
+void* g_scratch_dev[kNoAllocMaxDevices] = {};
+
+// Every kernel that a call can launch, loaded on the current device: the runtime loads a kernel's
+// code (device memory, and host time in the middle of a frame) at its first use otherwise, and
+// which of the builds runs goes by the block edge and the number of rays.
+cudaError_t load_kernels() {
+    const void* const kernels[] = {
+        (const void*)noalloc_map_xy_kernel,            (const void*)noalloc_map_z_kernel,
+        (const void*)render_rays_noalloc_kernel<0, 4>, (const void*)render_rays_noalloc_kernel<0, 8>,
+        (const void*)render_rays_noalloc_kernel<3, 4>, (const void*)render_rays_noalloc_kernel<3, 8>,
+        (const void*)render_rays_noalloc_kernel<4, 4>, (const void*)render_rays_noalloc_kernel<4, 8>,
+        (const void*)render_rays_noalloc_kernel<5, 4>, (const void*)render_rays_noalloc_kernel<5, 8>,
+        (const void*)render_rays_noalloc_kernel<6, 4>, (const void*)render_rays_noalloc_kernel<6, 8>};
+    for (const void* k : kernels) {
+        cudaFuncAttributes a;
+        const cudaError_t e = cudaFuncGetAttributes(&a, k);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// the current device's set-up, once per device: the kernels and the device address of
+// g_noalloc_scratch
+cudaError_t scratch_address(void** out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kNoAllocMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(g_setup_mu);
+    if (!g_scratch_dev[dev]) {
+        void* p = nullptr;
+        e = load_kernels();
+        if (e == cudaSuccess) e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+        if (e != cudaSuccess) return e;
+        g_scratch_dev[dev] = p;
+    }
+    *out = g_scratch_dev[dev];
+    return cudaSuccess;
 }
 
 bool desc_ok_noalloc(const snerg_scene_desc* d) {
