@@ -242,30 +242,27 @@ static const void* persistent_fn(const DevScene& s, bool param_weights, bool mul
     return with_block_build(s, [&](auto b) { return Forward<decltype(b)::lgB, decltype(b)::alpha>::persistent_fn(param_weights, multi); });
 }
 
-// snerg_prep.cu; adam: nullable, an optimiser step on the values first (m, v, g)
-cudaError_t launch_requantize(const int32_t* ind, const int32_t* blk_of_slot, float* values, float* m, float* v,
-                              const float* g, const AdamArgs* adam, int64_t nb, int N, int B, int lgB, uint2* patlas,
-                              uint8_t* atlas_out, cudaStream_t st);
+// snerg_prep.cu
+cudaError_t launch_requantize(const int32_t* ind, const int32_t* blk_of_slot, const float* values, int64_t nb, int N,
+                              int B, int lgB, uint2* patlas, uint8_t* atlas_out, cudaStream_t st);
+// an optimiser step on the values first (m, v, g)
+cudaError_t launch_adam_requantize(const int32_t* ind, const int32_t* blk_of_slot, float* values, float* m, float* v,
+                                   const float* g, const AdamArgs& adam, int64_t nb, int N, int B, int lgB,
+                                   uint2* patlas, uint8_t* atlas_out, cudaStream_t st);
 }  // namespace snerg
-
-static snerg_status requantize(snerg_scene* h, float* values, float* m, float* v, const float* g, const AdamArgs* adam,
-                               uint8_t* atlas_out, void* stream) {
-    Layout L;
-    make_layout(&h->desc, h->nb, &L);
-    const cudaError_t e = launch_requantize(h->ds.ind, (const int32_t*)(h->ws + L.blk), values, m, v, g, adam, h->nb,
-                                            h->ds.N, h->ds.B, h->ds.lgB, (uint2*)(h->ws + L.patlas), atlas_out,
-                                            (cudaStream_t)stream);
-    if (e != cudaSuccess) return SNERG_E_CUDA;
-    ++h->launches;
-    return SNERG_OK;
-}
 
 extern "C" snerg_status snerg_requantize_atlas(snerg_handle h, const float* d_values, uint8_t* d_atlas_out,
                                              void* stream) {
     if (!h) return SNERG_E_INVAL;
     if (h->nb == 0) return SNERG_OK;
     if (!d_values || ((uintptr_t)d_values & 15u) || ((uintptr_t)d_atlas_out & 7u)) return SNERG_E_INVAL;
-    return requantize(h, const_cast<float*>(d_values), nullptr, nullptr, nullptr, nullptr, d_atlas_out, stream);
+    Layout L;
+    make_layout(&h->desc, h->nb, &L);
+    if (launch_requantize(h->ds.ind, (const int32_t*)(h->ws + L.blk), d_values, h->nb, h->ds.N, h->ds.B, h->ds.lgB,
+                          (uint2*)(h->ws + L.patlas), d_atlas_out, (cudaStream_t)stream) != cudaSuccess)
+        return SNERG_E_CUDA;
+    ++h->launches;
+    return SNERG_OK;
 }
 
 extern "C" snerg_status snerg_adam_requantize_atlas(snerg_handle h, float* d_values, float* d_m, float* d_v,
@@ -276,7 +273,14 @@ extern "C" snerg_status snerg_adam_requantize_atlas(snerg_handle h, float* d_val
     if (h->nb == 0) return SNERG_OK;
     if (!d_values || !d_m || !d_v || !d_grad || ((uintptr_t)d_atlas_out & 7u)) return SNERG_E_INVAL;
     if (((uintptr_t)d_values | (uintptr_t)d_m | (uintptr_t)d_v | (uintptr_t)d_grad) & 15u) return SNERG_E_INVAL;
-    return requantize(h, d_values, d_m, d_v, d_grad, &a, d_atlas_out, stream);
+    Layout L;
+    make_layout(&h->desc, h->nb, &L);
+    if (launch_adam_requantize(h->ds.ind, (const int32_t*)(h->ws + L.blk), d_values, d_m, d_v, d_grad, a, h->nb, h->ds.N,
+                               h->ds.B, h->ds.lgB, (uint2*)(h->ws + L.patlas), d_atlas_out,
+                               (cudaStream_t)stream) != cudaSuccess)
+        return SNERG_E_CUDA;
+    ++h->launches;
+    return SNERG_OK;
 }
 
 static bool opts_debug(const snerg_render_opts* o) {

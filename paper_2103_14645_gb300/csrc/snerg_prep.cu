@@ -31,7 +31,47 @@ __global__ void validate_kernel(const int32_t* __restrict__ ind, int64_t n_ind, 
 // codes): every stored voxel takes channels 1..7 from floor(255 x + 1/2) of its values
 // (binary32, clamped) and keeps its density byte, so the empty-space maps built from the
 // densities stay valid; atlas_out (nullable) receives the codes in the unpadded layout.
-// ADAM: the values take one optimiser step first, so a fine-tuning step reads them once.
+//
+// By itself: one thread per padded entry, whose source it gathers, so that every store is
+// part of a row. Bound by memory: 70 M voxels 0.87 ms, whether codes change or not; by voxels,
+// as in the optimiser's pass below, 0.86 ms if none does and 1.42 if all do (the apron copies
+// are scattered 4-byte stores).
+__device__ __forceinline__ uint32_t quant8(float x) {
+    const float q = floorf(__fmaf_rn(x, 255.0f, 0.5f));
+    return q > 0.0f ? (q < 255.0f ? (uint32_t)q : 255u) : 0u;   // NaN -> 0
+}
+
+__global__ void requantize_padded_kernel(const int32_t* __restrict__ ind, const int32_t* __restrict__ blk_of_slot,
+                                         const float4* __restrict__ values, int64_t nb, int N, int B, int lgB,
+                                         uint2* __restrict__ patlas, uint2* __restrict__ atlas_out) {
+    const int P = B + 2, P3 = P * P * P, G = N >> lgB;
+    const int64_t total = nb * (int64_t)P3, B3 = (int64_t)B * B * B;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t slot = t / P3;
+        const int r = (int)(t - slot * P3);
+        const int px = r % P, py = (r / P) % P, pz = r / (P * P);
+        const int blk = blk_of_slot[slot];
+        if (blk < 0) continue;                                 // an unreferenced slot has no codes to keep
+        const int bx = blk % G, by = (blk / G) % G, bz = blk / (G * G);
+        const int gx = min(max(bx * B + px - 1, 0), N - 1);
+        const int gy = min(max(by * B + py - 1, 0), N - 1);
+        const int gz = min(max(bz * B + pz - 1, 0), N - 1);
+        const int owner = ind[((gz >> lgB) * G + (gy >> lgB)) * G + (gx >> lgB)];
+        if (owner < 0) continue;                               // apron of an empty block: stays 0
+        const int loc = ((gz & (B - 1)) * B + (gy & (B - 1))) * B + (gx & (B - 1));
+        const int64_t src = (int64_t)owner * B3 + loc;
+        const float4 a = values[2 * src], b = values[2 * src + 1];
+        const uint2 old = patlas[t];
+        uint2 v;
+        v.x = (old.x & 0xffu) | quant8(a.y) << 8 | quant8(a.z) << 16 | quant8(a.w) << 24;
+        v.y = quant8(b.x) | quant8(b.y) << 8 | quant8(b.z) << 16 | quant8(b.w) << 24;
+        patlas[t] = v;
+        if (atlas_out && px >= 1 && px <= B && py >= 1 && py <= B && pz >= 1 && pz <= B) atlas_out[src] = v;
+    }
+}
+
+// The end of a fine-tuning step: one optimiser step on the values and their codes, so that
+// the values are read once.
 //
 // One thread per 4 channels (16-byte loads of consecutive lanes, 4-byte code words). A voxel's
 // copies in the aprons are found from the voxel: along each axis it is also in the apron of
@@ -39,20 +79,15 @@ __global__ void validate_kernel(const int32_t* __restrict__ ind, int64_t n_ind, 
 // the grid's border, so at most 2 x 2 x 2 entries. A code word that does not change is not
 // stored (its copies hold the same word).
 // Bound by memory: a step on 125 M values, most of them untouched, reads 16 bytes of each (and
-// the codes) at 5.7 TB/s, 0.41 ms; an Adam pass over all of them and a requantisation that
-// gathered every padded entry's source took 0.74 + 0.19 ms.
-__device__ __forceinline__ uint32_t quant8(float x) {
-    const float q = floorf(__fmaf_rn(x, 255.0f, 0.5f));
-    return q > 0.0f ? (q < 255.0f ? (uint32_t)q : 255u) : 0u;   // NaN -> 0
-}
-
-template <bool ADAM>
-__global__ void __launch_bounds__(256) requantize_kernel(const int32_t* __restrict__ ind,
-                                                         const int32_t* __restrict__ blk_of_slot, float4* values,
-                                                         float4* __restrict__ m, float4* __restrict__ v,
-                                                         const float4* __restrict__ g, int64_t nb, int N, int B, int lgB,
-                                                         uint32_t* __restrict__ patlas, uint32_t* __restrict__ atlas_out,
-                                                         const AdamArgs a) {
+// the codes) at 5.7 TB/s, 0.41 ms; an Adam pass over all of them and a requantisation by
+// themselves took 0.74 + 0.19 ms. With every value's gradient set and every code changing,
+// 561 M values take 2.50 ms and the two calls 2.61.
+__global__ void __launch_bounds__(256) adam_requantize_kernel(const int32_t* __restrict__ ind,
+                                                              const int32_t* __restrict__ blk_of_slot, float4* values,
+                                                              float4* __restrict__ m, float4* __restrict__ v,
+                                                              const float4* __restrict__ g, int64_t nb, int N, int B,
+                                                              int lgB, uint32_t* __restrict__ patlas,
+                                                              uint32_t* __restrict__ atlas_out, const AdamArgs a) {
     const int P = B + 2, G = N >> lgB;
     const int64_t P3 = (int64_t)P * P * P, total = nb << (3 * lgB + 1);
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
@@ -61,15 +96,11 @@ __global__ void __launch_bounds__(256) requantize_kernel(const int32_t* __restri
         const int c[3] = {l & (B - 1), (l >> lgB) & (B - 1), l >> (2 * lgB)};
         uint32_t* own = patlas + 2 * (slot * P3 + ((c[2] + 1) * P + c[1] + 1) * P + c[0] + 1) + h;
         // all loads before the first is used
-        float4 x = values[t], gi, mi, vi;
-        if (ADAM) {
-            gi = __ldcs(g + t);
-            mi = m[t];
-            vi = v[t];
-        }
+        float4 x = values[t], mi = m[t], vi = v[t];
+        const float4 gi = __ldcs(g + t);
         const uint32_t old = *own;
         const int blk = __ldg(blk_of_slot + slot);
-        if (ADAM && adam_quad(a, gi, mi, vi, x)) {
+        if (adam_quad(a, gi, mi, vi, x)) {
             m[t] = mi;
             v[t] = vi;
             values[t] = x;
@@ -572,20 +603,23 @@ cudaError_t launch_prep_blocks(const int32_t* ind, const int32_t* blk_of_slot, c
     }
 }
 
-cudaError_t launch_requantize(const int32_t* ind, const int32_t* blk_of_slot, float* values, float* m, float* v,
-                              const float* g, const AdamArgs* adam, int64_t nb, int N, int B, int lgB, uint2* patlas,
-                              uint8_t* atlas_out, cudaStream_t st) {
+cudaError_t launch_requantize(const int32_t* ind, const int32_t* blk_of_slot, const float* values, int64_t nb, int N,
+                              int B, int lgB, uint2* patlas, uint8_t* atlas_out, cudaStream_t st) {
     if (nb <= 0) return cudaSuccess;
-    const unsigned grid = grid_for(nb << (3 * lgB + 1));
-    uint32_t* pa = reinterpret_cast<uint32_t*>(patlas);
-    uint32_t* out = reinterpret_cast<uint32_t*>(atlas_out);
-    if (adam)
-        requantize_kernel<true><<<grid, 256, 0, st>>>(ind, blk_of_slot, reinterpret_cast<float4*>(values),
-                                                      reinterpret_cast<float4*>(m), reinterpret_cast<float4*>(v),
-                                                      reinterpret_cast<const float4*>(g), nb, N, B, lgB, pa, out, *adam);
-    else
-        requantize_kernel<false><<<grid, 256, 0, st>>>(ind, blk_of_slot, reinterpret_cast<float4*>(values), nullptr,
-                                                       nullptr, nullptr, nb, N, B, lgB, pa, out, AdamArgs{});
+    const int64_t total = nb * (int64_t)(B + 2) * (B + 2) * (B + 2);
+    requantize_padded_kernel<<<grid_for(total), 256, 0, st>>>(ind, blk_of_slot, reinterpret_cast<const float4*>(values),
+                                                              nb, N, B, lgB, patlas, reinterpret_cast<uint2*>(atlas_out));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adam_requantize(const int32_t* ind, const int32_t* blk_of_slot, float* values, float* m, float* v,
+                                   const float* g, const AdamArgs& adam, int64_t nb, int N, int B, int lgB,
+                                   uint2* patlas, uint8_t* atlas_out, cudaStream_t st) {
+    if (nb <= 0) return cudaSuccess;
+    adam_requantize_kernel<<<grid_for(nb << (3 * lgB + 1)), 256, 0, st>>>(
+        ind, blk_of_slot, reinterpret_cast<float4*>(values), reinterpret_cast<float4*>(m), reinterpret_cast<float4*>(v),
+        reinterpret_cast<const float4*>(g), nb, N, B, lgB, reinterpret_cast<uint32_t*>(patlas),
+        reinterpret_cast<uint32_t*>(atlas_out), adam);
     return cudaGetLastError();
 }
 }  // namespace snerg
