@@ -1031,16 +1031,16 @@ struct AdamArgs {
 
 // One Adam step on four parameters: m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
 // p -= lr (m / c1) / (sqrt(v / c2) + eps). Where gradient and moments are all zero nothing
-// changes (finite lr), and false is returned: most voxels of a fine-tuned grid are never
-// touched, and three exact divisions and a root per parameter are what such a pass would be
-// bound by.
-__device__ __forceinline__ bool adam_quad(const AdamArgs& a, const float4& g, float4& m, float4& v, float4& p) {
+// changes (finite lr): most voxels of a fine-tuned grid are never touched.
+__device__ __forceinline__ bool adam_untouched(const AdamArgs& a, const float4& g, const float4& m, const float4& v) {
+    const uint32_t bits = __float_as_uint(g.x) | __float_as_uint(g.y) | __float_as_uint(g.z) | __float_as_uint(g.w) |
+                          __float_as_uint(m.x) | __float_as_uint(m.y) | __float_as_uint(m.z) | __float_as_uint(m.w) |
+                          __float_as_uint(v.x) | __float_as_uint(v.y) | __float_as_uint(v.z) | __float_as_uint(v.w);
+    return bits == 0u && a.lr < INFINITY;
+}
+__device__ __forceinline__ void adam_quad(const AdamArgs& a, const float4& g, float4& m, float4& v, float4& p) {
     const float ga[4] = {g.x, g.y, g.z, g.w};
     float ma[4] = {m.x, m.y, m.z, m.w}, va[4] = {v.x, v.y, v.z, v.w}, pa[4] = {p.x, p.y, p.z, p.w};
-    uint32_t bits = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) bits |= __float_as_uint(ga[k]) | __float_as_uint(ma[k]) | __float_as_uint(va[k]);
-    if (bits == 0u && a.lr < INFINITY) return false;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         ma[k] = a.b1 * ma[k] + (1.0f - a.b1) * ga[k];
@@ -1050,7 +1050,6 @@ __device__ __forceinline__ bool adam_quad(const AdamArgs& a, const float4& g, fl
     m = make_float4(ma[0], ma[1], ma[2], ma[3]);
     v = make_float4(va[0], va[1], va[2], va[3]);
     p = make_float4(pa[0], pa[1], pa[2], pa[3]);
-    return true;
 }
 
 // host: the constants, false for arguments snerg_adam_step refuses

@@ -100,7 +100,10 @@ __global__ void __launch_bounds__(256) adam_requantize_kernel(const int32_t* __r
         const float4 gi = __ldcs(g + t);
         const uint32_t old = *own;
         const int blk = __ldg(blk_of_slot + slot);
-        if (adam_quad(a, gi, mi, vi, x)) {
+        // three exact divisions and a root per parameter: a pass over mostly untouched values would
+        // be bound by them
+        if (!adam_untouched(a, gi, mi, vi)) {
+            adam_quad(a, gi, mi, vi, x);
             m[t] = mi;
             v[t] = vi;
             values[t] = x;
