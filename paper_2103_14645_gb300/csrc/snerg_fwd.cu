@@ -47,8 +47,8 @@ __host__ __device__ __forceinline__ int packet_width_log2(int lanes) {
 // the launch's start and end. The grid is nt + 4 smax CTAs: 4 smax sparse slots (S <= smax
 // used), then nt dense slots for the tiles S .. nt - 1 of the order (the last S idle).
 // A small image (lanes_per_warp) has `parts` CTAs per dense slot, each a band of the tile's rows
-// with 32 / parts rays per warp, and no sparse slots where that is as few; the first band's
-// duration stands for the tile's.
+// with 32 / parts rays per warp, and no sparse slots; the first band's duration stands for the
+// tile's.
 struct SchedSlot {
     int tile;       // -1: idle
     int quarter;    // -1: dense
@@ -385,21 +385,19 @@ cudaError_t Forward<LGB, A>::image(const DevScene& ds, const snerg_camera& cam, 
     return cudaGetLastError();
 }
 
-// A list is spread over the warps of one wave of 7 CTAs per SM: scattered rays have less in
-// common than an image's, and a second wave costs as much as the first (4,096 rays of a 1024^3
-// grid 122 us with 32 rays per warp, 70 with 1; 16,384: 131 and, with 4, 102; 65,536: 143 with
-// 32, 145 with 16, 150 with 8; 262,144: 274, 324 with 16); with debug outputs, which need more
-// registers, over one wave of 4. If 4 CTAs per SM hold it, it runs the build limited to 4 (the march
-// keeps its state in registers, and a single wave gains nothing from more CTAs); longer lists
-// keep 7 CTAs per SM to hide the march's latencies: 8 spill with the weights in device memory
-// (131,072 and 262,144 rays of a 1024^3 grid 163 and 277 us with 8, 153 and 268 with 7; 1,000,000
-// rays 731 and 747).
+// A short list is spread over 14 warps per SM (3.5 CTAs): 16,000 scattered rays of a 1024^3 grid
+// 76 us with 32 rays per warp, 53 with 8; beyond it 32 rays per warp are as good or better (52,000
+// rays with 32 / 16: 1024^3 90 / 97 us, 128^3 58 / 65). If 4 CTAs per SM hold the list, it runs the build
+// limited to 4 (the march keeps its state in registers, and a single wave gains nothing from more
+// CTAs); longer lists keep 7 CTAs per SM to hide the march's latencies: 8 spill with the weights in
+// device memory (131,072 and 262,144 rays of a 1024^3 grid 163 and 277 us with 8, 153 and 268 with
+// 7; 1,000,000 rays 731 and 747).
 template <int LGB, int A>
 cudaError_t Forward<LGB, A>::rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
                                const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, float2* record,
                                cudaStream_t st) {
     const bool d = dbg.aux || dbg.counts || dbg.trace;
-    const int lanes = lanes_per_warp(n, (int64_t)s.sms * (d ? 4 : 7) * 4);
+    const int lanes = lanes_per_warp(n, (int64_t)s.sms * 14);
     const bool one_wave = n <= (int64_t)s.sms * 4 * 4 * lanes;
     auto* kernel = pw ? (one_wave ? render_rays_kernel<LGB, A, false, true, 4> : render_rays_kernel<LGB, A, false, true, 7>)
                       : (one_wave ? render_rays_kernel<LGB, A, false, false, 4> : render_rays_kernel<LGB, A, false, false, 7>);

@@ -132,7 +132,9 @@ inline auto with_block_build(const DevScene& s, F&& f) {
 // (a power of two) as still make no more than that many warps; the other lanes idle. A launch
 // that leaves the chip part empty is as slow as its slowest warps, whose lanes wait for one
 // another at every branch of their rays' chains of dependent loads: with fewer rays beside it a
-// ray's chain is shorter, and the warps it costs have room. The launches say how many they take.
+// ray's chain is shorter, and the warps it costs have room. The launches say how many they take:
+// no more than were at no size slower than 32 rays per warp on grids of 128^3 to 2048^3. The rule
+// takes a launch to be alone on the GPU: beside others the idle lanes' issue slots are lost to those.
 inline int lanes_per_warp(int64_t n, int64_t warps) {
     int lanes = 32;
     while (lanes > 1 && n <= warps * (lanes / 2)) lanes /= 2;
@@ -967,15 +969,22 @@ struct SchedArgs {
     int32_t nt;                // the image's tiles
     int32_t tiles_x;
     int32_t smax;              // sparse slots of this launch (0 without previous buckets)
-    int32_t parts;             // CTAs per dense tile (1, 2, 4, 8: bands of its rows)
+    int32_t parts;             // CTAs per dense tile (1 or 8: bands of its rows)
 };
 
-// Rays per warp of a one-camera launch of n pixels: up to three waves of warps. 40,000 pixels of a
-// 1024^3 grid take 202 us with 32 rays per warp, 134 with 8 and 118 with 4 (2.1 waves); 160,000 take
-// 201, 171 with 16 (2.1) and 164 with 8 (4.1), but of a 512^3 grid 108, 102 and 111; from 470,000
-// on 32 is the best or within 5 % of it.
+// The grid's side as the rules for the rays per warp take it: the longer a ray's chain, the more a
+// warp's lanes wait for one another and the more issue slots it leaves to other warps.
+inline int64_t chain_side(const DevScene& s) { return s.N < 288 ? 288 : (s.N > 768 ? 768 : s.N); }
+
+// Rays per warp of a one-camera launch of n pixels:
+// up to 3/4 of a wave of warps in grids of up to 288^3, two waves from 768^3 on, in proportion
+// between. 38,809 pixels with 32 / 16 / 8 / 4 rays per warp: of a 1024^3 grid 102 / 101 / 87 / 71 us
+// (4: two waves), of a 512^3 one 93 / 82 / 62 / 64; 136,900 pixels with 32 / 16 (1.8 waves): of a
+// 1024^3 grid 123 / 104, 2048^3 243 / 209, but 256^3 60 / 69 and 128^3 45 / 53.
 constexpr int kImageWarps = 4;     // warps per CTA of the one-camera launch
-inline int image_lanes(const DevScene& s, int64_t n) { return lanes_per_warp(n, (int64_t)s.sms * 8 * kImageWarps * 3); }
+inline int image_lanes(const DevScene& s, int64_t n) {
+    return lanes_per_warp(n, (int64_t)s.sms * 8 * kImageWarps * chain_side(s) / 384);
+}
 
 inline const MlpWeights& no_weights() {
     static const MlpWeights z = {};

@@ -1,7 +1,8 @@
 """Launches that leave the chip part empty run fewer rays per warp (1, 2, 4, 8 or 16 lanes). Which
 rays share a warp changes no ray: images, row ranges, scheduled frames and ray lists of every
-size class are compared bit for bit with launches of 32 rays per warp, and the adjoint's sums
-(which rows a thread block adds up depends on the lanes) with the same rays in many small calls."""
+size class, on both sides of each class's limit, are compared bit for bit with launches of 32 rays
+per warp, and the adjoint's sums (which rows a thread block adds up depends on the lanes) with the
+same rays in many small calls. The sizes follow from the launch rules and the device's SMs."""
 import numpy as np
 import pytest
 import torch
@@ -10,6 +11,19 @@ from paper_2103_14645_gb300 import renderer, synth
 
 pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda:0")
+LANES = (1, 2, 4, 8, 16)
+N = 64                                                     # the scene's grid
+
+
+def _warps(rule):
+    """Warps that a launch spreads its rays over: lanes l for up to l times as many rays."""
+    sms = torch.cuda.get_device_properties(DEV).multi_processor_count
+    side = min(max(N, 288), 768)
+    return {"image": sms * 32 * side // 384, "list": sms * 14, "adjoint": sms * (1152 + side) // 120}[rule]
+
+
+def _lanes(n, rule):
+    return next((l for l in LANES if n <= _warps(rule) * l), 32)
 
 
 @pytest.fixture(scope="module")
@@ -24,16 +38,27 @@ def _camera(W, H):
     return np.asarray([synth.look_at_camera((1.5, -1.1, 0.9), (0.0, 0.0, 0.0), W, H, 45.0, 0)])
 
 
-@pytest.mark.parametrize("W,H", [(1, 1), (7, 3), (61, 37), (123, 111), (199, 143), (283, 205), (401, 283), (640, 479),
-                                 (1021, 523)])
-def test_images_of_every_size_class(scene, W, H):
+def _image(lanes, over):
+    """A ragged image of `lanes` rays per warp, near the class's limit, or the next class (over)."""
+    n = _warps("image") * min(lanes, 16)
+    W = int((4 * n / 3) ** 0.5) | 1
+    H = n // W
+    if over:
+        H += 1 + (n - W * H == 0)
+    assert _lanes(W * H, "image") == (32 if over and lanes == 16 else 2 * lanes if over else lanes)
+    return W, H
+
+
+@pytest.mark.parametrize("size", [(1, 1), (7, 3), (61, 37)] + [(l, over) for l in LANES for over in (False, True)])
+def test_images_of_every_size_class(scene, size):
+    W, H = _image(*size) if isinstance(size[1], bool) else size
     _, r, w = scene
     cam = _camera(W, H)
     want = r.render(cam, w, counts=True)["rgb"]            # debug outputs: 32 rays per warp
     assert torch.equal(r.render(cam, w), want)
     stored = r.render(cam, None, counts=True)["rgb"]
     assert torch.equal(r.render(cam, None), stored)
-    for _ in range(2):
+    for _ in range(3):
         assert torch.equal(r.render(cam, None, schedule=True), stored)
     rows = (H // 3, H - H // 4)
     out = torch.full((W * H, 3), -1.0, device=DEV)
@@ -45,8 +70,10 @@ def test_images_of_every_size_class(scene, W, H):
     r.check_status()
 
 
-@pytest.mark.parametrize("n", [1, 33, 4864, 4865, 9729, 19457, 38913, 77825, 155649])
-def test_ray_lists_of_every_size_class(scene, n):
+@pytest.mark.parametrize("lanes,more", [(0, 1), (0, 33)] + [(l, more) for l in LANES for more in (0, 1)] + [(36, 1)])
+def test_ray_lists_of_every_size_class(scene, lanes, more):
+    n = _warps("list") * lanes + more                      # 36: beyond one wave of 4 CTAs per SM
+    assert lanes in (0, 36) or _lanes(n, "list") == (lanes if not more else 2 * lanes)
     _, r, w = scene
     cam = _camera(1021, 523)
     image = r.render(cam, w, counts=True)["rgb"]
@@ -59,8 +86,10 @@ def test_ray_lists_of_every_size_class(scene, n):
     r.check_status()
 
 
-@pytest.mark.parametrize("n", [5, 2432, 2433, 4865, 9729, 19457, 38913])
-def test_adjoint_sums_of_every_size_class(scene, n):
+@pytest.mark.parametrize("lanes,more", [(0, 5)] + [(l, more) for l in LANES for more in (0, 1)])
+def test_adjoint_sums_of_every_size_class(scene, lanes, more):
+    n = _warps("adjoint") * lanes + more
+    assert lanes == 0 or _lanes(n, "adjoint") == (lanes if not more else 2 * lanes)
     sc, r, w = scene
     cam = _camera(640, 479)
     rng = np.random.default_rng(n)
