@@ -9,6 +9,7 @@
 
 #include <chrono>
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -103,6 +104,29 @@ struct PersistentConfig {
     }
 };
 
+// The streams of a handle's last one-camera launches, and from them how many such launches are
+// taken to be on the chip together: half as many as there are different streams (two streams'
+// launches, or a warm-up and a capture, are as fast as a launch alone). Which colours a call gives
+// does not depend on it; host threads that write it at once only blur the count. 16 views of
+// 390x390 pixels of a 1024^3 grid on 16 streams take 0.63 ms, and 0.73 if each is taken to be alone.
+struct RecentStreams {
+    static constexpr int kKept = 8;
+    std::atomic<uintptr_t> kept[kKept] = {};
+    std::atomic<uint32_t> calls{0};
+    int share(cudaStream_t st) {
+        const uint32_t c = calls.fetch_add(1, std::memory_order_relaxed);
+        kept[c % kKept].store((uintptr_t)st, std::memory_order_relaxed);
+        const int n = c < kKept ? (int)c + 1 : kKept;
+        uintptr_t now[kKept];
+        int different = 0;
+        for (int i = 0; i < n; ++i) {
+            now[i] = kept[i].load(std::memory_order_relaxed);
+            different += std::find(now, now + i, now[i]) == now + i;
+        }
+        return std::max(1, different / 2);
+    }
+};
+
 struct GraphEntry {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -130,6 +154,7 @@ struct snerg_scene {
     int32_t sched_w = 0, sched_h = 0;
     int sched_set = 0;
     bool sched_valid = false;
+    RecentStreams image_streams;
     std::vector<cudaStream_t> band_streams;   // snerg_render_to_host: one per band
     std::vector<cudaEvent_t> band_done;
     cudaEvent_t band_fork = nullptr;
@@ -227,14 +252,14 @@ namespace snerg {
 // debug outputs and the per-sample model are in build 0
 cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
                                 float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1,
-                                const SchedArgs* sch) {
+                                const SchedArgs* sch, int share) {
     row0 = std::max(row0, 0);
     row1 = std::min(row1, cam.H);
     if (cam.W <= 0 || row1 <= row0) return cudaSuccess;
     if (dbg.aux || dbg.counts || dbg.trace || (s.flags & SNERG_FLAG_PER_SAMPLE_MLP))
-        return Forward<0, kAnyAlpha>::image(s, cam, mlp, pw, rgb, dbg, st, row0, row1, nullptr);
+        return Forward<0, kAnyAlpha>::image(s, cam, mlp, pw, rgb, dbg, st, row0, row1, nullptr, share);
     return with_block_build(s, [&](auto b) {
-        return Forward<decltype(b)::lgB, decltype(b)::alpha>::image(s, cam, mlp, pw, rgb, dbg, st, row0, row1, sch);
+        return Forward<decltype(b)::lgB, decltype(b)::alpha>::image(s, cam, mlp, pw, rgb, dbg, st, row0, row1, sch, share);
     });
 }
 
@@ -511,7 +536,7 @@ extern "C" snerg_status snerg_render(snerg_handle h, const snerg_camera* cams, i
         // where it takes 4 rays per warp or fewer: 25,600 pixels of a 1024^3 grid 75 -> 67 us; 2 or 4
         // CTAs gain nothing over the sparse tiles: 115,600 pixels 94 us, with 2 97, with 4 99). Sparse
         // slots only with a previous frame to choose the slow tiles from
-        sa.parts = image_lanes(h->ds, (int64_t)cams[0].W * cams[0].H) <= 4 ? 8 : 1;
+        sa.parts = image_lanes(h->ds, (int64_t)cams[0].W * cams[0].H, 1) <= 4 ? 8 : 1;
         sa.smax = use && sa.parts == 1 ? std::min(kSchedMaxSparse, std::max(1, tiles / 8)) : 0;
         cudaError_t e = cudaMemsetAsync(wr, 0, kSchedCountBytes, st);
         if (e == cudaSuccess) e = launch_render_image(h->ds, cams[0], d_mlp, pw, d_rgb, dbg, st, 0, cams[0].H, &sa);
@@ -523,11 +548,12 @@ extern "C" snerg_status snerg_render(snerg_handle h, const snerg_camera* cams, i
         h->sched_valid = true;
         return SNERG_OK;
     }
+    const int share = h->image_streams.share(st);
     for (int i = 0; i < n_cams; ++i) {
         if (cams[i].W == 0 || cams[i].H == 0) continue;
         const int r0 = rows ? opts->row_begin : 0, r1 = rows ? opts->row_end : cams[i].H;
         if (std::min(r1, cams[i].H) <= r0) continue;
-        cudaError_t e = launch_render_image(h->ds, cams[i], d_mlp, pw, d_rgb, dbg, st, r0, r1);
+        cudaError_t e = launch_render_image(h->ds, cams[i], d_mlp, pw, d_rgb, dbg, st, r0, r1, nullptr, share);
         if (e != cudaSuccess) return SNERG_E_CUDA;
         h->launches++;
     }
@@ -557,9 +583,10 @@ extern "C" snerg_status snerg_render_to_host(snerg_handle h, const snerg_camera*
     cudaPointerAttributes pa;
     if (cudaPointerGetAttributes(&pa, h_rgb) == cudaSuccess && pa.type == cudaMemoryTypeHost && pa.devicePointer) {
         float* mapped = (float*)pa.devicePointer;
+        const int share = h->image_streams.share(st);
         for (int i = 0; i < n_cams; ++i) {
             if (cams[i].W == 0 || cams[i].H == 0) continue;
-            if (launch_render_image(h->ds, cams[i], d_mlp, pw, mapped, dbg, st, 0, cams[i].H) != cudaSuccess)
+            if (launch_render_image(h->ds, cams[i], d_mlp, pw, mapped, dbg, st, 0, cams[i].H, nullptr, share) != cudaSuccess)
                 return SNERG_E_CUDA;
             h->launches++;
         }

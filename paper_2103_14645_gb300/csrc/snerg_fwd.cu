@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(128, 8) render_persistent_kernel(const BlockSc
 template <int LGB, int A>
 cudaError_t Forward<LGB, A>::image(const DevScene& ds, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
                                 float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1,
-                                const SchedArgs* sch) {
+                                const SchedArgs* sch, int share) {
     using T = ImageTile<kImageWarps>;
     const BlockScene<LGB, A> s(ds);
     const int nt = 32 * kImageWarps;
@@ -362,7 +362,7 @@ cudaError_t Forward<LGB, A>::image(const DevScene& ds, const snerg_camera& cam, 
                                                                                *sch);
         return cudaGetLastError();
     }
-    const int lanes = ps || d ? 32 : image_lanes(ds, (int64_t)cam.W * (row1 - row0));
+    const int lanes = ps || d ? 32 : image_lanes(ds, (int64_t)cam.W * (row1 - row0), share);
     const int tw = T::WX << packet_width_log2(lanes), th = T::WY * (lanes >> packet_width_log2(lanes));
     const dim3 grid((cam.W + tw - 1) / tw, (row1 - row0 + th - 1) / th);
     auto* kernel = pw ? render_image_kernel<LGB, A, false, true, kImageWarps, false>

@@ -133,8 +133,9 @@ inline auto with_block_build(const DevScene& s, F&& f) {
 // that leaves the chip part empty is as slow as its slowest warps, whose lanes wait for one
 // another at every branch of their rays' chains of dependent loads: with fewer rays beside it a
 // ray's chain is shorter, and the warps it costs have room. The launches say how many they take:
-// no more than were at no size slower than 32 rays per warp on grids of 128^3 to 2048^3. The rule
-// takes a launch to be alone on the GPU: beside others the idle lanes' issue slots are lost to those.
+// no more than were at no size slower than 32 rays per warp on grids of 128^3 to 2048^3. Beside
+// other launches the idle lanes' issue slots are lost to those; what a launch cannot know of (other
+// handles' and other programs' launches) is taken not to be there.
 inline int lanes_per_warp(int64_t n, int64_t warps) {
     int lanes = 32;
     while (lanes > 1 && n <= warps * (lanes / 2)) lanes /= 2;
@@ -976,14 +977,14 @@ struct SchedArgs {
 // warp's lanes wait for one another and the more issue slots it leaves to other warps.
 inline int64_t chain_side(const DevScene& s) { return s.N < 288 ? 288 : (s.N > 768 ? 768 : s.N); }
 
-// Rays per warp of a one-camera launch of n pixels:
+// Rays per warp of a one-camera launch of n pixels (with `share` of its kind on the chip at a time):
 // up to 3/4 of a wave of warps in grids of up to 288^3, two waves from 768^3 on, in proportion
 // between. 38,809 pixels with 32 / 16 / 8 / 4 rays per warp: of a 1024^3 grid 102 / 101 / 87 / 71 us
 // (4: two waves), of a 512^3 one 93 / 82 / 62 / 64; 136,900 pixels with 32 / 16 (1.8 waves): of a
 // 1024^3 grid 123 / 104, 2048^3 243 / 209, but 256^3 60 / 69 and 128^3 45 / 53.
 constexpr int kImageWarps = 4;     // warps per CTA of the one-camera launch
-inline int image_lanes(const DevScene& s, int64_t n) {
-    return lanes_per_warp(n, (int64_t)s.sms * 8 * kImageWarps * chain_side(s) / 384);
+inline int image_lanes(const DevScene& s, int64_t n, int share) {
+    return lanes_per_warp(n * share, (int64_t)s.sms * 8 * kImageWarps * chain_side(s) / 384);
 }
 
 inline const MlpWeights& no_weights() {
@@ -995,12 +996,12 @@ inline const MlpWeights& no_weights() {
 // pw: weights as a kernel parameter (nullptr: read them from `mlp` in device memory).
 // image: rows [row0, row1); sch: nullable; with it the launch takes its tile order from the
 // previous frame's buckets and records its own tile costs (deferred model, all rows, no debug
-// outputs). rays: record: nullable, with debug outputs and device weights.
+// outputs); share: see image_lanes. rays: record: nullable, with debug outputs and device weights.
 struct PersistentParams;
 template <int LGB, int A>
 struct Forward {
     static cudaError_t image(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw, float* rgb,
-                             const DebugOut& dbg, cudaStream_t st, int row0, int row1, const SchedArgs* sch);
+                             const DebugOut& dbg, cudaStream_t st, int row0, int row1, const SchedArgs* sch, int share);
     static cudaError_t rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
                             const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, float2* record,
                             cudaStream_t st);
@@ -1021,7 +1022,7 @@ struct Adjoint {
 // snerg_api.cu: the build for the scene
 cudaError_t launch_render_image(const DevScene& s, const snerg_camera& cam, const float* mlp, const MlpWeights* pw,
                                 float* rgb, const DebugOut& dbg, cudaStream_t st, int row0, int row1,
-                                const SchedArgs* sch = nullptr);
+                                const SchedArgs* sch = nullptr, int share = 1);
 cudaError_t launch_validate(const int32_t* ind, int64_t n_ind, int64_t nb, int32_t* blk_of_slot, int32_t* err,
                             cudaStream_t st);
 // the padded atlas and the 8 octants' voxel-distance planes of every stored block; a launch

@@ -116,3 +116,21 @@ def test_adjoint_sums_of_every_size_class(scene, lanes, more):
         assert float((a - b).abs().max()) <= 2e-5 * scale + 1e-7
     assert float((whole[2] - whole[4]).abs().max()) <= 2e-5 * float(whole[2].abs().max())
     r.check_status()
+
+
+def test_images_on_several_streams(scene):
+    """A handle whose images come in on several streams gives them more rays per warp again (here 8
+    and 16 instead of 4, beside the 4 of the first calls): the same colours."""
+    _, r, _ = scene
+    W, H = _image(4, False)
+    cam = _camera(W, H)
+    want = r.render(cam, None, counts=True)["rgb"]
+    streams = [torch.cuda.Stream() for _ in range(8)]
+    torch.cuda.synchronize()
+    for _ in range(2):
+        outs = []
+        for s in streams:
+            with torch.cuda.stream(s):
+                outs.append(r.render(cam, None))
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, want) for o in outs)
