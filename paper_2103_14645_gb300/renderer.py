@@ -473,11 +473,15 @@ class SnergRenderFn(torch.autograd.Function):
     density channel (0) frozen at zero."""
 
     @staticmethod
-    def forward(ctx, mlp, atlas_values, renderer, cams, pix):
+    def forward(ctx, mlp, atlas_values, renderer, cams, pix, grad=True):
+        """grad: False under torch.no_grad(), which neither this call nor ctx.needs_input_grad shows:
+        nothing is kept for a backward that cannot come."""
         ctx.renderer = renderer
         ctx.cams = cams
         ctx.atlas_shape = atlas_values.shape
         w = mlp.detach().contiguous()
+        if not grad:
+            return renderer.render_rays(cams, pix, w)
         # per-ray state for the backward: with the composited samples if they are to be scattered
         if ctx.needs_input_grad[1]:
             rgb, state = renderer.render_rays_recorded(cams, pix, w)
@@ -496,17 +500,17 @@ class SnergRenderFn(torch.autograd.Function):
             g_atl = torch.empty(ctx.atlas_shape, dtype=torch.float32, device=r.device)
             g_mlp = torch.empty(MLP_PARAMS, dtype=torch.float32, device=r.device) if ctx.needs_input_grad[0] else None
             r.backward_recorded(ctx.cams, pix, w, g, state[0], g_atl, g_mlp)
-            return g_mlp, g_atl, None, None, None
+            return g_mlp, g_atl, None, None, None, None
         g_mlp = None
         if ctx.needs_input_grad[0]:
             g_mlp = torch.zeros(MLP_PARAMS, dtype=torch.float32, device=r.device)
             r.backward(ctx.cams, pix, w, g, None, g_mlp, fwd_aux=state[0], fwd_counts=state[1])
-        return g_mlp, None, None, None, None
+        return g_mlp, None, None, None, None, None
 
 
 def render_rays_autograd(renderer: Renderer, cams, pix: torch.Tensor, mlp: torch.Tensor,
                          atlas_values: torch.Tensor) -> torch.Tensor:
-    return SnergRenderFn.apply(mlp, atlas_values, renderer, cams, pix)
+    return SnergRenderFn.apply(mlp, atlas_values, renderer, cams, pix, torch.is_grad_enabled())
 
 
 def l2_loss(rgb: torch.Tensor, target: torch.Tensor, grad: torch.Tensor | None = None,

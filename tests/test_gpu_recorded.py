@@ -99,3 +99,23 @@ def test_no_rays_and_arguments():
     ga = torch.ones(sc.atlas.shape, device=DEV)
     r.backward_recorded(sc.cameras, pix[:0], w, rgb, state, ga, gm)
     assert rgb.shape == (0, 3) and not bool(ga.any()) and not bool(gm.any())
+
+
+def test_no_state_is_kept_without_a_backward():
+    sc = _scene(0, 0.3, 4)
+    r = renderer.Renderer.from_scene(sc, DEV)
+    n = 200000
+    pix = torch.from_numpy(synth.random_pixels(np.random.default_rng(1), sc.cameras, n)).to(DEV)
+    w = torch.from_numpy(sc.mlp).to(DEV).requires_grad_()
+    vals = (torch.from_numpy(sc.atlas).to(DEV).float() / 255.0).requires_grad_()
+    want = renderer.render_rays_autograd(r, sc.cameras, pix, w, vals)
+    assert want.requires_grad
+    torch.cuda.synchronize()
+    torch.cuda.reset_peak_memory_stats()
+    before = torch.cuda.memory_allocated()
+    with torch.no_grad():
+        rgb = renderer.render_rays_autograd(r, sc.cameras, pix, w, vals)
+    assert torch.equal(rgb, want) and not rgb.requires_grad
+    assert torch.cuda.max_memory_allocated() - before <= 12 * n + (2 << 20)       # the colours
+    with torch.inference_mode():
+        assert torch.equal(renderer.render_rays_autograd(r, sc.cameras, pix, w, vals), want)
