@@ -17,6 +17,10 @@ from . import synth
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsnerg.so")
 MLP_PARAMS = 883
+# Rays up to which a render whose atlas gradient is wanted records its composited samples for the
+# adjoint: 312 bytes per ray until the backward, 1.3 GB at the limit. More rays keep 48 bytes each
+# and the adjoint marches them again (4 M rays: a pass of 4.68 ms recorded, 5.33 marched again).
+RECORD_MAX_RAYS = 1 << 22
 FLAG_UNPREMULTIPLY = 1
 FLAG_PER_SAMPLE_MLP = 2
 FLAG_ALPHA_ATLAS = 4
@@ -483,7 +487,7 @@ class SnergRenderFn(torch.autograd.Function):
         if not grad:
             return renderer.render_rays(cams, pix, w)
         # per-ray state for the backward: with the composited samples if they are to be scattered
-        if ctx.needs_input_grad[1]:
+        if ctx.needs_input_grad[1] and pix.shape[0] <= RECORD_MAX_RAYS:
             rgb, state = renderer.render_rays_recorded(cams, pix, w)
             ctx.save_for_backward(mlp, pix, state)
             return rgb
@@ -496,16 +500,14 @@ class SnergRenderFn(torch.autograd.Function):
         mlp, pix, *state = ctx.saved_tensors
         r = ctx.renderer
         w, g = mlp.detach().contiguous(), grad_rgb.contiguous().float()
-        if ctx.needs_input_grad[1]:
-            g_atl = torch.empty(ctx.atlas_shape, dtype=torch.float32, device=r.device)
-            g_mlp = torch.empty(MLP_PARAMS, dtype=torch.float32, device=r.device) if ctx.needs_input_grad[0] else None
+        new = torch.empty if len(state) == 1 else torch.zeros        # the recorded adjoint clears its sums
+        g_mlp = new(MLP_PARAMS, dtype=torch.float32, device=r.device) if ctx.needs_input_grad[0] else None
+        g_atl = new(ctx.atlas_shape, dtype=torch.float32, device=r.device) if ctx.needs_input_grad[1] else None
+        if len(state) == 1:
             r.backward_recorded(ctx.cams, pix, w, g, state[0], g_atl, g_mlp)
-            return g_mlp, g_atl, None, None, None, None
-        g_mlp = None
-        if ctx.needs_input_grad[0]:
-            g_mlp = torch.zeros(MLP_PARAMS, dtype=torch.float32, device=r.device)
-            r.backward(ctx.cams, pix, w, g, None, g_mlp, fwd_aux=state[0], fwd_counts=state[1])
-        return g_mlp, None, None, None, None, None
+        elif g_mlp is not None or g_atl is not None:
+            r.backward(ctx.cams, pix, w, g, g_atl, g_mlp, fwd_aux=state[0], fwd_counts=state[1])
+        return g_mlp, g_atl, None, None, None, None
 
 
 def render_rays_autograd(renderer: Renderer, cams, pix: torch.Tensor, mlp: torch.Tensor,
@@ -639,17 +641,19 @@ class FineTuner:
             if ga is not None:
                 ga.zero_()
             self.r.train_rays(cams, pix, self.mlp, target, ga, self.grad, loss=self.loss)
-        elif ga is not None:
+        elif ga is not None and pix.shape[0] <= RECORD_MAX_RAYS:
             # larger batches: the forward at its own (higher) occupancy, keeping per-ray state
             rgb, state = self.r.render_rays_recorded(cams, pix, self.mlp)
             g = torch.empty_like(rgb)
             l2_loss(rgb, target, g, self.loss)
             self.r.backward_recorded(cams, pix, self.mlp, g, state, ga, self.grad)
         else:
+            if ga is not None:
+                ga.zero_()
             fwd = self.r.render_rays(cams, pix, self.mlp, aux=True, counts=True)
             g = torch.empty_like(fwd["rgb"])
             l2_loss(fwd["rgb"], target, g, self.loss)
-            self.r.backward(cams, pix, self.mlp, g, None, self.grad, fwd_aux=fwd["aux"], fwd_counts=fwd["counts"])
+            self.r.backward(cams, pix, self.mlp, g, ga, self.grad, fwd_aux=fwd["aux"], fwd_counts=fwd["counts"])
         if _data_parallel(self.group):
             allreduce_gradients(self.grad, ga, self.group)
         self.steps += 1

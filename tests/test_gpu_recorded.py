@@ -101,6 +101,32 @@ def test_no_rays_and_arguments():
     assert rgb.shape == (0, 3) and not bool(ga.any()) and not bool(gm.any())
 
 
+def test_rays_beyond_the_record_limit_keep_the_small_state(monkeypatch):
+    sc = _scene(0, 0.3, 4)
+    r = renderer.Renderer.from_scene(sc, DEV)
+    n = 60000
+    pix = torch.from_numpy(synth.random_pixels(np.random.default_rng(1), sc.cameras, n)).to(DEV)
+    w = torch.from_numpy(sc.mlp).to(DEV).requires_grad_()
+    vals = (torch.from_numpy(sc.atlas).to(DEV).float() / 255.0).requires_grad_()
+    target = torch.rand((n, 3), device=DEV, generator=torch.Generator(device=DEV).manual_seed(1))
+    grads, kept, moments = [], [], []
+    for limit in (n, n - 1):
+        monkeypatch.setattr(renderer, "RECORD_MAX_RAYS", limit)
+        before = torch.cuda.memory_allocated()
+        rgb = renderer.render_rays_autograd(r, sc.cameras, pix, w, vals)
+        kept.append(torch.cuda.memory_allocated() - before)
+        grads.append(torch.autograd.grad(rgb, (w, vals), rgb.detach() - target))
+        del rgb
+        ft = renderer.FineTuner(r, sc.mlp, atlas=sc.atlas, atlas_lr=0.0)
+        ft.fused_rays = 0
+        ft.step(sc.cameras, pix, target)
+        moments.append((ft.m.clone(), ft.ma.clone()))
+    assert kept[0] >= (12 + 312) * n and kept[1] <= (12 + 48) * n + 4096
+    for a, b in (grads, moments):
+        for x, y in zip(a, b):
+            assert float((x - y).abs().max()) <= 2e-5 * float(y.abs().max())
+
+
 def test_no_state_is_kept_without_a_backward():
     sc = _scene(0, 0.3, 4)
     r = renderer.Renderer.from_scene(sc, DEV)
