@@ -417,6 +417,8 @@ cudaError_t Forward<LGB, A>::rays(const DevScene& s, const CamTable& cams, int32
 
 template <int LGB, int A>
 const void* Forward<LGB, A>::persistent_fn(bool param_weights, bool multi) {
+    // the launches through this pointer pass a DevScene as the kernel's scene
+    static_assert(sizeof(BlockScene<LGB, A>) == sizeof(DevScene), "a build's scene adds no member");
     if (param_weights)
         return multi ? (const void*)render_persistent_kernel<LGB, A, true, true>
                      : (const void*)render_persistent_kernel<LGB, A, true, false>;
