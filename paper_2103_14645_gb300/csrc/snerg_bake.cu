@@ -32,7 +32,7 @@
 namespace bake_gpu {
 
 constexpr int kMaxBlobs = SNERG_BAKE_MAX_BLOBS;
-constexpr int kThreads = 256;
+constexpr int kThreads = 64;           // of the kernels for blocks below 8^3 (gather_blobs takes 64)
 constexpr int kScanThreads = 1024;
 constexpr int kMaxG = 256;
 constexpr size_t kAlign = 256;
@@ -40,8 +40,6 @@ constexpr size_t kAlign = 256;
 struct BakeParams {
     int32_t N, B, lgB, G;
     int32_t n_blob;
-    int32_t item_voxels;        // min(256, B^3)
-    int32_t lg_items;           // log2(B^3 / item_voxels)
     int32_t alpha_codes;        // channel 0 = 1 - exp(-sigma v) instead of sigma / sigma_max
     float v, tau, inv_sigma_max;
     float sigma_reject;         // a block whose density is below this everywhere is not kept
@@ -59,25 +57,14 @@ struct ItemBox {
     int32_t lo[3], hi[3];       // inclusive global voxel ranges of the item
 };
 
-// Voxel ranges covered by voxels [l0, l0 + iv) of block (bx, by, bz), local order
-// z-major then y then x: a partial row, whole rows of one slice, or whole slices.
-__device__ __forceinline__ ItemBox item_box(const BakeParams& P, int bx, int by, int bz, int l0) {
-    const int B = P.B, m = B - 1, l1 = l0 + P.item_voxels - 1;
-    const int x0 = l0 & m, y0 = (l0 >> P.lgB) & m, z0 = l0 >> (2 * P.lgB);
-    const int x1 = l1 & m, y1 = (l1 >> P.lgB) & m, z1 = l1 >> (2 * P.lgB);
+// the voxels of block b
+__device__ __forceinline__ ItemBox block_box(const BakeParams& P, int64_t b) {
+    const int c[3] = {(int)(b % P.G), (int)((b / P.G) % P.G), (int)(b / ((int64_t)P.G * P.G))};
     ItemBox r;
-    r.lo[2] = bz * B + z0;
-    r.hi[2] = bz * B + z1;
-    if (z0 == z1) {
-        r.lo[1] = by * B + y0;
-        r.hi[1] = by * B + y1;
-        r.lo[0] = bx * B + (y0 == y1 ? x0 : 0);
-        r.hi[0] = bx * B + (y0 == y1 ? x1 : m);
-    } else {
-        r.lo[1] = by * B;
-        r.hi[1] = by * B + m;
-        r.lo[0] = bx * B;
-        r.hi[0] = bx * B + m;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        r.lo[a] = c[a] * P.B;
+        r.hi[a] = r.lo[a] + P.B - 1;
     }
     return r;
 }
@@ -157,34 +144,20 @@ __global__ void __launch_bounds__(kThreads) bake_alpha_kernel(const __grid_const
     __shared__ float s_peak[kMaxBlobs];
     __shared__ int s_cnt[2];
     const int t = threadIdx.x, m = P.B - 1;
-    const int n_chunks = 1 << P.lg_items;
     for (int64_t b = blockIdx.x; b < G3; b += gridDim.x) {
-        const int bx = (int)(b % P.G), by = (int)((b / P.G) % P.G), bz = (int)(b / ((int64_t)P.G * P.G));
-        ItemBox box;
-        box.lo[0] = bx * P.B;
-        box.lo[1] = by * P.B;
-        box.lo[2] = bz * P.B;
-        box.hi[0] = box.lo[0] + m;
-        box.hi[1] = box.lo[1] + m;
-        box.hi[2] = box.lo[2] + m;
+        const ItemBox box = block_box(P, b);
         __syncthreads();                                   // the previous block's readers are done
         const int n = gather_blobs(P, box, false, s_blob, s_peak, s_cnt);
         if (n == 0) continue;                              // uniform: alpha = 0 < tau everywhere
-        for (int ch = 0; ch < n_chunks; ++ch) {
-            bool keep = false;
-            if (t < P.item_voxels) {
-                const int l = ch * P.item_voxels + t;
-                const float x = P.bmin[0] + ((float)(box.lo[0] + (l & m)) + 0.5f) * P.v;
-                const float y = P.bmin[1] + ((float)(box.lo[1] + ((l >> P.lgB) & m)) + 0.5f) * P.v;
-                const float z = P.bmin[2] + ((float)(box.lo[2] + (l >> (2 * P.lgB))) + 0.5f) * P.v;
-                const float sigma = density_at(s_blob, s_peak, n, x, y, z);
-                keep = -expm1f(-sigma * P.v) >= P.tau;   // alpha = 1 - exp(-sigma v)
-            }
-            if (__syncthreads_or(keep)) {
-                if (t == 0) keep_block(flags, b);
-                break;                                     // uniform
-            }
+        bool keep = false;
+        if (t < 1 << (3 * P.lgB)) {
+            const float x = P.bmin[0] + ((float)(box.lo[0] + (t & m)) + 0.5f) * P.v;
+            const float y = P.bmin[1] + ((float)(box.lo[1] + ((t >> P.lgB) & m)) + 0.5f) * P.v;
+            const float z = P.bmin[2] + ((float)(box.lo[2] + (t >> (2 * P.lgB))) + 0.5f) * P.v;
+            const float sigma = density_at(s_blob, s_peak, n, x, y, z);
+            keep = -expm1f(-sigma * P.v) >= P.tau;         // alpha = 1 - exp(-sigma v)
         }
+        if (__syncthreads_or(keep) && t == 0) keep_block(flags, b);
     }
 }
 
@@ -360,20 +333,16 @@ __global__ void __launch_bounds__(kThreads) bake_fill_kernel(const __grid_consta
     __shared__ int s_cnt[2];
     const int t = threadIdx.x, m = P.B - 1;
     const int64_t nb = min(*count, max_blocks);
-    const int64_t n_items = nb << P.lg_items;
     const int lg3 = 3 * P.lgB;
-    for (int64_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const int64_t slot = it >> P.lg_items;
-        const int l0 = (int)(it & ((1 << P.lg_items) - 1)) * P.item_voxels;
+    for (int64_t slot = blockIdx.x; slot < nb; slot += gridDim.x) {
         const int64_t b = list[slot];
-        const int bx = (int)(b % P.G), by = (int)((b / P.G) % P.G), bz = (int)(b / ((int64_t)P.G * P.G));
+        const ItemBox box = block_box(P, b);
         __syncthreads();
-        const int n = gather_blobs(P, item_box(P, bx, by, bz, l0), true, s_blob, s_peak, s_cnt);
-        if (t >= P.item_voxels) continue;
-        const int l = l0 + t;
-        const float fx = (float)(bx * P.B + (l & m)) + 0.5f;
-        const float fy = (float)(by * P.B + ((l >> P.lgB) & m)) + 0.5f;
-        const float fz = (float)(bz * P.B + (l >> (2 * P.lgB))) + 0.5f;
+        const int n = gather_blobs(P, box, true, s_blob, s_peak, s_cnt);
+        if (t >= 1 << lg3) continue;
+        const float fx = (float)(box.lo[0] + (t & m)) + 0.5f;
+        const float fy = (float)(box.lo[1] + ((t >> P.lgB) & m)) + 0.5f;
+        const float fz = (float)(box.lo[2] + (t >> (2 * P.lgB))) + 0.5f;
         const float cx = P.bmin[0] + fx * P.v, cy = P.bmin[1] + fy * P.v, cz = P.bmin[2] + fz * P.v;
         // sum over blobs of peak * sum over samples of 2^(-k |D + jv_s|^2), D = centre - c,
         // expanded as -k |D|^2 - 2k D . jv_s - k |jv_s|^2: four FMAs per blob and sample
@@ -398,7 +367,7 @@ __global__ void __launch_bounds__(kThreads) bake_fill_kernel(const __grid_consta
             sincosf(a, &sa, &ca);
             q[1 + c] = code8(fmaf(0.5f, fmaf(sa, P.cbar[c], ca * P.sbar[c]), 0.5f));
         }
-        atlas[(slot << lg3) + l] = make_uint2(q[0] | q[1] << 8 | q[2] << 16 | q[3] << 24,
+        atlas[(slot << lg3) + t] = make_uint2(q[0] | q[1] << 8 | q[2] << 16 | q[3] << 24,
                                               q[4] | q[5] << 8 | q[6] << 16 | q[7] << 24);
     }
 }
@@ -734,8 +703,7 @@ cudaError_t launch_fill(const BakeParams& P, const int32_t* list, const int64_t*
         case 5: return fill_sep<5>(P, list, d_count, count, max_blocks, atlas, st);
         case 6: return fill_sep<6>(P, list, d_count, count, max_blocks, atlas, st);
     }
-    const int64_t items = count << P.lg_items;
-    bake_fill_kernel<<<grid_for((const void*)bake_fill_kernel, kThreads, 0, items), kThreads, 0, st>>>(
+    bake_fill_kernel<<<grid_for((const void*)bake_fill_kernel, kThreads, 0, count), kThreads, 0, st>>>(
         P, list, d_count, max_blocks, atlas);
     return cudaGetLastError();
 }
@@ -760,10 +728,7 @@ BakeParams make_params(const snerg_scene_desc* desc, const snerg_bake_field* fie
     P.lgB = ilog2_exact(desc->B);
     P.G = desc->N / desc->B;
     P.n_blob = field->n_blob;
-    const int B3 = desc->B * desc->B * desc->B;
-    P.item_voxels = B3 < kThreads ? B3 : kThreads;
     P.alpha_codes = (desc->flags & SNERG_FLAG_ALPHA_ATLAS) ? 1 : 0;
-    P.lg_items = ilog2_exact(B3 / P.item_voxels);
     const double v = (double)desc->extent / (double)desc->N;
     P.v = (float)v;
     P.tau = field->tau_alpha;
