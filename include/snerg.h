@@ -347,7 +347,7 @@ snerg_status snerg_adam_step(float* d_param, float* d_m, float* d_v, const float
  * Limit: N / B <= 64; larger grids return SNERG_E_UNSUPPORTED. Of the scene flags only
  * SNERG_FLAG_UNPREMULTIPLY is accepted (others return SNERG_E_INVAL).
  * Scratch: a status word and the block-level empty-space distance map live in one static
- * device array of 786,688 bytes that every GPU loading this library holds until the
+ * device array of 524,544 bytes that every GPU loading this library holds until the
  * process exits. The first call on each device, with rays or without (n = 0), looks up that
  * array's device address and loads every kernel that later calls can launch, for all block
  * edges and ray counts (with the device current): make that first call before any stream

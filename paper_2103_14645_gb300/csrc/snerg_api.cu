@@ -214,7 +214,6 @@ extern "C" snerg_status snerg_create(const snerg_scene_desc* desc, const int32_t
 
     DevScene& s = h->ds;
     s.ind = ws_ind;
-    s.bdist = bdist;
     s.vskip = vskip;
     s.ind_oct = G3;
     s.vskip_oct = num_blocks * (int64_t)P * P * P;

@@ -66,7 +66,7 @@ constexpr int kStatusStepLimit = SNERG_E_STEP_LIMIT;
 
 struct DevScene {
     const int32_t* ind;    // octant 0's copy; octant o's at ind + o * ind_oct
-    const uint8_t* bdist;
+    const uint8_t* bdist;   // block distances (snerg_render_rays_noalloc only; a handle has them in ind)
     const uint8_t* vskip;  // octant 0's plane; octant o's at vskip + o * vskip_oct
     const uint2* patlas;
     int32_t* status;

@@ -7,7 +7,7 @@
 // buffers it was handed. snerg_render_rays_noalloc serves them: it renders straight from
 // the caller's indirection grid and uint8 atlas (no padded copy, no voxel distance map),
 // and keeps its only scratch -- a status word and the block-level empty-space distance
-// map with its two transform temporaries -- in one file-scope __device__ array of fixed
+// map with its transform's temporary -- in one file-scope __device__ array of fixed
 // size that every GPU loading the library holds until the process exits.
 //
 // The array's host-side name is only a stand-in; its device address is fetched with
@@ -33,10 +33,10 @@ namespace {
 constexpr int kNoAllocMaxG = 64;                               // N / B <= 64
 constexpr size_t kNoAllocG3 = (size_t)kNoAllocMaxG * kNoAllocMaxG * kNoAllocMaxG;
 constexpr size_t kNoAllocHeader = 256;                         // status word at byte 0
-constexpr size_t kNoAllocBytes = kNoAllocHeader + 3 * kNoAllocG3;   // 786,688 bytes
+constexpr size_t kNoAllocBytes = kNoAllocHeader + 2 * kNoAllocG3;   // 524,544 bytes
 constexpr int kNoAllocMaxDevices = 64;
 
-// [0, 256): status word | bdist [G^3] | two G^3 temporaries of the distance transform
+// [0, 256): status word | bdist [G^3] | the distance transform after its x and y passes [G^3]
 __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocBytes];
 
 // ---------------------------------------------------------------------------------

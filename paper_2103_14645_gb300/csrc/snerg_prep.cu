@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256) adam_requantize_kernel(const int32_t* __r
 }
 
 // ---------------------------------------------------------------------------------
-// Chebyshev (L-infinity) distance transform of cubes of side n, in three separable
+// Chebyshev (L-infinity) distance transform of a cube of side n, in three separable
 // passes: along one axis, out(p) = min over q on p's line of max(|q - p|, in(q)),
 // capped at `cap`. Starting from in = 0 on occupied cells and cap elsewhere, after the
 // x, y and z passes out(p) = min over occupied q of max_i |q_i - p_i| (max distributes
@@ -172,15 +172,13 @@ __device__ __forceinline__ int dt_line(const uint8_t* __restrict__ in, int64_t b
 // the side of axis i for octant o (bit i of o set: the ray runs towards -i)
 __host__ __device__ __forceinline__ int octant_side(int o, int i) { return ((o >> i) & 1) ? kSideLow : kSideHigh; }
 
-// axis: 0 = x (stride 1), 1 = y (stride n), 2 = z (stride n^2); cubes are contiguous
-__global__ void dt_pass_kernel(const uint8_t* __restrict__ in, uint8_t* __restrict__ out, int n, int64_t ncubes,
-                               int axis, int cap, int side) {
-    const int64_t n3 = (int64_t)n * n * n;
-    const int64_t total = ncubes * n3;
+// axis: 0 = x (stride 1), 1 = y (stride n), 2 = z (stride n^2)
+__global__ void dt_pass_kernel(const uint8_t* __restrict__ in, uint8_t* __restrict__ out, int n, int axis, int cap,
+                               int side) {
+    const int64_t total = (int64_t)n * n * n;
     const int64_t stride = axis == 0 ? 1 : (axis == 1 ? n : (int64_t)n * n);
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t cube = t / n3;
-        const int r = (int)(t - cube * n3);
+        const int r = (int)t;                                  // n <= 1024
         const int c[3] = {r % n, (r / n) % n, r / (n * n)};
         const int pos = c[axis];
         const int64_t base = t - (int64_t)pos * stride;
@@ -543,9 +541,9 @@ static void block_distance(const int32_t* ind, int G, int cap, uint8_t* tmp0, ui
                            const int side[3], cudaStream_t st) {
     const int64_t n = (int64_t)G * G * G;
     block_seed_kernel<<<grid_for(n), 256, 0, st>>>(ind, n, cap, tmp0);
-    dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp0, tmp1, G, 1, 0, cap, side[0]);
-    dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp1, tmp0, G, 1, 1, cap, side[1]);
-    dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp0, bdist, G, 1, 2, cap, side[2]);
+    dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp0, tmp1, G, 0, cap, side[0]);
+    dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp1, tmp0, G, 1, cap, side[1]);
+    dt_pass_kernel<<<grid_for(n), 256, 0, st>>>(tmp0, bdist, G, 2, cap, side[2]);
 }
 
 // For each octant o, ind_oct[o] = the indirection grid `ind` with every empty entry replaced by
