@@ -532,9 +532,10 @@ extern "C" snerg_status snerg_render(snerg_handle h, const snerg_camera* cams, i
         sa.nt = tiles;
         sa.tiles_x = (cams[0].W + 15) / 16;
         // a small image's tiles take 8 CTAs each and no sparse slots (by the rule of the plain image,
-        // where it takes 4 rays per warp or fewer: 25,600 pixels of a 1024^3 grid 75 -> 67 us; 2 or 4
-        // CTAs gain nothing over the sparse tiles: 115,600 pixels 94 us, with 2 97, with 4 99). Sparse
-        // slots only with a previous frame to choose the slow tiles from
+        // where it takes 4 rays per warp or fewer: 25,600 pixels of a 1024^3 grid 75 -> 67 us, 32,400 of a
+        // 512^3 one 83 -> 62; 2 or 4 CTAs gain nothing over the sparse tiles: 115,600 pixels of a 1024^3
+        // grid 94 us, with 2 97, with 4 99). Sparse slots only with a previous frame to choose the slow
+        // tiles from
         sa.parts = image_lanes(h->ds, (int64_t)cams[0].W * cams[0].H, 1) <= 4 ? 8 : 1;
         sa.smax = use && sa.parts == 1 ? std::min(kSchedMaxSparse, std::max(1, tiles / 8)) : 0;
         cudaError_t e = cudaMemsetAsync(wr, 0, kSchedCountBytes, st);

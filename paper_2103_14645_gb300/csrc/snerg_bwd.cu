@@ -422,11 +422,10 @@ static cudaError_t backward_launch(const DevScene& s, const CamTable& cams, int3
                                    const int32_t* fwd_counts, const float2* record, const float* target, float* rgb_out, float* loss,
                                    float* grad_atlas, float* grad_mlp, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    // a short list is spread over 12 warps per SM (3 CTAs) in grids of up to 288^3, 16 from 768^3 on:
-    // a step of 10,000 rays with 32 / 16 / 8 rays per warp (8: 8 warps per SM) takes 89 / 66 / 58 us on
-    // a 1024^3 grid and 55 / 50 / 47 on a 256^3 one, of 33,000 with 32 / 16 (14 warps) 95 / 89 and
-    // 62 / 71
-    const int lanes = lanes_per_warp(n, s.sms * (1152 + chain_side(s)) / 120);
+    // up to about one wave of 4 CTAs per SM (16 warps): a step of 10,000 rays with 32 / 16 / 8 rays per warp (8:
+    // 8 warps per SM) takes 89 / 66 / 58 us on a 1024^3 grid and 55 / 50 / 47 on a 256^3 one, of 33,000
+    // with 32 / 16 (14 warps) 95 / 89 and 62 / 71
+    const int lanes = lanes_per_warp(n, s.sms, {by_side(s, 20, 10, 14), by_side(s, 32, 11, 14), by_side(s, 32, 10, 12), 9, 9});
     const size_t smem = backward_smem_bytes(lanes);
     // the opt-in for > 48 KB of dynamic shared memory, once per device
     static std::atomic<bool> attr_set[kMaxDevices];

@@ -385,19 +385,21 @@ cudaError_t Forward<LGB, A>::image(const DevScene& ds, const snerg_camera& cam, 
     return cudaGetLastError();
 }
 
-// A short list is spread over 14 warps per SM (3.5 CTAs): 16,000 scattered rays of a 1024^3 grid
-// 76 us with 32 rays per warp, 53 with 8; beyond it 32 rays per warp are as good or better (52,000
-// rays with 32 / 16: 1024^3 90 / 97 us, 128^3 58 / 65). If 4 CTAs per SM hold the list, it runs the build
-// limited to 4 (the march keeps its state in registers, and a single wave gains nothing from more
-// CTAs); longer lists keep 7 CTAs per SM to hide the march's latencies: 8 spill with the weights in
-// device memory (131,072 and 262,144 rays of a 1024^3 grid 163 and 277 us with 8, 153 and 268 with
-// 7; 1,000,000 rays 731 and 747).
+// A short list is spread over the warps of one wave of 7 CTAs per SM (28 warps), with debug outputs,
+// which need more registers, of 4: 16,000 scattered rays of a 1024^3 grid take 76 us with 32 rays per
+// warp and 53 with 8 or 4. With 16 and 8 the limits grow with the grid's side: 43,241 rays with 32 / 16
+// (18 warps) 84 / 68 on a 768^3 grid, but 58 / 61 on a 256^3 one. If 4 CTAs per SM hold the list, it runs
+// the build limited to 4 (the march keeps its state in registers, and a single wave gains nothing
+// from more CTAs); longer lists keep 7 CTAs per SM to hide the march's latencies: 8 spill with the
+// weights in device memory (131,072 and 262,144 rays of a 1024^3 grid 163 and 277 us with 8, 153 and
+// 268 with 7; 1,000,000 rays 731 and 747).
 template <int LGB, int A>
 cudaError_t Forward<LGB, A>::rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
                                const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, float2* record,
                                cudaStream_t st) {
     const bool d = dbg.aux || dbg.counts || dbg.trace;
-    const int lanes = lanes_per_warp(n, (int64_t)s.sms * 14);
+    const int lanes = d ? lanes_per_warp(n, s.sms, {16, 16, 16, 16, 16})
+                        : lanes_per_warp(n, s.sms, {by_side(s, 16, 16, 28), by_side(s, 16, 20, 28), 28, 28, 28});
     const bool one_wave = n <= (int64_t)s.sms * 4 * 4 * lanes;
     auto* kernel = pw ? (one_wave ? render_rays_kernel<LGB, A, false, true, 4> : render_rays_kernel<LGB, A, false, true, 7>)
                       : (one_wave ? render_rays_kernel<LGB, A, false, false, 4> : render_rays_kernel<LGB, A, false, false, 7>);

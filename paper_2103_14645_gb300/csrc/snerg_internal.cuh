@@ -128,19 +128,30 @@ inline auto with_block_build(const DevScene& s, F&& f) {
     return f(Build<0, kAnyAlpha>{});
 }
 
-// Rays per warp for n rays where `warps` warps are worth launching: 32, or as many lanes fewer
-// (a power of two) as still make no more than that many warps; the other lanes idle. A launch
-// that leaves the chip part empty is as slow as its slowest warps, whose lanes wait for one
-// another at every branch of their rays' chains of dependent loads: with fewer rays beside it a
-// ray's chain is shorter, and the warps it costs have room. The launches say how many they take:
-// no more than were at no size slower than 32 rays per warp on grids of 128^3 to 2048^3. Beside
-// other launches the idle lanes' issue slots are lost to those; what a launch cannot know of (other
+// Rays per warp for n rays: 32, or fewer lanes (a power of two, the others idle) as long as they
+// make no more warps than are worth launching with so few each. A launch that leaves the chip part
+// empty is as slow as its slowest warps, whose lanes wait for one another at every branch of their
+// rays' chains of dependent loads: with fewer rays beside it a ray's chain is shorter, and the warps
+// it costs have room. The limits (warps per SM with 16, 8, 4, 2 and 1 rays each) are each launch's
+// own, and by the grid's side N where that decides: the longer the chains, the more issue slots a
+// warp leaves to others. They are where the times cross over in sweeps of 1 to 32 rays per warp on
+// 25 grids of 128^3 to 2048^3, 33 sizes each: launches are within 2 % of the best number for each on
+// average, and 1.3 to 1.4 times as fast as with 32 rays per warp. The crossing of one image or list
+// depends on what its slowest warps see (an image of 64,009 pixels of one 448^3 grid of 64^3 blocks
+// is 11 % slower than with 32, the next sizes as fast), so the lines are the means'. Beside other
+// launches the idle lanes' issue slots are lost to those; what a launch cannot know of (other
 // handles' and other programs' launches) is taken not to be there.
-inline int lanes_per_warp(int64_t n, int64_t warps) {
-    int lanes = 32;
-    while (lanes > 1 && n <= warps * (lanes / 2)) lanes /= 2;
-    return lanes;
+struct LaneLimits {
+    int l16, l8, l4, l2, l1;
+};
+inline int lanes_per_warp(int64_t n, int sms, const LaneLimits& w) {
+    const int limit[] = {w.l1, w.l2, w.l4, w.l8, w.l16};
+    for (int i = 0; i < 5; ++i)
+        if (n <= ((int64_t)sms * limit[i]) << i) return 1 << i;
+    return 32;
 }
+// N / d, from lo to hi
+inline int by_side(const DevScene& s, int d, int lo, int hi) { return s.N / d < lo ? lo : (s.N / d > hi ? hi : s.N / d); }
 
 // App. C: the scale min(1, 1.5 a) / a applied after compositing to (C_d, alpha, V) when
 // un-premultiply is on and a = 1 - T > 0 (else 1). Depends on density only.
@@ -973,18 +984,15 @@ struct SchedArgs {
     int32_t parts;             // CTAs per dense tile (1 or 8: bands of its rows)
 };
 
-// The grid's side as the rules for the rays per warp take it: the longer a ray's chain, the more a
-// warp's lanes wait for one another and the more issue slots it leaves to other warps.
-inline int64_t chain_side(const DevScene& s) { return s.N < 288 ? 288 : (s.N > 768 ? 768 : s.N); }
-
 // Rays per warp of a one-camera launch of n pixels (with `share` of its kind on the chip at a time):
-// up to 3/4 of a wave of warps in grids of up to 288^3, two waves from 768^3 on, in proportion
-// between. 38,809 pixels with 32 / 16 / 8 / 4 rays per warp: of a 1024^3 grid 102 / 101 / 87 / 71 us
-// (4: two waves), of a 512^3 one 93 / 82 / 62 / 64; 136,900 pixels with 32 / 16 (1.8 waves): of a
-// 1024^3 grid 123 / 104, 2048^3 243 / 209, but 256^3 60 / 69 and 128^3 45 / 53.
+// about one wave of warps (32 per SM) at most in grids of up to 256^3, three in the largest. 38,809 pixels
+// with 32 / 16 / 8 / 4 rays per warp: of a 1024^3 grid 102 / 101 / 87 / 71 us (4: 64 warps per SM), of
+// a 512^3 one 93 / 82 / 62 / 64; 136,900 pixels with 32 / 16 (56): of a 1024^3 grid 123 / 104, 2048^3
+// 243 / 209, but 256^3 60 / 69 and 128^3 45 / 53.
 constexpr int kImageWarps = 4;     // warps per CTA of the one-camera launch
 inline int image_lanes(const DevScene& s, int64_t n, int share) {
-    return lanes_per_warp(n * share, (int64_t)s.sms * 8 * kImageWarps * chain_side(s) / 384);
+    const int w = by_side(s, 8, 40, 96);
+    return lanes_per_warp(n * share, s.sms, {by_side(s, 10, 28, 96), w, w, by_side(s, 4, 32, 80), by_side(s, 6, 40, 56)});
 }
 
 inline const MlpWeights& no_weights() {

@@ -359,9 +359,9 @@ extern "C" snerg_status snerg_render_rays_noalloc(const snerg_scene_desc* desc, 
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         s.sms = sms;
-        // a short list is spread over 12 warps per SM: 10,000 rays of a 1024^3 grid 118 us with 32 rays
-        // per warp, 84 with 8; 38,000 with 32 / 16 (16 warps) 191 / 157, but of a 128^3 grid 84 / 89
-        const int lanes = lanes_per_warp(n, (int64_t)sms * 12);
+        // one wave of 4 CTAs per SM: 10,000 rays of a 1024^3 grid 118 us with 32 rays per warp, 79 with 4;
+        // 38,000 with 32 / 16 (16 warps per SM) 191 / 157, but of a 128^3 grid 84 / 89
+        const int lanes = lanes_per_warp(n, sms, {by_side(s, 12, 12, 16), 16, 16, 16, 16});
         const int64_t ctas = (n + 4 * lanes - 1) / (4 * lanes);
         with_block_build(s, [&](auto build) {
             constexpr int L = decltype(build)::lgB;

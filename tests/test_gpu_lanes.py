@@ -15,15 +15,20 @@ LANES = (1, 2, 4, 8, 16)
 N = 64                                                     # the scene's grid
 
 
-def _warps(rule):
-    """Warps that a launch spreads its rays over: lanes l for up to l times as many rays."""
+def _most(lanes, rule):
+    """The most rays that take no more than `lanes` per warp."""
     sms = torch.cuda.get_device_properties(DEV).multi_processor_count
-    side = min(max(N, 288), 768)
-    return {"image": sms * 32 * side // 384, "list": sms * 14, "adjoint": sms * (1152 + side) // 120}[rule]
+
+    def side(d, lo, hi):
+        return min(max(N // d, lo), hi)
+    warps = {"image": [side(6, 40, 56), side(4, 32, 80), side(8, 40, 96), side(8, 40, 96), side(10, 28, 96)],
+             "list": [28, 28, 28, side(16, 20, 28), side(16, 16, 28)], "debug list": [16] * 5,
+             "adjoint": [9, 9, side(32, 10, 12), side(32, 11, 14), side(20, 10, 14)]}[rule]
+    return sms * warps[LANES.index(lanes)] * lanes
 
 
 def _lanes(n, rule):
-    return next((l for l in LANES if n <= _warps(rule) * l), 32)
+    return next((l for l in LANES if n <= _most(l, rule)), 32)
 
 
 @pytest.fixture(scope="module")
@@ -40,7 +45,7 @@ def _camera(W, H):
 
 def _image(lanes, over):
     """A ragged image of `lanes` rays per warp, near the class's limit, or the next class (over)."""
-    n = _warps("image") * min(lanes, 16)
+    n = _most(lanes, "image")
     W = int((4 * n / 3) ** 0.5) | 1
     H = n // W
     if over:
@@ -70,10 +75,12 @@ def test_images_of_every_size_class(scene, size):
     r.check_status()
 
 
+@pytest.mark.parametrize("rule", ["list", "debug list"])
 @pytest.mark.parametrize("lanes,more", [(0, 1), (0, 33)] + [(l, more) for l in LANES for more in (0, 1)] + [(36, 1)])
-def test_ray_lists_of_every_size_class(scene, lanes, more):
-    n = _warps("list") * lanes + more                      # 36: beyond one wave of 4 CTAs per SM
-    assert lanes in (0, 36) or _lanes(n, "list") == (lanes if not more else 2 * lanes)
+def test_ray_lists_of_every_size_class(scene, lanes, more, rule):
+    # 36: beyond one wave of 4 CTAs per SM
+    n = more + (0 if lanes == 0 else _most(1, "debug list") * 36 if lanes == 36 else _most(lanes, rule))
+    assert lanes in (0, 36) or _lanes(n, rule) == (lanes if not more else 2 * lanes)
     _, r, w = scene
     cam = _camera(1021, 523)
     image = r.render(cam, w, counts=True)["rgb"]
@@ -88,7 +95,7 @@ def test_ray_lists_of_every_size_class(scene, lanes, more):
 
 @pytest.mark.parametrize("lanes,more", [(0, 5)] + [(l, more) for l in LANES for more in (0, 1)])
 def test_adjoint_sums_of_every_size_class(scene, lanes, more):
-    n = _warps("adjoint") * lanes + more
+    n = more + (_most(lanes, "adjoint") if lanes else 0)
     assert lanes == 0 or _lanes(n, "adjoint") == (lanes if not more else 2 * lanes)
     sc, r, w = scene
     cam = _camera(640, 479)
