@@ -385,7 +385,9 @@ __global__ void __launch_bounds__(kThreads) bake_fill_kernel(const __grid_consta
 // with 64 blobs 6.98 -> 1.50 ms; 4 x 4 x 2 tiles without the per-blob sums took 1.49 ms, bound
 // by shared-memory returns, and 8 x 4 x 2 with every operand stored twice 1.85 ms.
 // Three CTAs per SM with some spills: the whole bake takes 1.75 ms, with two and none 1.92; six
-// blobs a chunk or no unrolling of the samples change it by 1 % at most.
+// blobs a chunk or no unrolling of the samples change it by 1 % at most. Edges of 8 and 16 take six,
+// 504 bytes of spills at 16: a 512^3 grid of 16^3 blocks 476 us, with five 473, four 508, three 505;
+// a 256^3 grid of 8^3 blocks 271, 262, 262, 267.
 // ---------------------------------------------------------------------------------
 template <int LGB>
 struct FillShape {

@@ -173,6 +173,9 @@ __device__ __forceinline__ void image_pixel(const SC& s, const snerg_camera& cam
     }
 }
 
+// 8 CTAs per SM leave 64 registers: the builds per block edge spill 8 bytes with the weights as
+// parameters and 56 with the weights in device memory (the any-edge build, with more instructions,
+// none), and are the faster all the same: a full-HD view with weights in device memory 833 -> 794 us.
 template <int LGB, int A, bool DBG, bool PW, int NW, bool PS, bool SCHED = false>
 __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const BlockScene<LGB, A> s, const snerg_camera cam,
                                                                         const float* __restrict__ mlp,

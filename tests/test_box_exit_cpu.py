@@ -1,10 +1,13 @@
-"""The march's unconfirmed block exits, replayed on the CPU in binary32.
+"""The margin of the march's unconfirmed block exits (exit_margin), replayed on the CPU in binary32.
 
 A block (or empty box) run ends at the first lattice sample whose nearest voxel leaves
-the box. The kernel estimates that index from the ray/face distance and, when the real
-crossing is at least a margin away from every integer, takes the estimate without
-checking samples on the lattice. This test replays that arithmetic with numpy float32
-(one rounding per operation, as the kernel's binary32 control arithmetic does), with the
+the box. That index is estimated from the ray/face distance and, when the real crossing
+is at least a margin away from every integer, taken without checking samples on the
+lattice. This test shows that the margin is enough for boxes whose faces at the grid's
+border are open (infinite); the march's own estimate (march_exit), with the faces ahead
+left where they are, is replayed in test_march_exit_cpu.py on the same kinds of rays. The
+arithmetic is replayed with numpy float32 (one rounding per operation, as the kernel's
+binary32 control arithmetic does), with the
 reciprocal of each direction component perturbed by up to 2 ulp (the error bound of the
 approximate reciprocal the kernel uses), on random rays and on rays built so that a face
 crossing falls within 1e-3 samples of a lattice point, and on rays whose first face
