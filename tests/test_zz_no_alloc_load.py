@@ -1,5 +1,5 @@
 """snerg_render_rays_noalloc loads every kernel it can launch at its first call on a device: a fresh
-process makes one call without rays, and the driver then reports each of the entry point's
+process makes one call without rays, and CUDA then reports each of the entry point's
 kernels as loaded; a call of another block edge and of more than one wave of rays is captured,
 and its replay gives what the plain call gives."""
 import subprocess
