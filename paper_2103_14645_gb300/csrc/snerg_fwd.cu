@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) render_image_kernel(const Bl
     }
 }
 
-// MINB: resident CTAs per SM the build is limited to (7: 72 registers; 4: up to 128);
+// MINB: resident CTAs per SM the build is limited to (8: 64 registers; 7: 72; 4: up to 128);
 // lanes: rays per warp (the other lanes idle); REC: each ray's composited samples go to
 // record (entry j of ray i at record[j * n + i], see march) for the adjoint
 template <int LGB, int A, bool DBG, bool PW, int MINB, bool REC = false>
@@ -393,9 +393,11 @@ cudaError_t Forward<LGB, A>::image(const DevScene& ds, const snerg_camera& cam, 
 // warp and 53 with 8 or 4. With 16 and 8 the limits grow with the grid's side: 43,241 rays with 32 / 16
 // (18 warps) 84 / 68 on a 768^3 grid, but 58 / 61 on a 256^3 one. If 4 CTAs per SM hold the list, it runs
 // the build limited to 4 (the march keeps its state in registers, and a single wave gains nothing
-// from more CTAs); longer lists keep 7 CTAs per SM to hide the march's latencies: 8 spill with the
-// weights in device memory (131,072 and 262,144 rays of a 1024^3 grid 163 and 277 us with 8, 153 and
-// 268 with 7; 1,000,000 rays 731 and 747).
+// from more CTAs). Longer lists keep 7 CTAs per SM to hide the march's latencies (8 spill with the
+// weights in device memory: 130,313 and 218,548 rays of a 1024^3 grid 149 and 229 us with 8, 141 and
+// 222 with 7), or 8 where those hold the list in one or two waves and 7 need one more (154,825 and
+// 308,499 rays 184 and 286 us with 7, 160 and 278 with 8; of a 256^3 grid 125 and 191, 123 and 192),
+// and, from 1024^3 on, where they save any wave (1,030,921 rays of a 2048^3 grid 4 % less).
 template <int LGB, int A>
 cudaError_t Forward<LGB, A>::rays(const DevScene& s, const CamTable& cams, int32_t n_cams, const int32_t* pix, int64_t n,
                                const float* mlp, const MlpWeights* pw, float* rgb, const DebugOut& dbg, float2* record,
@@ -403,19 +405,32 @@ cudaError_t Forward<LGB, A>::rays(const DevScene& s, const CamTable& cams, int32
     const bool d = dbg.aux || dbg.counts || dbg.trace;
     const int lanes = d ? lanes_per_warp(n, s.sms, {16, 16, 16, 16, 16})
                         : lanes_per_warp(n, s.sms, {by_side(s, 16, 16, 28), by_side(s, 16, 20, 28), 28, 28, 28});
-    const bool one_wave = n <= (int64_t)s.sms * 4 * 4 * lanes;
-    auto* kernel = pw ? (one_wave ? render_rays_kernel<LGB, A, false, true, 4> : render_rays_kernel<LGB, A, false, true, 7>)
-                      : (one_wave ? render_rays_kernel<LGB, A, false, false, 4> : render_rays_kernel<LGB, A, false, false, 7>);
+    const int64_t ctas = (n + 4 * lanes - 1) / (4 * lanes), w7 = (ctas + 7 * s.sms - 1) / (7 * s.sms),
+                  w8 = (ctas + 8 * s.sms - 1) / (8 * s.sms);
+    const int per = ctas <= 4 * (int64_t)s.sms ? 4 : (w8 < w7 && (w8 <= 2 || s.N >= 1024) ? 8 : 7);
+    // the build for `per` CTAs per SM
+    auto* kernel = pw ? (per == 4   ? render_rays_kernel<LGB, A, false, true, 4>
+                         : per == 7 ? render_rays_kernel<LGB, A, false, true, 7>
+                                    : render_rays_kernel<LGB, A, false, true, 8>)
+                      : (per == 4   ? render_rays_kernel<LGB, A, false, false, 4>
+                         : per == 7 ? render_rays_kernel<LGB, A, false, false, 7>
+                                    : render_rays_kernel<LGB, A, false, false, 8>);
     if (record) {                       // weights in device memory
-        kernel = one_wave ? render_rays_kernel<LGB, A, true, false, 4, true> : render_rays_kernel<LGB, A, true, false, 7, true>;
+        kernel = per == 4   ? render_rays_kernel<LGB, A, true, false, 4, true>
+                 : per == 7 ? render_rays_kernel<LGB, A, true, false, 7, true>
+                            : render_rays_kernel<LGB, A, true, false, 8, true>;
     } else if (d) {
         if constexpr (LGB == 0)
-            kernel = pw ? (one_wave ? render_rays_kernel<LGB, A, true, true, 4> : render_rays_kernel<LGB, A, true, true, 7>)
-                        : (one_wave ? render_rays_kernel<LGB, A, true, false, 4> : render_rays_kernel<LGB, A, true, false, 7>);
+            kernel = pw ? (per == 4   ? render_rays_kernel<LGB, A, true, true, 4>
+                           : per == 7 ? render_rays_kernel<LGB, A, true, true, 7>
+                                      : render_rays_kernel<LGB, A, true, true, 8>)
+                        : (per == 4   ? render_rays_kernel<LGB, A, true, false, 4>
+                           : per == 7 ? render_rays_kernel<LGB, A, true, false, 7>
+                                      : render_rays_kernel<LGB, A, true, false, 8>);
         else
             return cudaErrorInvalidValue;
     }
-    kernel<<<(unsigned)((n + 4 * lanes - 1) / (4 * lanes)), 128, 0, st>>>(
+    kernel<<<(unsigned)ctas, 128, 0, st>>>(
         BlockScene<LGB, A>(s), cams, n_cams, pix, n, mlp, pw ? *pw : no_weights(), rgb, dbg, record, lanes);
     return cudaGetLastError();
 }

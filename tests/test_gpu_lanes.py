@@ -76,11 +76,12 @@ def test_images_of_every_size_class(scene, size):
 
 
 @pytest.mark.parametrize("rule", ["list", "debug list"])
-@pytest.mark.parametrize("lanes,more", [(0, 1), (0, 33)] + [(l, more) for l in LANES for more in (0, 1)] + [(36, 1)])
+@pytest.mark.parametrize("lanes,more", [(0, 1), (0, 33)] + [(l, more) for l in LANES for more in (0, 1)] +
+                         [(per, more) for per in (40, 70, 80, 140, 160) for more in (0, 1)])
 def test_ray_lists_of_every_size_class(scene, lanes, more, rule):
-    # 36: beyond one wave of 4 CTAs per SM
-    n = more + (0 if lanes == 0 else _most(1, "debug list") * 36 if lanes == 36 else _most(lanes, rule))
-    assert lanes in (0, 36) or _lanes(n, rule) == (lanes if not more else 2 * lanes)
+    # 40, 70, 80, 140, 160: 4, 7, 8, 14, 16 CTAs per SM of 128 rays, where the builds change
+    n = more + (0 if lanes == 0 else _most(1, "debug list") * 32 * lanes // 40 if lanes >= 40 else _most(lanes, rule))
+    assert lanes in (0, 40, 70, 80, 140, 160) or _lanes(n, rule) == (lanes if not more else 2 * lanes)
     _, r, w = scene
     cam = _camera(1021, 523)
     image = r.render(cam, w, counts=True)["rgb"]

@@ -22,7 +22,7 @@ def _scene(flags, sigma_vox, seed):
 
 
 @pytest.mark.parametrize("flags,sigma_vox,n", [(0, 0.6, 1), (0, 0.05, 700), (1, 0.6, 9728), (4, 0.6, 9729), (8, 0.05, 20000),
-                                               (5, 0.3, 77825), (0, 5.0, 155649)])
+                                               (5, 0.3, 77825), (0, 0.3, 150000), (0, 5.0, 155649)])
 def test_recorded_pair_matches_the_plain_pair(flags, sigma_vox, n):
     sc = _scene(flags, sigma_vox, 3)
     r = renderer.Renderer.from_scene(sc, DEV)
