@@ -531,12 +531,13 @@ extern "C" snerg_status snerg_render(snerg_handle h, const snerg_camera* cams, i
         sa.cap = kSchedMaxTiles;
         sa.nt = tiles;
         sa.tiles_x = (cams[0].W + 15) / 16;
-        // a small image's tiles take 8 CTAs each and no sparse slots (by the rule of the plain image,
-        // where it takes 4 rays per warp or fewer: 25,600 pixels of a 1024^3 grid 75 -> 67 us, 32,400 of a
-        // 512^3 one 83 -> 62; 2 or 4 CTAs gain nothing over the sparse tiles: 115,600 pixels of a 1024^3
-        // grid 94 us, with 2 97, with 4 99). Sparse slots only with a previous frame to choose the slow
-        // tiles from
-        sa.parts = image_lanes(h->ds, (int64_t)cams[0].W * cams[0].H, 1) <= 4 ? 8 : 1;
+        // a small image's tiles take 8 CTAs each (4 rays per warp) and no sparse slots: 25,600 pixels of a
+        // 1024^3 grid 75 -> 67 us, 32,400 of a 512^3 one 83 -> 62, 57,600 of a 2048^3 one 212 -> 125, but
+        // 41,209 of a 256^3 one 51 -> 60; 2 or 4 CTAs gain nothing over the sparse tiles (115,600 pixels of
+        // a 1024^3 grid 94 us, with 2 97, with 4 99). Sparse slots only with a previous frame to choose the
+        // slow tiles from
+        const int64_t warps = (int64_t)h->num_sms * by_side(h->ds, 8, 40, 96);
+        sa.parts = (int64_t)cams[0].W * cams[0].H <= 4 * warps ? 8 : 1;
         sa.smax = use && sa.parts == 1 ? std::min(kSchedMaxSparse, std::max(1, tiles / 8)) : 0;
         cudaError_t e = cudaMemsetAsync(wr, 0, kSchedCountBytes, st);
         if (e == cudaSuccess) e = launch_render_image(h->ds, cams[0], d_mlp, pw, d_rgb, dbg, st, 0, cams[0].H, &sa);

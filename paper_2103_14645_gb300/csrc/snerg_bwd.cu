@@ -424,8 +424,11 @@ static cudaError_t backward_launch(const DevScene& s, const CamTable& cams, int3
     if (n <= 0) return cudaSuccess;
     // up to about one wave of 4 CTAs per SM (16 warps): a step of 10,000 rays with 32 / 16 / 8 rays per warp (8:
     // 8 warps per SM) takes 89 / 66 / 58 us on a 1024^3 grid and 55 / 50 / 47 on a 256^3 one, of 33,000
-    // with 32 / 16 (14 warps) 95 / 89 and 62 / 71
-    const int lanes = lanes_per_warp(n, s.sms, {by_side(s, 20, 10, 14), by_side(s, 32, 11, 14), by_side(s, 32, 10, 12), 9, 9});
+    // with 32 / 16 (14 warps) 95 / 89 and 62 / 71. With alpha codes, whose rays composite more, few rays
+    // per warp pay for longer: 4,291 rays of a 1024^3 grid with 32 / 4 / 2 (14 warps) 115 / 78 / 60
+    const LaneLimits density{by_side(s, 20, 10, 14), by_side(s, 32, 11, 14), by_side(s, 32, 10, 12), 9, 9};
+    const LaneLimits alpha{by_side(s, 20, 13, 16), 14, 16, 16, 16};
+    const int lanes = lanes_per_warp(n, s.sms, s.flags & SNERG_FLAG_ALPHA_ATLAS ? alpha : density);
     const size_t smem = backward_smem_bytes(lanes);
     // the opt-in for > 48 KB of dynamic shared memory, once per device
     static std::atomic<bool> attr_set[kMaxDevices];

@@ -365,7 +365,8 @@ cudaError_t Forward<LGB, A>::image(const DevScene& ds, const snerg_camera& cam, 
                                                                                *sch);
         return cudaGetLastError();
     }
-    const int lanes = ps || d ? 32 : image_lanes(ds, (int64_t)cam.W * (row1 - row0), share);
+    const int64_t pixels = (int64_t)cam.W * (row1 - row0);
+    const int lanes = ps || d ? 32 : image_lanes(ds, row1 - row0 < cam.H ? pixels + pixels / 4 : pixels, share);
     const int tw = T::WX << packet_width_log2(lanes), th = T::WY * (lanes >> packet_width_log2(lanes));
     const dim3 grid((cam.W + tw - 1) / tw, (row1 - row0 + th - 1) / th);
     auto* kernel = pw ? render_image_kernel<LGB, A, false, true, kImageWarps, false>

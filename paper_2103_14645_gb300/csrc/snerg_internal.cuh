@@ -985,14 +985,17 @@ struct SchedArgs {
 };
 
 // Rays per warp of a one-camera launch of n pixels (with `share` of its kind on the chip at a time):
-// about one wave of warps (32 per SM) at most in grids of up to 256^3, three in the largest. 38,809 pixels
-// with 32 / 16 / 8 / 4 rays per warp: of a 1024^3 grid 102 / 101 / 87 / 71 us (4: 64 warps per SM), of
-// a 512^3 one 93 / 82 / 62 / 64; 136,900 pixels with 32 / 16 (56): of a 1024^3 grid 123 / 104, 2048^3
-// 243 / 209, but 256^3 60 / 69 and 128^3 45 / 53.
+// up to about one wave of warps (32 per SM) in grids of up to 400^3, three in the largest. 38,809
+// pixels with 32 / 16 / 8 / 4 rays per warp: of a 1024^3 grid 102 / 101 / 87 / 71 us (4: 64 warps per
+// SM), of a 512^3 one 93 / 82 / 62 / 64; 136,900 pixels with 32 / 16 (56): of a 1024^3 grid 123 / 104,
+// 2048^3 243 / 209, but 256^3 60 / 69 and 128^3 45 / 53. The sweeps were of whole objects and of
+// their middle rows, with density and alpha codes: an image with few rays that miss leaves less room
+// (72,852 pixels of such rows of a 512^3 grid with alpha codes 81 / 88 / 106), so a range of rows counts
+// for a quarter more.
 constexpr int kImageWarps = 4;     // warps per CTA of the one-camera launch
 inline int image_lanes(const DevScene& s, int64_t n, int share) {
-    const int w = by_side(s, 8, 40, 96);
-    return lanes_per_warp(n * share, s.sms, {by_side(s, 10, 28, 96), w, w, by_side(s, 4, 32, 80), by_side(s, 6, 40, 56)});
+    return lanes_per_warp(n * share, s.sms, {by_side(s, 14, 28, 96), by_side(s, 12, 40, 96), by_side(s, 10, 36, 96),
+                                             by_side(s, 10, 40, 80), by_side(s, 8, 36, 56)});
 }
 
 inline const MlpWeights& no_weights() {

@@ -21,7 +21,7 @@ def _most(lanes, rule):
 
     def side(d, lo, hi):
         return min(max(N // d, lo), hi)
-    warps = {"image": [side(6, 40, 56), side(4, 32, 80), side(8, 40, 96), side(8, 40, 96), side(10, 28, 96)],
+    warps = {"image": [side(8, 36, 56), side(10, 40, 80), side(10, 36, 96), side(12, 40, 96), side(14, 28, 96)],
              "list": [28, 28, 28, side(16, 20, 28), side(16, 16, 28)], "debug list": [16] * 5,
              "adjoint": [9, 9, side(32, 10, 12), side(32, 11, 14), side(20, 10, 14)]}[rule]
     return sms * warps[LANES.index(lanes)] * lanes
