@@ -91,7 +91,7 @@ struct DevScene {
 // and whether channel 0 holds alpha (A 0 or 1; 2: by the scene's flags). The march's padded
 // indices, face distances and stencil addresses then take immediate operands, and a composited
 // sample has one arithmetic: 64 mixed views of a 1024^3 grid of 32^3 blocks 5.60 -> 5.18 ms, one
-// 800^2 view 168 -> 158 us on the same box (the edge alone: 4.5 and 2 %). Edges of 8 to 64 have builds of their
+// 800^2 view 168 -> 158 us in one run (the edge alone: 4.5 and 2 %). Edges of 8 to 64 have builds of their
 // own; smaller blocks, and debug outputs and the per-sample model on any edge, run the build
 // with members.
 template <int LGB>
@@ -357,7 +357,7 @@ __device__ __forceinline__ float box_search(const Ray& r, float kmax, float k, f
 // again for those in stored blocks (the march is bound by issue in full launches, by the chain
 // of dependent steps in small ones); one shared copy with a face instead of a box per axis:
 // 64 mixed views of a 1024^3 grid 6.01 -> 5.64 ms, one 800^2 view 190 -> 183 us, 262,147
-// scattered rays 283 -> 255 us (one box; boxes differ by up to 15 %).
+// scattered rays 283 -> 255 us (one run; machines differ by up to 15 %).
 template <class SC>
 __device__ __forceinline__ float march_exit(const SC& s, const Ray& r, const float inv_d[3], float kh,
                                             const int j[3], int D, float half) {
